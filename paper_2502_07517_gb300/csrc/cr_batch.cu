@@ -63,10 +63,10 @@ __device__ __forceinline__ void el_tile(const BatchArgs<real>& A, KParams<real>*
     cur = tile.prob;
   }
   if (A.deg[tile.prob] == 3) {
-    if (PHASE == 0) local_body<2, 3, Eq2, real, MIXED, T>(*sP, A.tb[0], tile.blk);
+    if (PHASE == 0) local_phase<2, 3, Eq2, real, MIXED, T>(*sP, A.tb[0], tile.blk);
     else update_body<2, 3, Eq2, real, MIXED, T>(*sP, A.tb[0], A.td[0], tile.blk, A.nblk_upd[tile.prob]);
   } else {
-    if (PHASE == 0) local_body<2, 4, Eq2, real, MIXED, T>(*sP, A.tb[1], tile.blk);
+    if (PHASE == 0) local_phase<2, 4, Eq2, real, MIXED, T>(*sP, A.tb[1], tile.blk);
     else update_body<2, 4, Eq2, real, MIXED, T>(*sP, A.tb[1], A.td[1], tile.blk, A.nblk_upd[tile.prob]);
   }
   __syncthreads();  // the next tile reuses the dynamic shared memory
@@ -110,7 +110,7 @@ __global__ void __launch_bounds__(DegShape<N, T>::TB, (BatchMinBlocks<real, T, 0
   constexpr bool MIXED = sizeof(real) == 4;
   const BatchTile tile = A.t_el[A.el_first[N - 3] + blockIdx.x];
   load_params(&sP, A.P + tile.prob);
-  local_body<2, N, Eq2, real, MIXED, DegShape<N, T>::TB>(sP, A.tb[N - 3], tile.blk);
+  local_phase<2, N, Eq2, real, MIXED, DegShape<N, T>::TB>(sP, A.tb[N - 3], tile.blk);
 }
 
 template <typename real, int N, int T>

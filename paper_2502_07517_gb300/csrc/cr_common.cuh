@@ -6,6 +6,8 @@
 #include <math.h>
 #include <stdint.h>
 
+#include "cr_fixed.cuh"
+
 namespace crk {
 
 constexpr int kMaxN = 4;
@@ -158,6 +160,17 @@ struct DiffScaled {
   real Dtx[kMaxNodes1 * kMaxNodes1], Dty[kMaxNodes1 * kMaxNodes1];
 };
 
+// FP64: also as fixed-point coefficients (cr_fixed.cuh) for the integer-pipe
+// contractions, with the exponent offsets (fix_exp) of the x and y matrices.
+template <>
+struct DiffScaled<double> {
+  double Dx[kMaxNodes1 * kMaxNodes1], Dy[kMaxNodes1 * kMaxNodes1];
+  double Dtx[kMaxNodes1 * kMaxNodes1], Dty[kMaxNodes1 * kMaxNodes1];
+  int2 fDx[kMaxNodes1 * kMaxNodes1], fDy[kMaxNodes1 * kMaxNodes1];
+  int2 fDtx[kMaxNodes1 * kMaxNodes1], fDty[kMaxNodes1 * kMaxNodes1];
+  int oD[2], oDt[2];
+};
+
 template <typename real>
 struct KParams {
   Mesh m;
@@ -188,6 +201,17 @@ inline void fill_scaled(const double* D, const double* w, const double* l0, cons
       ds->Dtx[i * n + j] = real(dt * invdx);
       ds->Dty[i * n + j] = real(dt * invdy);
     }
+  if constexpr (sizeof(real) == 8) {
+    auto fixed = [&](const double* A, int2* F) {
+      const int scale = fix_scale(A, n * n);
+      for (int i = 0; i < kMaxNodes1 * kMaxNodes1; ++i) F[i] = i < n * n ? fix_coef(A[i], scale) : make_int2(0, 0);
+      return fix_exp(scale);
+    };
+    ds->oD[0] = fixed(ds->Dx, ds->fDx);
+    ds->oD[1] = fixed(ds->Dy, ds->fDy);
+    ds->oDt[0] = fixed(ds->Dtx, ds->fDtx);
+    ds->oDt[1] = fixed(ds->Dty, ds->fDty);
+  }
 }
 
 // ---------------------------------------------------------------------------
@@ -259,8 +283,35 @@ __device__ __forceinline__ bool gt0(double x) {
   const long long b = __double_as_longlong(x);
   return b > 0ll && b <= 0x7ff0000000000000ll;
 }
-template <typename real>
-__device__ __forceinline__ real sqrt_pos(real x) { return sqrt(gt0(x) ? x : real(0)); }
+__device__ __forceinline__ float sqrt_pos(float x) { return sqrt(x > 0.0f ? x : 0.0f); }
+// FP64 square root of max(x, 0): two Newton steps g += (x - g^2) h on g = x y, h
+// = y / 2 from the hardware's approximation y of 1 / sqrt(x) (20 bits; 2^-40 and
+// then below the rounding of the last FMA, so the error is that rounding's).
+// Five FP64 instructions, where sqrt() takes nine (measured 143 SM cycles per
+// warp).  Outside the normal range: sqrt().
+__device__ __forceinline__ double sqrt_pos(double x) {
+  const int h = __double2hiint(x);
+  if (unsigned(h - 0x00100000) >= 0x7fe00000u) return gt0(x) ? sqrt(x) : 0.0;
+  double y;
+  asm("rsqrt.approx.ftz.f64 %0, %1;" : "=d"(y) : "d"(x));
+  double g = x * y;
+  const double hf = __hiloint2double(__double2hiint(y) - (1 << 20), __double2loint(y));
+  g = fma(fma(-g, g, x), hf, g);
+  return fma(fma(-g, g, x), hf, g);
+}
+// 1 / x.  FP64: one step r (1 + e + e^2), e = 1 - x r, of the third-order
+// (Halley-type) iteration on the hardware's 20-bit approximation: e^3 is below
+// 2^-60, so the error is the rounding of the last FMA (and x = 0 or inf gives
+// NaN).  Three FP64 instructions, where the division takes five (86 SM cycles
+// per warp).
+__device__ __forceinline__ float recip(float x) { return 1.0f / x; }
+__device__ __forceinline__ double recip(double x) {
+  double r;
+  asm("rcp.approx.ftz.f64 %0, %1;" : "=d"(r) : "d"(x));
+  double e = fma(-x, r, 1.0);
+  e = fma(e, e, e);
+  return fma(r, e, r);
+}
 
 struct EqLinAdv {  // u_t + a . grad u = 0, Sec. 5.1.1
   static constexpr int M = 1, K = 0;
@@ -436,11 +487,11 @@ struct EqEuler {
   template <typename real>
   __device__ static void flux(const real* u, int dir, real* f, const Phys<real>& ph) {
     real p;
-    flux_r(u, dir, real(1) / u[0], f, &p, ph);
+    flux_r(u, dir, recip(u[0]), f, &p, ph);
   }
   template <typename real>
   __device__ static void flux_xy(const real* u, real* f, real* g, const Phys<real>& ph) {
-    const real rinv = real(1) / u[0];
+    const real rinv = recip(u[0]);
     if (DIM == 1) {
       real p;
       flux_r(u, 0, rinv, f, &p, ph);
@@ -460,14 +511,14 @@ struct EqEuler {
   }
   template <typename real>
   __device__ static void flux_speed(const real* u, int dir, real* f, real* s, const Phys<real>& ph) {
-    const real rinv = real(1) / u[0];
+    const real rinv = recip(u[0]);
     real p;
     flux_r(u, dir, rinv, f, &p, ph);
     *s = fabs(u[1 + dir] * rinv) + sqrt_pos(ph.gamma * p * rinv);
   }
   template <typename real>
   __device__ static real speed(const real* u, int dir, const Phys<real>& ph) {
-    const real rinv = real(1) / u[0];
+    const real rinv = recip(u[0]);
     const real p = ph.gm1 * (u[E] - kinetic_rho(u) * rinv);
     return fabs(u[1 + dir] * rinv) + sqrt_pos(ph.gamma * p * rinv);
   }
@@ -514,11 +565,11 @@ struct EqTenMoment {
   }
   template <typename real>
   __device__ static void flux(const real* u, int dir, real* f, const Phys<real>& ph) {
-    flux_r(u, dir, real(1) / u[0], f, ph);
+    flux_r(u, dir, recip(u[0]), f, ph);
   }
   template <typename real>
   __device__ static void flux_xy(const real* u, real* f, real* g, const Phys<real>& ph) {
-    const real rinv = real(1) / u[0];
+    const real rinv = recip(u[0]);
     flux_r(u, 0, rinv, f, ph);
     flux_r(u, 1, rinv, g, ph);
   }
@@ -530,18 +581,18 @@ struct EqTenMoment {
   }
   template <typename real>
   __device__ static void flux_speed(const real* u, int dir, real* f, real* s, const Phys<real>& ph) {
-    const real rinv = real(1) / u[0];
+    const real rinv = recip(u[0]);
     flux_r(u, dir, rinv, f, ph);
     *s = speed_r(u, dir, rinv);
   }
   template <typename real>
   __device__ static real speed(const real* u, int dir, const Phys<real>&) {
-    return speed_r(u, dir, real(1) / u[0]);
+    return speed_r(u, dir, recip(u[0]));
   }
   template <typename real>
   __device__ static real constraint(const real* u, int k, const Phys<real>&) {
     if (k == 0) return u[0];
-    const real rinv = real(1) / u[0];
+    const real rinv = recip(u[0]);
     const real p11 = real(2) * u[3] - u[1] * u[1] * rinv;
     const real p12 = real(2) * u[4] - u[1] * u[2] * rinv;
     const real p22 = real(2) * u[5] - u[2] * u[2] * rinv;
@@ -558,7 +609,7 @@ struct EqTenMoment {
   }
   template <typename real>
   __device__ static real indicator_var(const real* u, const Phys<real>&) {
-    const real rinv = real(1) / u[0];
+    const real rinv = recip(u[0]);
     const real p11 = real(2) * u[3] - u[1] * u[1] * rinv;
     const real p22 = real(2) * u[5] - u[2] * u[2] * rinv;
     return u[0] * real(0.5) * (p11 + p22);

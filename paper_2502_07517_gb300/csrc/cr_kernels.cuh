@@ -803,6 +803,19 @@ __device__ __forceinline__ void local_body(const KParams<real>& P, const Tab<rea
 #undef ATPE
 }
 
+}  // namespace crk
+
+#include "cr_local64.cuh"
+
+namespace crk {
+
+// The element phase of a block: FP64 in two dimensions has its own body.
+template <int DIM, int N, class EQ, typename real, bool MIXED, int T>
+__device__ __forceinline__ void local_phase(const KParams<real>& P, const Tab<real>& tb, const int blk) {
+  if constexpr (DIM == 2 && !MIXED) local_body_f64<N, EQ, T>(P, tb, blk);
+  else local_body<DIM, N, EQ, real, MIXED, T>(P, tb, blk);
+}
+
 // Resident blocks per SM the step kernels ask for (measured on GB300,
 // 2D Euler N = 4, 512x512): FP32_BULK blocks are latency bound and gain from
 // four 256-thread blocks per SM (64 registers; k_local 1.39 -> 1.05 ms,
@@ -826,7 +839,7 @@ template <int NP, bool MIXED> using UpdateShape = BlockShape<NP, MIXED ? 128 : 2
 
 template <int DIM, int N, class EQ, typename real, bool MIXED>
 __global__ void __launch_bounds__(256, MinBlocks<MIXED>::local) k_local(const __grid_constant__ KParams<real> P) {
-  local_body<DIM, N, EQ, real, MIXED, BlockShape<DIM == 2 ? (N + 1) * (N + 1) : N + 1>::T>(P, P.tb, blockIdx.x);
+  local_phase<DIM, N, EQ, real, MIXED, BlockShape<DIM == 2 ? (N + 1) * (N + 1) : N + 1>::T>(P, P.tb, blockIdx.x);
 }
 
 // ===========================================================================

@@ -1,0 +1,609 @@
+// The FP64 element kernel in two dimensions (the body that k_local and the
+// batched kernels run for real = double, DIM = 2): the same phases and the same
+// outputs as local_body, arranged for the FP64 pipe.
+//
+// What bounds it: GB300 issues one FP64 warp instruction per SM every 16
+// cycles, against two integer or FP32 ones per cycle, and the pipe was 90% busy
+// at 10% of the issue slots (2D Euler N = 4, 512 x 512: 12.57 ms, 1,031 FP64
+// instructions per solution point).  So every FP64 instruction that integer or
+// FP32 work can replace without touching the result is worth 30 of those:
+//   - the D contractions (a third of the FP64 work) run in fixed point on the
+//     integer pipe (cr_fixed.cuh);
+//   - the trace of the time-averaged solution is the average of the stage
+//     traces, which the face-node threads form anyway, and the wave speed of
+//     the u^n trace shares the first stage's flux;
+//   - which of the three slopes minmod takes, which of two wave speeds is the
+//     larger and whether the MUSCL-Hancock states are admissible are decided in
+//     FP32 where the answer is clear by a margin above the FP32 rounding, and
+//     in FP64 where it is not; only the chosen slope and speed are formed;
+//   - reciprocals and square roots by one third-order and two Newton steps from
+//     the hardware's approximations (recip, sqrt_pos), and factors that depend
+//     on the step or the node row alone formed once per block.
+// Measured (k_local, the same workload): 612 FP64 instructions per point, 12.57
+// -> 8.42 ms; ten-moment N = 3 at 256 x 256 2.61 -> 2.03 ms.
+#pragma once
+#include "cr_common.cuh"
+#include "cr_fixed.cuh"
+
+namespace crk {
+
+// |relative error| of an FP32 comparison below: truncated operands (2^-23
+// each), the approximate square root and a few FP32 operations stay under half
+// of it.
+constexpr float kTieF = 1.9073486e-6f;  // 2^-19
+
+// x as FP32, truncated, from the bit pattern: magnitudes below FP32's normal
+// range give a value below 2^-126, larger ones its largest finite value.
+__device__ __forceinline__ float trunc_f32(double x) {
+  const int h = __double2hiint(x);
+  int m = (h & 0x7fffffff) - (896 << 20);
+  m = min(max(m, 0), 0x0fefffff);
+  const unsigned b = __funnelshift_l((unsigned)__double2loint(x), (unsigned)m, 3);
+  return __uint_as_float(b | (unsigned(h) & 0x80000000u));
+}
+
+__device__ __forceinline__ float sqrt_f32(float x) {
+  float r;
+  asm("sqrt.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(fmaxf(x, 0.0f)));
+  return r;
+}
+
+// minmod of the slopes d1 b1, d2 b2, d3 b3 (b > 0) with f1, f2, f3 = b in FP32.
+__device__ __forceinline__ double minmod_scaled(double d1, double d2, double d3, double b1, double b2,
+                                                double b3, float f1, float f2, float f3) {
+  const long long i1 = __double_as_longlong(d1), i2 = __double_as_longlong(d2), i3 = __double_as_longlong(d3);
+  if (((i1 ^ i2) | (i1 ^ i3)) < 0 || (i1 << 1) == 0 || (i2 << 1) == 0 || (i3 << 1) == 0) return 0.0;
+  const float m1 = fabsf(trunc_f32(d1)) * f1, m2 = fabsf(trunc_f32(d2)) * f2, m3 = fabsf(trunc_f32(d3)) * f3;
+  const float lim = fminf(m1, fminf(m2, m3)) * (1.0f + kTieF);
+  const bool c1 = m1 <= lim, c2 = m2 <= lim, c3 = m3 <= lim;
+  if (int(c1) + int(c2) + int(c3) != 1) return minmod3(d1 * b1, d2 * b2, d3 * b3);
+  return (c1 ? d1 : (c2 ? d2 : d3)) * (c1 ? b1 : (c2 ? b2 : b3));
+}
+
+// Flux in direction dir with the normal velocity and the squared sound speed
+// (the wave speed is |vn| + sqrt(c2)); equations without one: vn = the speed.
+template <class EQ>
+__device__ __forceinline__ void flux_c2(const double* u, int dir, double* f, double* vn, double* c2,
+                                        const Phys<double>& ph) {
+  if constexpr (IsEuler<EQ>::value) {
+    const double rinv = recip(u[0]);
+    double p;
+    EQ::flux_r(u, dir, rinv, f, &p, ph);
+    *vn = u[1 + dir] * rinv;
+    *c2 = ph.gamma * p * rinv;
+  } else if constexpr (EQ::M == 6) {
+    const double rinv = recip(u[0]);
+    EQ::flux_r(u, dir, rinv, f, ph);
+    *vn = u[1 + dir] * rinv;
+    *c2 = 3.0 * (2.0 * u[3 + 2 * dir] - u[1 + dir] * *vn) * rinv;
+  } else {
+    EQ::flux(u, dir, f, ph);
+    *vn = EQ::speed(u, dir, ph);
+    *c2 = 0.0;
+  }
+}
+
+// max(|vL| + sqrt(cL), |vR| + sqrt(cR)), c <= 0 counted as 0: the larger side
+// is picked in FP32 unless the two are within kTieF.
+__device__ __forceinline__ double wave_max(double vL, double cL, double vR, double cR) {
+  const float sL = fabsf(trunc_f32(vL)) + sqrt_f32(trunc_f32(cL));
+  const float sR = fabsf(trunc_f32(vR)) + sqrt_f32(trunc_f32(cR));
+  if (fabsf(sL - sR) > kTieF * (sL + sR)) {
+    const bool left = sL > sR;
+    return fabs(left ? vL : vR) + sqrt_pos(left ? cL : cR);
+  }
+  return fmax(fabs(vL) + sqrt_pos(cL), fabs(vR) + sqrt_pos(cR));
+}
+
+// Twice the Rusanov flux (the factor 1/2 goes into the caller's constants,
+// exactly).
+template <class EQ>
+__device__ __forceinline__ void rusanov_twice(const double* uL, const double* uR, int dir, double* out,
+                                              const Phys<double>& ph) {
+  double fL[EQ::M], fR[EQ::M], vL, vR, cL, cR, lam;
+  flux_c2<EQ>(uL, dir, fL, &vL, &cL, ph);
+  flux_c2<EQ>(uR, dir, fR, &vR, &cR, ph);
+  if constexpr (EQ::K > 0) lam = wave_max(vL, cL, vR, cR);
+  else lam = vL;  // linear advection: the speed does not depend on the state
+#pragma unroll
+  for (int v = 0; v < EQ::M; ++v) out[v] = fma(-lam, uR[v] - uL[v], fL[v] + fR[v]);
+}
+
+// FP32 screen of the MUSCL-Hancock states: s is a state and A bounds the
+// magnitudes its parts are summed from.  True only when the state is admissible
+// by a margin of 2e-5 of those magnitudes, an order above the FP32 rounding of
+// the sums and products.
+template <class EQ>
+__device__ __forceinline__ bool clearly_admissible(const float* s, const float* A) {
+  if constexpr (EQ::K == 0) return true;
+  if (!(s[0] > 2e-5f * A[0])) return false;
+  if constexpr (IsEuler<EQ>::value) {
+    const float q = s[3] * s[0] - 0.5f * (s[1] * s[1] + s[2] * s[2]);
+    return q > 2e-5f * (A[3] * A[0] + A[1] * A[1] + A[2] * A[2]);
+  } else if constexpr (EQ::M == 6) {
+    const float a11 = 2.0f * s[0] * s[3] - s[1] * s[1], a22 = 2.0f * s[0] * s[5] - s[2] * s[2];
+    const float a12 = 2.0f * s[0] * s[4] - s[1] * s[2];
+    const float B = 2.0f * A[0] * (A[3] + A[4] + A[5]) + A[1] * A[1] + A[2] * A[2];
+    return a11 > 2e-5f * B && a11 * a22 - a12 * a12 > 1e-4f * B * B;
+  }
+  return true;
+}
+
+// Shared memory of the body beyond the five node arrays, in bytes.
+template <int N, class EQ>
+__host__ __device__ constexpr size_t local64_extra(int epb) {
+  constexpr int n = N + 1, S = Tableau<N>::S;
+  return (size_t)epb * sizeof(double) + (size_t)(4 * n * n) * sizeof(int2) + (size_t)(S * S + 4 * n) * sizeof(double) +
+         (size_t)epb * (4 + 2 * n * EQ::M) * sizeof(int);
+}
+
+template <int N, class EQ, int T>
+__device__ __forceinline__ void local_body_f64(const KParams<double>& P, const Tab<double>& tb, const int blk) {
+  constexpr int n = N + 1, NP = n * n, M = EQ::M, S = Tableau<N>::S, NSLOT = 4 * n;
+  constexpr int SPT = (NSLOT + NP - 1) / NP;
+  using TB = Tableau<N>;
+  const Mesh& m = P.m;
+  const Phys<double>& ph = P.ph;
+  constexpr int epb = (T + NP - 1) / NP, epr = T / NP;
+  const int tid = threadIdx.x;
+  const int el = tid / NP, k = tid - el * NP, p = k % n, q = k / n;
+  const int e = blk * epr + el;
+  const bool valid = el < epr && e < m.ne;
+  const int ee = valid ? e : m.ne - 1;
+  const int ix = ee % m.nx, iy = ee / m.nx;
+
+  const double dt = P.b.ctl->dt_step;
+  if (!gt0(dt)) return;
+
+  // node arrays [M][epb][NP]: u^n; the stage state, then the MUSCL-Hancock
+  // states; the stage fluxes in fixed point; the time-averaged solution (for a
+  // source), then the y+ states
+  extern __shared__ __align__(16) unsigned char smem_raw[];
+  constexpr int stride = epb * NP, arr = M * stride;
+  double* s0 = reinterpret_cast<double*>(smem_raw);
+  double* sA = s0 + arr;
+  double* sB = sA + arr;
+  double* sC = sB + arr;
+  double* sD = sC + arr;
+  int2* xB = reinterpret_cast<int2*>(sB);
+  int2* xC = reinterpret_cast<int2*>(sC);
+  double* sAlpha = sD + arr;                                  // [epb]
+  int2* tDx = reinterpret_cast<int2*>(sAlpha + epb);          // [n][n] each
+  int2* tDy = tDx + n * n;
+  int2* tDtx = tDy + n * n;
+  int2* tDty = tDtx + n * n;
+  double* sAdt = reinterpret_cast<double*>(tDty + n * n);     // dt a_ij
+  double* sHx = sAdt + S * S;                                 // dt / (2 w_p dx), dt / (2 w_q dy)
+  double* sHy = sHx + n;
+  double* sWx = sHy + n;                                      // 1 / (2 w_p dx), 1 / (2 w_q dy)
+  double* sWy = sWx + n;
+  int* sNbr = reinterpret_cast<int*>(sWy + n);                // [epb][4]
+  int* sKx = sNbr + epb * 4;                                  // line keys [epb][n][M]
+  int* sKy = sKx + epb * n * M;
+
+  double un[M];
+#pragma unroll
+  for (int v = 0; v < M; ++v) un[v] = P.b.u[((size_t)v * m.ne + ee) * NP + k];
+  for (int t = tid; t < 2 * epb * n * M; t += T) sKx[t] = 0;
+  for (int e2 = tid; e2 < epb; e2 += T) {
+    const int eg0 = blk * epr + e2;
+    const bool v2 = e2 < epr && eg0 < m.ne;
+    const int eg = v2 ? eg0 : m.ne - 1;
+    int nbs[4];
+#pragma unroll
+    for (int f = 0; f < 4; ++f) sNbr[e2 * 4 + f] = nbs[f] = neighbour(m, eg, f);
+    double al = 0.0;
+    if (m.alpha_mode == 1) {
+      al = m.alpha_fixed;
+    } else if (m.limiter & kLimBlend) {
+      al = P.b.alpha_raw[eg];
+#pragma unroll
+      for (int f = 0; f < 4; ++f)
+        if (nbs[f] >= 0) al = fmax(al, 0.5 * P.b.alpha_raw[nbs[f]]);
+    }
+    sAlpha[e2] = al;
+    if (v2) P.b.alpha[eg] = al;
+  }
+  for (int t = tid; t < n * n; t += T) {
+    tDx[t] = P.ds.fDx[t];
+    tDy[t] = P.ds.fDy[t];
+    tDtx[t] = P.ds.fDtx[t];
+    tDty[t] = P.ds.fDty[t];
+  }
+  // (per-block factors by threads of the last warps: the first ones smooth alpha)
+  for (int t = T - 1 - tid; t < S * S + 2 * n; t += T) {
+    if (t < S * S) {
+      sAdt[t] = dt * TB::a(t / S, t % S);
+    } else {
+      const int r = t - S * S, pp = r % n;
+      const double w = 0.5 * tb.invw[pp] * (r < n ? ph.invdx : ph.invdy);
+      sWx[r] = w;
+      sHx[r] = dt * w;
+    }
+  }
+  vst_sh<M, stride>(s0 + tid, un);
+  __syncthreads();
+  const double alpha = sAlpha[el];
+  const bool blend = (m.limiter & kLimBlend) || m.alpha_mode == 1;
+  const bool need_lo = blend || (m.limiter & kLimFlux);
+  const double a = blend ? alpha : 0.0;
+
+  constexpr bool SRC = EQ::M == 6 || HasGravity<EQ>::value;
+  const bool has_src = (EQ::M == 6 && m.source == 1) || (HasGravity<EQ>::value && m.source == 2);
+  double dWx = 0.0, dWy = 0.0;
+  if (HasGravity<EQ>::value && has_src) {
+    dWx = m.grav[0];
+    dWy = m.grav[1];
+  } else if (SRC && has_src) {
+    const double x = m.x0 + (ix + tb.xi[p]) * m.dx, y = m.y0 + (iy + tb.xi[q]) * m.dy;
+    source_grad<2, double>(m, x - m.src_cx, y - m.src_cy, &dWx, &dWy);
+  }
+
+  // ---------------- local cRK stages -----------------------------------
+  double Lst[S > 1 ? S - 1 : 1][M], Fa[M], Ga[M];
+  double ea[SPT][M], Ut[SPT][M];
+#pragma unroll
+  for (int v = 0; v < M; ++v) {
+    Fa[v] = Ga[v] = 0.0;
+#pragma unroll
+    for (int mm = 0; mm < SPT; ++mm) ea[mm][v] = Ut[mm][v] = 0.0;
+  }
+  int* const kx = sKx + (el * n + q) * M;  // this node's x-line and y-line
+  int* const ky = sKy + (el * n + p) * M;
+  const int line_x = el * NP + n * q, line_y = el * NP + p;
+
+  // The x and y fluxes of this node into the line arrays in fixed point, and a
+  // barrier.  A line keeps its exponent from the first stage until a value
+  // needs two more bits; then (rarely: the vote) the line takes the larger one.
+  auto put_lines = [&](const double (&f)[M], const double (&g)[M], bool first) {
+    if (first) {
+#pragma unroll
+      for (int v = 0; v < M; ++v) {
+        atomicMax(kx + v, mag_key(f[v]));
+        atomicMax(ky + v, mag_key(g[v]));
+      }
+      __syncthreads();
+    }
+    unsigned over = 0u;  // bit 2v: f[v] outgrew its line's exponent, bit 2v + 1: g[v]
+#pragma unroll
+    for (int v = 0; v < M; ++v) {
+      const int ex = line_exp(kx[v]), ey = line_exp(ky[v]);
+      over |= (unsigned((mag_key(f[v]) >> 20) > ex + 1) << (2 * v)) | (unsigned((mag_key(g[v]) >> 20) > ey + 1) << (2 * v + 1));
+      xB[v * stride + tid] = to_fixed(f[v], ex);
+      xC[v * stride + tid] = to_fixed(g[v], ey);
+    }
+    if (first) {
+      __syncthreads();
+    } else if (__syncthreads_or(valid && over)) {
+#pragma unroll
+      for (int v = 0; v < M; ++v) {
+        if ((over >> (2 * v)) & 1u) atomicMax(kx + v, mag_key(f[v]));
+        if ((over >> (2 * v + 1)) & 1u) atomicMax(ky + v, mag_key(g[v]));
+      }
+      __syncthreads();
+#pragma unroll
+      for (int v = 0; v < M; ++v) {
+        xB[v * stride + tid] = to_fixed(f[v], line_exp(kx[v]));
+        xC[v * stride + tid] = to_fixed(g[v], line_exp(ky[v]));
+      }
+      __syncthreads();
+    }
+  };
+  // sum_r Ax[p][r] f(line_x, r) + Ay[q][r] g(line_y, r) of variable v
+  auto line_dot = [&](int v, const int2* Ax, const int2* Ay, int ox, int oy) -> double {
+    FixAcc ax{0, 0}, ay{0, 0};
+#pragma unroll
+    for (int r = 0; r < n; ++r) {
+      fix_mad(ax, xB[v * stride + line_x + r], Ax[p * n + r]);
+      fix_mad(ay, xC[v * stride + line_y + n * r], Ay[q * n + r]);
+    }
+    const int ex = line_exp(kx[v]), ey = line_exp(ky[v]);
+    if (max(ex, ey) > kMaxLineExp) return __longlong_as_double(0x7ff8000000000000ll);
+    return from_fixed2(fix_sum(ax), ex + ox, fix_sum(ay), ey + oy);
+  };
+
+#pragma unroll
+  for (int i = 0; i < S; ++i) {
+    double ui[M], f[M], g[M];
+#pragma unroll
+    for (int v = 0; v < M; ++v) ui[v] = un[v];
+#pragma unroll
+    for (int j = 0; j < i; ++j)
+      if (TB::a(i, j) != 0.0) vfma(ui, -sAdt[i * S + j], Lst[j]);
+    EQ::flux_xy(ui, f, g, ph);
+    if (TB::b(i) != 0.0) {
+      vfma(Fa, TB::b(i), f);
+      vfma(Ga, TB::b(i), g);
+    }
+    if (SRC && has_src) {  // the time-averaged solution, for its source
+#pragma unroll
+      for (int v = 0; v < M; ++v) {
+        double* ua = sD + v * stride + tid;
+        if (i == 0) *ua = TB::b(0) * ui[v];
+        else if (TB::b(i) != 0.0) *ua = fma(TB::b(i), ui[v], *ua);
+      }
+    }
+    vst_sh<M, stride>(sA + tid, ui);
+    if (i < S - 1) put_lines(f, g, i == 0);
+    else __syncthreads();
+    if (i < S - 1) {
+#pragma unroll
+      for (int v = 0; v < M; ++v) Lst[i < S - 1 ? i : 0][v] = line_dot(v, tDx, tDy, P.ds.oD[0], P.ds.oD[1]);
+      if (SRC && has_src) {
+        double us[M], s[M];
+        vld_sh<M, stride>(us, sA + tid);
+        source_eval<EQ>(us, dWx, dWy, s);
+#pragma unroll
+        for (int v = 0; v < M; ++v) Lst[i < S - 1 ? i : 0][v] -= s[v];
+      }
+    }
+    if (i == 0 || TB::b(i) != 0.0) {
+#pragma unroll
+      for (int mm = 0; mm < SPT; ++mm) {
+        const FaceSlot fs = face_slot<NSLOT, n>(tid + mm * T);
+        const int eg = blk * epr + fs.el;
+        if (fs.el < epr && eg < m.ne) {
+          const int side = fs.side, j = fs.j;
+          double ut[M];
+#pragma unroll
+          for (int v = 0; v < M; ++v) ut[v] = 0.0;
+#pragma unroll
+          for (int r = 0; r < n; ++r) {
+            const double l = (side & 1) ? tb.l1[r] : tb.l0[r];
+            vfma_sh<M, stride>(ut, l, sA + fs.el * NP + (side < 2 ? r + n * j : j + n * r));
+          }
+          if (TB::b(i) != 0.0) {
+            vfma(Ut[mm], TB::b(i), ut);
+            if (m.dissipation == 2) {  // D-CSX: the stage trace, for the face kernel
+#pragma unroll
+              for (int v = 0; v < M; ++v)
+                P.b.slot[slot_index(1 + 4 * M + i * M + v, side, eg, j, 4, m.ne, n)] = ut[v];
+            }
+          }
+          if (i == 0 || m.central == 0) {
+            double fn[M], vn, c2;
+            flux_c2<EQ>(ut, side >> 1, fn, &vn, &c2, ph);
+            if (TB::b(i) != 0.0 && m.central == 0) vfma(ea[mm], TB::b(i), fn);  // EA, eq. (evaluate)
+            if (i == 0) {  // u^n trace: its wave speed, and the trace itself for D1
+              P.b.slot[slot_index(0, side, eg, j, 4, m.ne, n)] = EQ::K > 0 ? fabs(vn) + sqrt_pos(c2) : vn;
+              if (m.dissipation == 1) {
+#pragma unroll
+                for (int v = 0; v < M; ++v) P.b.slot[slot_index(1 + v, side, eg, j, 4, m.ne, n)] = ut[v];
+              }
+            }
+          }
+        }
+      }
+    }
+    __syncthreads();
+  }
+
+  // ---------------- time averages: high-order volume part, face data ----
+  if (m.central == 1) {  // AE: the averages themselves, for their traces
+    vst_sh<M, stride>(sA + tid, Fa);
+  }
+  put_lines(Fa, Ga, false);
+  double HO[M];
+#pragma unroll
+  for (int v = 0; v < M; ++v) HO[v] = line_dot(v, tDtx, tDty, P.ds.oDt[0], P.ds.oDt[1]);
+  // HO becomes the high-order part of the update, u^n - dt (1 - a) HO + dt S,
+  // with the source of the time-averaged solution (linear in u)
+  const double dho = dt * (1.0 - a);
+  vfma(HO, -dho, HO, un);
+  if (SRC && has_src) {
+    double us[M], Sa[M];
+    vld_sh<M, stride>(us, sD + tid);
+    source_eval<EQ>(us, dWx, dWy, Sa);
+    vfma(HO, dt, Sa);
+  }
+#pragma unroll
+  for (int mm = 0; mm < SPT; ++mm) {
+    const FaceSlot fs = face_slot<NSLOT, n>(tid + mm * T);
+    const int eg = blk * epr + fs.el;
+    if (fs.el < epr && eg < m.ne) {
+      // slots 1..M: the trace the dissipation jumps over (U; D1 stored u^n's);
+      // slots 1+M..: the EA average (AE: below)
+#pragma unroll
+      for (int v = 0; v < M; ++v) {
+        if (m.dissipation != 1) P.b.slot[slot_index(1 + v, fs.side, eg, fs.j, 4, m.ne, n)] = Ut[mm][v];
+        if (m.central == 0) P.b.slot[slot_index(1 + M + v, fs.side, eg, fs.j, 4, m.ne, n)] = ea[mm][v];
+      }
+    }
+  }
+  if (m.central == 1) {  // AE, eq. (extrapolate): the trace of F on x faces, of G on y faces
+    for (int dir = 0; dir < 2; ++dir) {
+      if (dir == 1) {
+        __syncthreads();
+        vst_sh<M, stride>(sA + tid, Ga);
+        __syncthreads();
+      }
+#pragma unroll
+      for (int mm = 0; mm < SPT; ++mm) {
+        const FaceSlot fs = face_slot<NSLOT, n>(tid + mm * T);
+        const int eg = blk * epr + fs.el;
+        if (fs.el < epr && eg < m.ne && (fs.side >> 1) == dir) {
+          double Ft[M];
+#pragma unroll
+          for (int v = 0; v < M; ++v) Ft[v] = 0.0;
+#pragma unroll
+          for (int r = 0; r < n; ++r) {
+            const double l = (fs.side & 1) ? tb.l1[r] : tb.l0[r];
+            vfma_sh<M, stride>(Ft, l, sA + fs.el * NP + (dir == 0 ? r + n * fs.j : fs.j + n * r));
+          }
+#pragma unroll
+          for (int v = 0; v < M; ++v) P.b.slot[slot_index(1 + M + v, fs.side, eg, fs.j, 4, m.ne, n)] = Ft[v];
+        }
+      }
+    }
+  }
+  __syncthreads();
+
+  // ---------------- MUSCL-Hancock / first-order subcells -----------------
+  double LO[M];
+#pragma unroll
+  for (int v = 0; v < M; ++v) LO[v] = 0.0;
+  if (need_lo) {
+    double xm[M], xp[M], ym[M], yp[M];
+#pragma unroll
+    for (int v = 0; v < M; ++v) xm[v] = xp[v] = ym[v] = yp[v] = un[v];
+    if (m.limiter & kLimMH) {
+      const double beta = 2.0 - alpha;
+      double sx[M], sy[M];
+      // slopes along one direction: the neighbour nodes of the line, across a
+      // face the neighbour element's, at a boundary the side's ghost node
+      // (outflow: the own node; wall: its reflection; Dirichlet, inflow: given)
+      auto slopes = [&](double (&sl)[M], int c, int step, int side0, int far_lo, int far_hi, int mom) {
+        const int nbl = c == 0 ? sNbr[el * 4 + side0] : -1, nbr = c == N ? sNbr[el * 4 + side0 + 1] : -1;
+        const int sg = c == 0 ? side0 : side0 + 1, bc = m.bcs[sg];
+        double gv[M];
+#pragma unroll
+        for (int v = 0; v < M; ++v) gv[v] = un[v];
+        if (bc == kBcDirichlet || bc == kBcInflow) ghost_at<M>(m, sg, P.b.ctl->t, gv);
+        else if (bc == kBcWall && M > 1) gv[M > 1 ? mom : 0] = -un[M > 1 ? mom : 0];
+        const double bm = beta * tb.ihm[c], bc0 = tb.ihc[c], bp = beta * tb.ihp[c];
+        const float fm = trunc_f32(bm), fc = trunc_f32(bc0), fp = trunc_f32(bp);
+#pragma unroll
+        for (int v = 0; v < M; ++v) {
+          const double um = c > 0 ? s0[v * stride + tid - step]
+                                  : (nbl >= 0 ? P.b.u[((size_t)v * m.ne + nbl) * NP + far_lo] : gv[v]);
+          const double up = c < N ? s0[v * stride + tid + step]
+                                  : (nbr >= 0 ? P.b.u[((size_t)v * m.ne + nbr) * NP + far_hi] : gv[v]);
+          sl[v] = minmod_scaled(un[v] - um, up - um, up - un[v], bm, bc0, bp, fm, fc, fp);
+        }
+      };
+      slopes(sx, p, 1, 0, N + n * q, n * q, 1);
+      slopes(sy, q, n, 2, p + n * N, p, 2);
+      double fxm[M], fxp[M], fym[M], fyp[M], Fm[M], Fp[M], ex[M];
+      vfma(fxm, tb.dm[p], sx, un);
+      vfma(fxp, tb.dp[p], sx, un);
+      vfma(fym, tb.dm[q], sy, un);
+      vfma(fyp, tb.dp[q], sy, un);
+      EQ::flux(fxm, 0, Fm, ph);
+      EQ::flux(fxp, 0, Fp, ph);
+      vsub(ex, Fp, Fm);
+      vmul(ex, ex, sHx[p]);
+      EQ::flux(fym, 1, Fm, ph);
+      EQ::flux(fyp, 1, Fp, ph);
+      vsub(Fp, Fp, Fm);
+      vfma(ex, sHy[q], Fp);
+      bool ok = true;
+      if constexpr (EQ::K > 0) {
+        float uf[M], xf[M], yf[M], ef[M], A[M], st[M];
+        const float dmx = trunc_f32(tb.dm[p]), dpx = trunc_f32(tb.dp[p]);
+        const float dmy = trunc_f32(tb.dm[q]), dpy = trunc_f32(tb.dp[q]);
+#pragma unroll
+        for (int v = 0; v < M; ++v) {
+          uf[v] = trunc_f32(un[v]);
+          xf[v] = trunc_f32(sx[v]);
+          yf[v] = trunc_f32(sy[v]);
+          ef[v] = trunc_f32(ex[v]);
+          A[v] = fabsf(uf[v]) + fabsf(xf[v]) + fabsf(yf[v]) + fabsf(ef[v]);
+        }
+#pragma unroll
+        for (int c = 0; c < 8; ++c) {  // four face states, then evolved
+          const float d = (c & 3) == 0 ? dmx : (c & 3) == 1 ? dpx : (c & 3) == 2 ? dmy : dpy;
+#pragma unroll
+          for (int v = 0; v < M; ++v) {
+            st[v] = fmaf(d, (c & 2) ? yf[v] : xf[v], uf[v]);
+            if (c & 4) st[v] -= ef[v];
+          }
+          ok = ok && clearly_admissible<EQ>(st, A);
+        }
+      }
+      double exm[M], exp_[M], eym[M], eyp[M];
+      vsub(exm, fxm, ex);
+      vsub(exp_, fxp, ex);
+      vsub(eym, fym, ex);
+      vsub(eyp, fyp, ex);
+      if (!ok)
+        ok = EQ::admissible_fast(fxm, ph) && EQ::admissible_fast(fxp, ph) && EQ::admissible_fast(exm, ph) &&
+             EQ::admissible_fast(exp_, ph) && EQ::admissible_fast(fym, ph) && EQ::admissible_fast(fyp, ph) &&
+             EQ::admissible_fast(eym, ph) && EQ::admissible_fast(eyp, ph);
+      if (ok) {
+#pragma unroll
+        for (int v = 0; v < M; ++v) {
+          xm[v] = exm[v];
+          xp[v] = exp_[v];
+          ym[v] = eym[v];
+          yp[v] = eyp[v];
+        }
+      }
+    }
+    vst_sh<M, stride>(sA + tid, xm);
+    vst_sh<M, stride>(sB + tid, xp);
+    vst_sh<M, stride>(sC + tid, ym);
+    vst_sh<M, stride>(sD + tid, yp);
+    __syncthreads();
+    // subcell fluxes (twice their value), numbered across the block: element r /
+    // NSF, its N n x-subfaces, then its n N y-subfaces; the flux right of (above)
+    // node (p2, q2) overwrites that node's x+ (y+) state, which no other reads
+    constexpr int NSX = N * n, NSF = 2 * N * n;
+    for (int gs = tid; gs < epr * NSF; gs += T) {
+      const int el2 = gs / NSF, r = gs - el2 * NSF;
+      const bool isx = r < NSX;
+      const int rr = isx ? r : r - NSX;
+      const int p2 = isx ? rr % N : rr % n, q2 = isx ? rr / N : rr / n;
+      const int node = el2 * NP + p2 + n * q2;
+      double* sL = (isx ? sB : sD) + node;
+      const double* sR = (isx ? sA : sC) + node + (isx ? 1 : n);
+      double uL[M], uR[M], fr[M];
+      vld_sh<M, stride>(uL, sL);
+      vld_sh<M, stride>(uR, sR);
+      rusanov_twice<EQ>(uL, uR, isx ? 0 : 1, fr, ph);
+      vst_sh<M, stride>(sL, fr);
+    }
+    __syncthreads();
+    // low-order residual of the interior subfaces (eq. (low.order.update))
+    {
+      double fr[M], fl[M];
+#pragma unroll
+      for (int v = 0; v < M; ++v) fr[v] = fl[v] = 0.0;
+      if (p < N) vld_sh<M, stride>(fr, sB + tid);
+      if (p > 0) vld_sh<M, stride>(fl, sB + tid - 1);
+      vsub(fr, fr, fl);
+      vmul(LO, fr, sWx[p]);
+#pragma unroll
+      for (int v = 0; v < M; ++v) fr[v] = fl[v] = 0.0;
+      if (q < N) vld_sh<M, stride>(fr, sD + tid);
+      if (q > 0) vld_sh<M, stride>(fl, sD + tid - n);
+      vsub(fr, fr, fl);
+      vfma(LO, sWy[q], fr);
+    }
+    // face-node data for the face kernel: evolved boundary state u* and the
+    // candidate base of the flux limiter, u_b -+ c f_adj
+    const double hdt = 0.5 * dt;
+#pragma unroll
+    for (int mm = 0; mm < SPT; ++mm) {
+      const FaceSlot fs = face_slot<NSLOT, n>(tid + mm * T);
+      const int eg = blk * epr + fs.el;
+      if (fs.el < epr && eg < m.ne) {
+        const int side = fs.side, j = fs.j, base = fs.el * NP;
+        const int nb_node = base + (side == 0 ? n * j : side == 1 ? N + n * j : side == 2 ? j : j + n * N);
+        const int adj_node = nb_node - (side == 1 ? 1 : side == 3 ? n : 0);
+        const double* ust = side == 0 ? sA : side == 1 ? sB : side == 2 ? sC : sD;
+        const double* adj = side < 2 ? sB : sD;
+        const double c = hdt * ((side & 1) ? ph.cflim[side] : -ph.cflim[side]);
+        double us[M], ub[M], fa[M];
+        vld_sh<M, stride>(us, ust + nb_node);
+        vld_sh<M, stride>(ub, s0 + nb_node);
+        vld_sh<M, stride>(fa, adj + adj_node);
+        vfma(ub, c, fa);
+#pragma unroll
+        for (int v = 0; v < M; ++v) {
+          P.b.slot[slot_index(1 + 2 * M + v, side, eg, j, 4, m.ne, n)] = us[v];
+          P.b.slot[slot_index(1 + 3 * M + v, side, eg, j, 4, m.ne, n)] = ub[v];
+        }
+      }
+    }
+  }
+
+  // ---------------- partial update --------------------------------------
+  if (valid) {
+    double val[M];
+    vfma(val, -(dt * a), LO, HO);
+#pragma unroll
+    for (int v = 0; v < M; ++v) P.b.P[((size_t)v * m.ne + e) * NP + k] = val[v];
+  }
+}
+
+}  // namespace crk
