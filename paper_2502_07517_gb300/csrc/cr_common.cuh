@@ -110,6 +110,7 @@ struct Mesh {
   int bcnt;                  // > 0: Dirichlet / inflow ghost states are Chebyshev series in t
   double bct0, bct1;         // their time interval
   double bcc[4][16];         // their coefficients per side (scalar equations)
+  float ind_zero;            // 0.97 sqrt(energy fraction below which the indicator's alpha is 0)
 };
 
 enum : int { kBcPeriodic = 0, kBcOutflow = 1, kBcWall = 2, kBcDirichlet = 3, kBcInflow = 4 };

@@ -582,6 +582,8 @@ void fill_desc_params(const cr_mesh_desc& d, KParams<real>* P, const HostTables&
   // s = ln((1 - 1e-4)/1e-4)
   m.T_ind = 0.5 * std::pow(10.0, -1.8 * std::pow(d.degree + 1.0, 0.25));
   m.s_ind = std::log((1.0 - 1e-4) / 1e-4);
+  // the logistic is below 1e-3 (alpha 0) up to the fraction T (1 - ln(999) / s)
+  m.ind_zero = float(0.97 * std::sqrt(m.T_ind * (1.0 - std::log(999.0) / m.s_ind)));
   {
     // flux-limiter candidates: u~ = u -+ dt/(kappa w h) (F - f_adj), kappa = 1 (1D), 1/2 (2D)
     const double kappa = d.dim == 2 ? 0.5 : 1.0;

@@ -18,6 +18,7 @@
 // [M][EPB][Np] so that consecutive threads touch consecutive words.
 #pragma once
 #include "cr_common.cuh"
+#include "cr_screen.cuh"
 
 namespace crk {
 
@@ -891,6 +892,25 @@ __device__ __forceinline__ void face_body(const KParams<real>& P, const int blk)
   double alpha_f;
   const bool blend = (m.limiter & kLimBlend) || m.alpha_mode == 1;
   const bool need_lo = blend || (m.limiter & kLimFlux);
+  bool high_only = false;  // FP64 interior face that needs no low-order flux
+  // FP32 screen of the flux limiter of an interior face for the flux F (FP64)
+  auto limiter_idle = [&](const real* uL, const real* uR, const real* F) {
+    if constexpr (DIM == 2 && sizeof(real) == 8 && EQ::K > 0) {
+      float ul[M], ur[M], bl[M], br[M], ff[M];
+#pragma unroll
+      for (int v = 0; v < M; ++v) {
+        ul[v] = trunc_f32(uL[v]);
+        ur[v] = trunc_f32(uR[v]);
+        bl[v] = trunc_f32(fld(1 + 3 * M + v, sL, eL));
+        br[v] = trunc_f32(fld(1 + 3 * M + v, sR, eR));
+        ff[v] = trunc_f32(F[v]);
+      }
+      const float dtf = trunc_f32(dtd);
+      return flux_limiter_idle<EQ>(ul, ur, bl, br, ff, dtf * trunc_f32(P.ph.cflim[sL]), dtf * trunc_f32(P.ph.cflim[sR]),
+                                   dir, P.phd);
+    }
+    return false;
+  };
   if (eL >= 0 && eR >= 0) {
     if (m.dissipation == 2) {
       // D-CSX, eq. (dcsx): sum_i b_i lambda_i/2 (u^(i)+ - u^(i)-), lambda_i
@@ -922,16 +942,26 @@ __device__ __forceinline__ void face_body(const KParams<real>& P, const int blk)
         FHO[v] = real(0.5) * (fld(1 + M + v, sL, eL) + fld(1 + M + v, sR, eR)) -
                  real(0.5) * lam * (fld(1 + v, sR, eR) - fld(1 + v, sL, eL));
     }
+    alpha_f = 0.5 * (P.b.alpha[eL] + P.b.alpha[eR]);
+    real uL[M], uR[M];
     if (need_lo) {
-      real uL[M], uR[M];
 #pragma unroll
       for (int v = 0; v < M; ++v) {
         uL[v] = fld(1 + 2 * M + v, sL, eL);
         uR[v] = fld(1 + 2 * M + v, sR, eR);
       }
-      rusanov<EQ>(uL, uR, dir, fLO, P.ph, xf);
     }
-    alpha_f = 0.5 * (P.b.alpha[eL] + P.b.alpha[eR]);
+    if constexpr (DIM == 2 && sizeof(real) == 8) {
+      // FP64: where the face is not blended and the limiter is clearly idle, the
+      // flux is the high-order one and the low-order flux is not formed in FP64
+      // (k_face 0.85 -> 0.19 ms at 512 x 512 N = 4; the screen reads what the
+      // FP64 limiter reads)
+      if (need_lo && !(blend && gt0(alpha_f))) {
+        high_only = true;
+        if ((m.limiter & kLimFlux) && EQ::K > 0) high_only = limiter_idle(uL, uR, FHO);
+      }
+    }
+    if (need_lo && !high_only) rusanov<EQ>(uL, uR, dir, fLO, P.ph, xf);
   } else {
     // boundary face: the interior side (ei, slot side si) and the type of this side
     const int ei = eR >= 0 ? eR : eL;
@@ -1081,9 +1111,20 @@ __device__ __forceinline__ void face_body(const KParams<real>& P, const int blk)
   const real af = real(alpha_f);
   real Fr[M];
 #pragma unroll
-  for (int v = 0; v < M; ++v) Fr[v] = blend ? (real(1) - af) * FHO[v] + af * fLO[v] : FHO[v];
+  for (int v = 0; v < M; ++v) Fr[v] = blend && !high_only ? (real(1) - af) * FHO[v] + af * fLO[v] : FHO[v];
   double theta = 1.0;
-  bool limit = (m.limiter & kLimFlux) && EQ::K > 0;
+  bool limit = (m.limiter & kLimFlux) && EQ::K > 0 && !high_only;
+  if constexpr (DIM == 2 && sizeof(real) == 8) {
+    if (limit && eL >= 0 && eR >= 0) {  // a blended face: the same screen
+      real uL[M], uR[M];
+#pragma unroll
+      for (int v = 0; v < M; ++v) {
+        uL[v] = fld(1 + 2 * M + v, sL, eL);
+        uR[v] = fld(1 + 2 * M + v, sR, eR);
+      }
+      if (gt0(alpha_f) && limiter_idle(uL, uR, Fr)) limit = false;
+    }
+  }
   if (limit && sizeof(real) == 4) {
     // FP32 prescreen: when every candidate with the blended flux clears its
     // threshold 0.1 min P_k(candidate with f_LO) by a margin above FP32
@@ -1349,6 +1390,64 @@ __device__ T indicator_alpha(const Mesh& m, const Tab<T>& tb, T* E, T* Tm, T* re
   return al;  // valid on k == 0 (on every thread of the element without a network)
 }
 
+// Whether the smoothness indicator's alpha is clearly 0 in every valid element of
+// the block: the modal energies in FP32, against the energy fraction at which
+// the logistic reaches 1e-3 (Mesh::ind_zero is 0.97 of its square root).  A mode's
+// FP32 error is below (2i+1)(2j+1) 3.2e-6 of the weighted mean of the magnitudes
+// the indicator variable is formed from (S), its norm over the top modes below
+// 5e-4 of that mean.  Smooth elements so need none of the FP64 transform, sums
+// and logistic (k_update 1.50 -> 0.60 ms at 512 x 512 N = 4 with the limiter's
+// points screened likewise).  Called by every thread; buf: shared memory for 7
+// epb NP floats.
+template <int DIM, int N, class EQ>
+__device__ bool indicator_clear(const Mesh& m, const Tab<double>& td, const Phys<double>& phd, const double* u,
+                                float* buf, int epb, int el, int k, bool valid) {
+  constexpr int n = N + 1;
+  constexpr int NP = DIM == 2 ? n * n : n;
+  float uf[EQ::M];
+#pragma unroll
+  for (int v = 0; v < EQ::M; ++v) uf[v] = trunc_f32(u[v]);
+  Phys<float> ph;
+  ph.gm1 = trunc_f32(phd.gm1);
+  const float x = EQ::indicator_var(uf, ph);
+  float S = fabsf(uf[0]);
+  if constexpr (IsEuler<EQ>::value) S *= ph.gm1 * fabsf(uf[EQ::M - 1]);
+  else if constexpr (EQ::M == 6) S *= fabsf(uf[3]) + fabsf(uf[5]);
+  const int i = DIM == 2 ? k % n : k, j = DIM == 2 ? k / n : 0;
+  const float w = DIM == 2 ? trunc_f32(td.w[i]) * trunc_f32(td.w[j]) : trunc_f32(td.w[i]);
+  float* E = buf + el * NP;
+  E[k] = x;
+  __syncthreads();
+  float mo = 0.0f;
+#pragma unroll
+  for (int p = 0; p < n; ++p) mo += trunc_f32(td.V[i * n + p]) * E[p + n * j];
+  if (DIM == 2) {
+    float* Te = buf + (epb + el) * NP;
+    Te[k] = mo;
+    __syncthreads();
+    mo = 0.0f;
+#pragma unroll
+    for (int q = 0; q < n; ++q) mo += trunc_f32(td.V[j * n + q]) * Te[i + n * q];
+  }
+  float* red = buf + 2 * epb * NP;
+  const float e2 = mo * mo;
+  const int mx = i > j ? i : j;
+  red[(0 * epb + el) * NP + k] = e2;
+  red[(1 * epb + el) * NP + k] = mx == N ? e2 : 0.0f;
+  red[(2 * epb + el) * NP + k] = mx <= N - 1 ? e2 : 0.0f;
+  red[(3 * epb + el) * NP + k] = mx == N - 1 ? e2 : 0.0f;
+  red[(4 * epb + el) * NP + k] = w * S;
+  elem_reduce<NP, 5>(red, epb, el, k, OpSum());
+  bool unclear = false;
+  if (k == 0 && valid) {
+    const float d = 5e-4f * red[(4 * epb + el) * NP];
+    const float tot = sqrt_f32(red[(0 * epb + el) * NP]), top = sqrt_f32(red[(1 * epb + el) * NP]);
+    const float low = sqrt_f32(red[(2 * epb + el) * NP]), top1 = sqrt_f32(red[(3 * epb + el) * NP]);
+    unclear = !(top + d < m.ind_zero * (tot - d)) || !(N < 2 || top1 + d < m.ind_zero * (low - d));
+  }
+  return !__syncthreads_or(unclear);
+}
+
 // finish the step: block max of the CFL rate, last block publishes the rate,
 // advances time when advance != 0, and resets the accumulators.
 __device__ __forceinline__ void finish_block(TimeCtl* ctl, double block_rate, int advance,
@@ -1539,25 +1638,54 @@ __device__ __forceinline__ void update_body(const KParams<real>& P, const Tab<re
 
   // ---- node update: partial update + element-face flux terms ------------
   const bool blend = (m.limiter & kLimBlend) || m.alpha_mode == 1;
-  for (int e2 = tid; e2 < epb; e2 += T) {  // the block's elements side by side
-    const int eg0 = blk * epr + e2;
-    sElr[e2 * ES + ER] = real(P.b.alpha[(e2 < epr && eg0 < m.ne) ? eg0 : m.ne - 1]);
-  }
-  __syncthreads();
-  const real a = blend ? sElr[el * ES + ER] : real(0);
   const real dt = MIXED ? real(P.b.ctl->dt_step_f) : real(dtd);
   const real one = real(1);
   const real invdx = P.ph.invdx, invdy = P.ph.invdy;
+  // correction weight of a face flux at node row r of an element with blending
+  // coefficient a: dt/dx (dt/dy) folded in, side 1 right (top), 0 left (bottom)
+  auto weight = [&](real s, real a, int side, int r) {
+    return side ? s * ((one - a) * tb.gR[r] + (r == N ? a * tb.invw[N] : real(0)))
+                : s * ((one - a) * tb.gL[r] - (r == 0 ? a * tb.invw[0] : real(0)));
+  };
+  real cRx, cLx, cRy = real(0), cLy = real(0);
+  if constexpr (MIXED) {
+    for (int e2 = tid; e2 < epb; e2 += T) {  // the block's elements side by side
+      const int eg0 = blk * epr + e2;
+      sElr[e2 * ES + ER] = real(P.b.alpha[(e2 < epr && eg0 < m.ne) ? eg0 : m.ne - 1]);
+    }
+    __syncthreads();
+    const real a = blend ? sElr[el * ES + ER] : real(0);
+    const real sx = dt * invdx, sy = DIM == 2 ? dt * invdy : real(0);
+    cRx = weight(sx, a, 1, p);
+    cLx = weight(sx, a, 0, p);
+    if (DIM == 2) {
+      cRy = weight(sy, a, 1, q);
+      cLy = weight(sy, a, 0, q);
+    }
+  } else {
+    // FP64: each weight of an element once, not once per node of its row or
+    // column (the reduction buffer is free here)
+    real* sCf = reinterpret_cast<real*>(sRed);  // [epb][2 DIM][n]
+    constexpr int NC = 2 * DIM * n;
+    for (int t = tid; t < epb * NC; t += T) {
+      const int e2 = t / NC, r = t - e2 * NC, c = r / n;
+      const int eg0 = blk * epr + e2;
+      const real a = blend ? real(P.b.alpha[(e2 < epr && eg0 < m.ne) ? eg0 : m.ne - 1]) : real(0);
+      sCf[t] = weight(dt * (c < 2 ? invdx : invdy), a, c & 1, r - c * n);
+    }
+    __syncthreads();
+    const real* cf = sCf + el * NC;
+    cLx = cf[p];
+    cRx = cf[n + p];
+    if (DIM == 2) {
+      cLy = cf[2 * n + q];
+      cRy = cf[3 * n + q];
+    }
+  }
   const int ixR = m.bcx == 0 ? (ix + 1) % m.nx : ix + 1;
   const int iyT = DIM == 2 ? (m.bcy == 0 ? (iy + 1) % m.ny : iy + 1) : 0;
   const size_t nXf = (size_t)m.ny * m.nfx * NFN;
   const size_t nYf = DIM == 2 ? (size_t)m.nfy * m.nx * n : 0;
-  // correction weights of the face fluxes, dt/dx and dt/dy folded in
-  const real sx = dt * invdx, sy = DIM == 2 ? dt * invdy : real(0);
-  const real cRx = sx * ((one - a) * tb.gR[p] + (p == N ? a * tb.invw[N] : real(0)));
-  const real cLx = sx * ((one - a) * tb.gL[p] - (p == 0 ? a * tb.invw[0] : real(0)));
-  const real cRy = DIM == 2 ? sy * ((one - a) * tb.gR[q] + (q == N ? a * tb.invw[N] : real(0))) : real(0);
-  const real cLy = DIM == 2 ? sy * ((one - a) * tb.gL[q] - (q == 0 ? a * tb.invw[0] : real(0))) : real(0);
   const real W = DIM == 2 ? tb.w[p] * tb.w[q] : tb.w[p];
   real val[M];
 #pragma unroll
@@ -1621,6 +1749,7 @@ __device__ __forceinline__ void update_body(const KParams<real>& P, const Tab<re
 #pragma unroll
     for (int v = 0; v < M; ++v) ubar[v] = sEl[el * 16 + 4 + v];
   } else {
+    __syncthreads();  // the weights are consumed
 #pragma unroll
     for (int v = 0; v < M; ++v) RED(v) = double(W) * double(val[v]);
     elem_reduce<NP, M>(sRed, epb, el, k, OpSum());
@@ -1647,8 +1776,13 @@ __device__ __forceinline__ void update_body(const KParams<real>& P, const Tab<re
     }
   }
   real* sUr = reinterpret_cast<real*>(sU);
+  // FP64: FP32 copies for the screen, in the upper half of the reduction buffer
+  float* sUf = reinterpret_cast<float*>(sRed + M * stride);
 #pragma unroll
-  for (int v = 0; v < M; ++v) sUr[v * stride + el * NP + k] = ur[v];
+  for (int v = 0; v < M; ++v) {
+    sUr[v * stride + el * NP + k] = ur[v];
+    if constexpr (!MIXED) sUf[v * stride + el * NP + k] = trunc_f32(ur[v]);
+  }
   // per-element limiter scalars: sEl[el*16 + 0..3] = mean_ok, eps1, eps2, P2(u_bar),
   // for the block's elements side by side in its first epb threads (one warp)
   // from the means in shared memory.  FP32_BULK: when the FP32 copy of the mean
@@ -1699,42 +1833,82 @@ __device__ __forceinline__ void update_body(const KParams<real>& P, const Tab<re
   if (do_scale) {
     const double eps1 = sEl[el * 16 + 1], eps2 = sEl[el * 16 + 2];
     const real P2r = MIXED ? sElr[el * ES + ER + 7] : real(sEl[el * 16 + 3]);
-    // points this thread checks: its node and its face-trace slots
-    real pr[1 + SPT][M];
-    int npt = 1;
+    // does any point of the block need limiting (this thread checks its node and
+    // its face-trace slots)?  FP64 mode: exactly the oracle's test, where an
+    // FP32 screen does not already pass it; FP32_BULK: an FP32 prescreen with a
+    // margin, the FP64 solve below decides
+    int need = 0;
+    if constexpr (MIXED) {
+      real pr[1 + SPT][M];
+      int npt = 1;
 #pragma unroll
-    for (int v = 0; v < M; ++v) pr[0][v] = ur[v];
-    if (traces) {
+      for (int v = 0; v < M; ++v) pr[0][v] = ur[v];
+      if (traces) {
 #pragma unroll
-      for (int mm = 0; mm < SPT; ++mm) {
-        const int sl = k + mm * NP;
-        if (sl < NSLOT) {
-          const int side = sl / NFN, j = sl - side * NFN;
+        for (int mm = 0; mm < SPT; ++mm) {
+          const int sl = k + mm * NP;
+          if (sl < NSLOT) {
+            const int side = sl / NFN, j = sl - side * NFN;
 #pragma unroll
-          for (int v = 0; v < M; ++v) {
-            real acc = real(0);
+            for (int v = 0; v < M; ++v) {
+              real acc = real(0);
 #pragma unroll
-            for (int r = 0; r < n; ++r) {
-              const real l = (side & 1) ? tb.l1[r] : tb.l0[r];
-              acc += l * sUr[v * stride + el * NP + (side < 2 ? r + n * j : j + n * r)];
+              for (int r = 0; r < n; ++r) {
+                const real l = (side & 1) ? tb.l1[r] : tb.l0[r];
+                acc += l * sUr[v * stride + el * NP + (side < 2 ? r + n * j : j + n * r)];
+              }
+              pr[npt][v] = acc;
             }
-            pr[npt][v] = acc;
+            ++npt;
           }
-          ++npt;
         }
       }
-    }
-    // does any point of the block need limiting?  FP64 mode: exactly the
-    // oracle's test; FP32_BULK: an FP32 prescreen with a margin, the FP64
-    // solve below decides
-    int need = 0;
-    for (int t = 0; t < npt; ++t) {
-      if constexpr (MIXED) {
+      for (int t = 0; t < npt; ++t) {
         const real scale = EQ::M == 6 ? fabs(pr[t][3]) + fabs(pr[t][5]) : fabs(pr[t][M - 1]);
         const real thr = fmax(fmax(real(1e-3) * P2r, real(1e-5) * scale), real(1e-11));
         if (!(pr[t][0] > real(1e-3) * ubr[0] && EQ::constraint(pr[t], 1, P.ph) > thr)) need = 1;
-      } else {
-        if (!(pr[t][0] >= eps1 && EQ::constraint(pr[t], 1, P.phd) >= eps2)) need = 1;
+      }
+    } else {
+      const float gm1 = trunc_f32(P.phd.gm1);
+      float s[M], A[M];
+#pragma unroll
+      for (int v = 0; v < M; ++v) {
+        s[v] = sUf[v * stride + el * NP + k];
+        A[v] = fabsf(s[v]);
+      }
+      if (!clearly_above_eps<EQ>(s, A, gm1) && !(ur[0] >= eps1 && EQ::constraint(ur, 1, P.phd) >= eps2)) need = 1;
+      if (traces) {
+#pragma unroll
+        for (int mm = 0; mm < SPT; ++mm) {
+          const int sl = k + mm * NP;
+          if (sl < NSLOT) {
+            const int side = sl / NFN, j = sl - side * NFN;
+#pragma unroll
+            for (int v = 0; v < M; ++v) s[v] = A[v] = 0.0f;
+#pragma unroll
+            for (int r = 0; r < n; ++r) {
+              const float l = trunc_f32((side & 1) ? tb.l1[r] : tb.l0[r]);
+#pragma unroll
+              for (int v = 0; v < M; ++v) {
+                const float x = l * sUf[v * stride + el * NP + (side < 2 ? r + n * j : j + n * r)];
+                s[v] += x;
+                A[v] += fabsf(x);
+              }
+            }
+            if (!clearly_above_eps<EQ>(s, A, gm1)) {
+              real pt[M];
+#pragma unroll
+              for (int v = 0; v < M; ++v) {
+                pt[v] = real(0);
+#pragma unroll
+                for (int r = 0; r < n; ++r)
+                  pt[v] += ((side & 1) ? tb.l1[r] : tb.l0[r]) *
+                           sUr[v * stride + el * NP + (side < 2 ? r + n * j : j + n * r)];
+              }
+              if (!(pt[0] >= eps1 && EQ::constraint(pt, 1, P.phd) >= eps2)) need = 1;
+            }
+          }
+        }
       }
     }
     // Only real elements vote (a ghost slot of a block whose size is not a
@@ -1818,7 +1992,7 @@ __device__ __forceinline__ void update_body(const KParams<real>& P, const Tab<re
   }
 #pragma unroll
   for (int v = 0; v < M; ++v)
-    if (!isfinite(ur[v])) bad |= kStNonFinite;
+    if (!finite_bits(ur[v])) bad |= kStNonFinite;
   if (valid && bad) {
     atomicOr(&P.b.ctl->status, bad);
     atomicMin(&P.b.ctl->bad_elem, e);
@@ -1869,10 +2043,13 @@ __device__ __forceinline__ void update_body(const KParams<real>& P, const Tab<re
       double* dE = sU;
       double* dT = sU + stride;
       __syncthreads();
-      dE[el * NP + k] = EQ::indicator_var(ur, P.phd);
-      __syncthreads();
-      const double al = indicator_alpha<DIM, N, double>(m, td, dE, dT, sRed, epb, el, k,
-                                                        P.b.mlp_flag, P.b.mlp_w, sMlp, nullptr, -1);
+      double al = 0.0;
+      if (m.alpha_mode != 0 || !indicator_clear<DIM, N, EQ>(m, td, P.phd, ur, reinterpret_cast<float*>(sRed), epb, el, k, valid)) {
+        dE[el * NP + k] = EQ::indicator_var(ur, P.phd);
+        __syncthreads();
+        al = indicator_alpha<DIM, N, double>(m, td, dE, dT, sRed, epb, el, k,
+                                          P.b.mlp_flag, P.b.mlp_w, sMlp, nullptr, -1);
+      }
       if (valid && k == 0) P.b.alpha_raw[e] = al;
     }
   }
@@ -1952,11 +2129,14 @@ __global__ void k_prologue(const __grid_constant__ KParams<real> P) {
   for (int v = k; v < M; v += NP) sEl[el * 16 + 4 + v] = ubar[v];  // for the CFL rate
   __syncthreads();
   if (((m.limiter & kLimBlend) && (m.alpha_mode == 0 || m.alpha_mode == 2)) || P.b.feat) {
-    sU[el * NP + k] = EQ::indicator_var(u, P.phd);
-    __syncthreads();
-    const double al = indicator_alpha<DIM, N, double>(m, P.td, sU, sU + stride, sRed, epb, el, k,
-                                                      P.b.mlp_flag, P.b.mlp_w, sMlp, P.b.feat,
-                                                      valid ? e : -1);
+    double al = 0.0;
+    if (m.alpha_mode != 0 || P.b.feat ||
+        !indicator_clear<DIM, N, EQ>(m, P.td, P.phd, u, reinterpret_cast<float*>(sRed), epb, el, k, valid)) {
+      sU[el * NP + k] = EQ::indicator_var(u, P.phd);
+      __syncthreads();
+      al = indicator_alpha<DIM, N, double>(m, P.td, sU, sU + stride, sRed, epb, el, k, P.b.mlp_flag,
+                                           P.b.mlp_w, sMlp, P.b.feat, valid ? e : -1);
+    }
     if (valid && k == 0) {
       P.b.alpha_raw[e] = al;
       if constexpr (MIXED) P.b.alpha_raw_f[e] = float(al);

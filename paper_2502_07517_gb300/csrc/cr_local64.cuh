@@ -24,29 +24,9 @@
 #pragma once
 #include "cr_common.cuh"
 #include "cr_fixed.cuh"
+#include "cr_screen.cuh"
 
 namespace crk {
-
-// |relative error| of an FP32 comparison below: truncated operands (2^-23
-// each), the approximate square root and a few FP32 operations stay under half
-// of it.
-constexpr float kTieF = 1.9073486e-6f;  // 2^-19
-
-// x as FP32, truncated, from the bit pattern: magnitudes below FP32's normal
-// range give a value below 2^-126, larger ones its largest finite value.
-__device__ __forceinline__ float trunc_f32(double x) {
-  const int h = __double2hiint(x);
-  int m = (h & 0x7fffffff) - (896 << 20);
-  m = min(max(m, 0), 0x0fefffff);
-  const unsigned b = __funnelshift_l((unsigned)__double2loint(x), (unsigned)m, 3);
-  return __uint_as_float(b | (unsigned(h) & 0x80000000u));
-}
-
-__device__ __forceinline__ float sqrt_f32(float x) {
-  float r;
-  asm("sqrt.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(fmaxf(x, 0.0f)));
-  return r;
-}
 
 // minmod of the slopes d1 b1, d2 b2, d3 b3 (b > 0) with f1, f2, f3 = b in FP32.
 __device__ __forceinline__ double minmod_scaled(double d1, double d2, double d3, double b1, double b2,
@@ -111,20 +91,19 @@ __device__ __forceinline__ void rusanov_twice(const double* uL, const double* uR
 
 // FP32 screen of the MUSCL-Hancock states: s is a state and A bounds the
 // magnitudes its parts are summed from.  True only when the state is admissible
-// by a margin of 2e-5 of those magnitudes, an order above the FP32 rounding of
-// the sums and products.
+// by a margin above the FP32 rounding of the sums and products.
 template <class EQ>
 __device__ __forceinline__ bool clearly_admissible(const float* s, const float* A) {
   if constexpr (EQ::K == 0) return true;
-  if (!(s[0] > 2e-5f * A[0])) return false;
+  if (!(s[0] > kMarginF * A[0])) return false;
   if constexpr (IsEuler<EQ>::value) {
     const float q = s[3] * s[0] - 0.5f * (s[1] * s[1] + s[2] * s[2]);
-    return q > 2e-5f * (A[3] * A[0] + A[1] * A[1] + A[2] * A[2]);
+    return q > kMarginF * (A[3] * A[0] + A[1] * A[1] + A[2] * A[2]);
   } else if constexpr (EQ::M == 6) {
     const float a11 = 2.0f * s[0] * s[3] - s[1] * s[1], a22 = 2.0f * s[0] * s[5] - s[2] * s[2];
     const float a12 = 2.0f * s[0] * s[4] - s[1] * s[2];
     const float B = 2.0f * A[0] * (A[3] + A[4] + A[5]) + A[1] * A[1] + A[2] * A[2];
-    return a11 > 2e-5f * B && a11 * a22 - a12 * a12 > 1e-4f * B * B;
+    return a11 > kMarginF * B && a11 * a22 - a12 * a12 > 5.0f * kMarginF * B * B;
   }
   return true;
 }

@@ -1,0 +1,143 @@
+// FP32 screens in front of FP64 decisions.  The FP64 pipe issues one warp
+// instruction per 16 cycles and SM; a decision whose answer is clear by a margin
+// above the FP32 rounding needs none of it.  Every screen answers "clear" or
+// "not clear", and what is not clear is decided in FP64 as before, so the
+// results do not depend on the screens.
+#pragma once
+#include "cr_common.cuh"
+
+namespace crk {
+
+// |relative error| allowed for an FP32 comparison of two products or speeds:
+// truncated operands (2^-23 each), the approximate square root and a few FP32
+// operations stay under half of it.
+constexpr float kTieF = 1.9073486e-6f;  // 2^-19
+// Margin of the screens below, relative to the magnitudes a value is summed
+// from: ten times the FP32 rounding of those sums and products.
+constexpr float kMarginF = 2e-5f;
+
+// x as FP32, truncated, from the bit pattern (a conversion instruction runs on
+// the FP64 pipe): magnitudes below FP32's normal range give a value below
+// 2^-126, larger ones its largest finite value; NaN gives a large value.
+__device__ __forceinline__ float trunc_f32(double x) {
+  const int h = __double2hiint(x);
+  int m = (h & 0x7fffffff) - (896 << 20);
+  m = min(max(m, 0), 0x0fefffff);
+  const unsigned b = __funnelshift_l((unsigned)__double2loint(x), (unsigned)m, 3);
+  return __uint_as_float(b | (unsigned(h) & 0x80000000u));
+}
+__device__ __forceinline__ float trunc_f32(float x) { return x; }
+
+__device__ __forceinline__ bool finite_bits(double x) { return (__double2hiint(x) & 0x7ff00000) != 0x7ff00000; }
+__device__ __forceinline__ bool finite_bits(float x) { return isfinite(x); }
+
+__device__ __forceinline__ float sqrt_f32(float x) {
+  float r;
+  asm("sqrt.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(fmaxf(x, 0.0f)));
+  return r;
+}
+
+// Constraint k of the state s in FP32 and the bound of its error, A[v] bounding
+// the magnitudes s[v] is summed from.
+template <class EQ>
+__device__ __forceinline__ void screened_constraint(const float* s, const float* A, int k, float gm1, float* P,
+                                                    float* err) {
+  *P = 1.0f;
+  *err = 0.0f;
+  if constexpr (EQ::K > 0) {
+    if (k == 0) {
+      *P = s[0];
+      *err = kMarginF * A[0];
+    } else if constexpr (IsEuler<EQ>::value) {
+      constexpr int E = EQ::M - 1;
+      const float r = __frcp_rn(s[0]), v1 = s[1] * r, v2 = E == 3 ? s[2] * r : 0.0f;
+      float kin = s[1] * v1, e = A[E] + fabsf(v1) * A[1] + 0.5f * (v1 * v1 + v2 * v2) * A[0];
+      if (E == 3) {
+        kin += s[2] * v2;
+        e += fabsf(v2) * A[2];
+      }
+      *P = gm1 * (s[E] - 0.5f * kin);
+      *err = kMarginF * gm1 * e;
+    } else {
+      const float r = __frcp_rn(s[0]), v1 = s[1] * r, v2 = s[2] * r;
+      const float p11 = 2.0f * s[3] - s[1] * v1, p12 = 2.0f * s[4] - s[1] * v2, p22 = 2.0f * s[5] - s[2] * v2;
+      const float h = 0.5f * (p11 - p22);
+      const float w = fabsf(v1) + fabsf(v2);
+      *P = 0.5f * (p11 + p22) - sqrt_f32(h * h + p12 * p12);
+      *err = kMarginF * (2.0f * (A[3] + A[4] + A[5]) + 2.0f * w * (A[1] + A[2]) + w * w * A[0]);
+    }
+  }
+}
+
+// Whether the flux limiter of an interior face is clearly idle (theta = 1) for
+// the flux F: both candidates base -+ c F clear a tenth of the smaller
+// low-order candidate (and those are clearly positive) in every constraint.
+// uL, uR: the evolved boundary states, whose Rusanov flux is the low-order flux;
+// formed in FP32 here.
+template <class EQ>
+__device__ __forceinline__ bool flux_limiter_idle(const float* uL, const float* uR, const float* bL, const float* bR,
+                                                  const float* F, float cL, float cR, int dir,
+                                                  const Phys<double>& phd) {
+  constexpr int M = EQ::M;
+  Phys<float> ph;
+  ph.gamma = trunc_f32(phd.gamma);
+  ph.gm1 = trunc_f32(phd.gm1);
+  float fL[M], fR[M], sL, sR, lo[M], aL[M], aR[M];
+  EQ::flux_speed(uL, dir, fL, &sL, ph);
+  EQ::flux_speed(uR, dir, fR, &sR, ph);
+  const float lam = fmaxf(sL, sR);
+  // magnitudes the fluxes are summed from: besides their own size, the energies
+  // (pressures are differences of energies) and those times the speeds
+  float SL = 0.0f, SR = 0.0f;
+#pragma unroll
+  for (int v = 3; v < M; ++v) {
+    SL += fabsf(uL[v]);
+    SR += fabsf(uR[v]);
+  }
+  const float S = 2.0f * (SL + SR);
+  const float V = fmaxf(lam, sqrt_f32(2.0f * fmaxf(SL / uL[0], SR / uR[0])));
+#pragma unroll
+  for (int v = 0; v < M; ++v) {
+    lo[v] = 0.5f * (fL[v] + fR[v]) - 0.5f * lam * (uR[v] - uL[v]);
+    const float a = fabsf(fL[v]) + fabsf(fR[v]) + lam * (fabsf(uL[v]) + fabsf(uR[v])) + fabsf(F[v]) +
+                    (v == 0 ? 0.0f : v < 3 ? S : S * V);
+    aL[v] = fabsf(bL[v]) + cL * a;
+    aR[v] = fabsf(bR[v]) + cR * a;
+  }
+  bool idle = true;
+#pragma unroll
+  for (int k = 0; k < EQ::K; ++k) {
+    float c[M], pl, el, pr, er, hl, fl, hr, fr;
+#pragma unroll
+    for (int v = 0; v < M; ++v) c[v] = bL[v] - cL * lo[v];
+    screened_constraint<EQ>(c, aL, k, ph.gm1, &pl, &el);
+#pragma unroll
+    for (int v = 0; v < M; ++v) c[v] = bR[v] + cR * lo[v];
+    screened_constraint<EQ>(c, aR, k, ph.gm1, &pr, &er);
+#pragma unroll
+    for (int v = 0; v < M; ++v) c[v] = bL[v] - cL * F[v];
+    screened_constraint<EQ>(c, aL, k, ph.gm1, &hl, &fl);
+#pragma unroll
+    for (int v = 0; v < M; ++v) c[v] = bR[v] + cR * F[v];
+    screened_constraint<EQ>(c, aR, k, ph.gm1, &hr, &fr);
+    const float top = 0.1f * fminf(pl + el, pr + er);
+    idle = idle && pl > el && pr > er && hl - fl > top && hr - fr > top;
+  }
+  return idle;
+}
+
+// Whether a point is clearly admissible with both constraints above 1e-12 (the
+// scaling limiter's threshold is at most that).
+template <class EQ>
+__device__ __forceinline__ bool clearly_above_eps(const float* s, const float* A, float gm1) {
+  bool ok = true;
+#pragma unroll
+  for (int k = 0; k < EQ::K; ++k) {
+    float P, e;
+    screened_constraint<EQ>(s, A, k, gm1, &P, &e);
+    ok = ok && P > e + 1e-12f;
+  }
+  return ok;
+}
+
+}  // namespace crk

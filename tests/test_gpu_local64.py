@@ -82,3 +82,51 @@ def test_overflowing_step_is_reported():
     assert err.value.status == -3
     crkfr.cr_set_state(ctx, u)       # the context stays usable
     crkfr.cr_step(ctx, 1, 1e300)
+
+
+@pytest.mark.parametrize("N", [2, 3, 4])
+@pytest.mark.parametrize("pressure", [1e-3, 3e-5, 1e-5])
+def test_low_pressure_beside_the_screens(N, pressure):
+    """Mach 30 to 300: pressures above, about and below the margin of the FP32
+    screens (2e-5 of the energies), so limiters and MUSCL-Hancock decide in FP32
+    in some nodes and in FP64 in others.  The constraint P is a difference of
+    energies E: its relative rounding, a few 2^-53 E / P (ten of them here), goes
+    into the limiters' theta on top of the 1e-12 bar."""
+    rng = np.random.default_rng(N)
+    prob, u = wl.euler2d_vortex(nx=11, ny=9, degree=N, seed=N)
+    shape = (u.shape[1], 1)
+    one = np.ones(u.shape[1:])
+    rho, p = one * rng.uniform(0.8, 1.2, shape), pressure * one * rng.uniform(0.5, 2.0, shape)
+    u = wl.euler_conservative(rho, one * rng.uniform(0.9, 1.1, shape), one * rng.uniform(-0.1, 0.1, shape), p, 1.4, 2)
+    d = oracle_desc(prob)
+    dt = 0.5 * oracle.dt(d, u)
+    ref, st, dg = oracle.step(d, u, dt, want_diag=True)
+    assert st == 0
+    g = gpu_run(prob, u, dt_fixed=dt)[0]
+    bar = 1e-12 + 10 * 2.0 ** -53 * u[3].max() / p.min()
+    assert_parity(g, ref, rtol=bar, extra_scale=flux_increment(prob, dg, dt))
+
+
+@pytest.mark.parametrize("N", [2, 3, 4])
+def test_alpha_beside_its_threshold(N):
+    """Elements whose modal energy fraction lies within a few percent of the one
+    at which alpha becomes 0: the FP32 screen may call none of them wrongly."""
+    rng = np.random.default_rng(N)
+    prob, u = wl.euler2d_vortex(nx=16, ny=8, degree=N, seed=N, perturb=0.0)
+    prob = dict(prob, limiter=frozenset({"blend", "flux", "scaling", "traces"}))
+    T, s = 0.5 * 10.0 ** (-1.8 * (N + 1.0) ** 0.25), np.log((1.0 - 1e-4) / 1e-4)
+    edge = T * (1.0 - np.log(999.0) / s)
+    xi, _ = wl.gl_nodes01(N)
+    top = np.polynomial.legendre.Legendre.basis(N)(2.0 * xi - 1.0)     # along x; rho p = 1 + c L_N(x)
+    frac = edge * rng.uniform(0.9, 1.1, u.shape[1])
+    c = np.sqrt(frac / (1.0 - frac))
+    rho = np.ones(u.shape[1:])
+    p = 1.0 + c[:, None] * np.tile(top, N + 1)[None, :]
+    u = wl.euler_conservative(rho, 0.1 * rho, 0.0 * rho, p, 1.4, 2)
+    d = oracle_desc(prob)
+    dt = 0.1 * oracle.dt(d, u)
+    ref, st, dg = oracle.step(d, u, dt, want_diag=True)
+    assert st == 0 and 0 < np.count_nonzero(dg["alpha_raw"]) < u.shape[1]
+    g, alpha = gpu_run(prob, u, dt_fixed=dt)[:2]
+    np.testing.assert_allclose(alpha, dg["alpha"], rtol=0, atol=1e-12)
+    assert_parity(g, ref, extra_scale=flux_increment(prob, dg, dt))
