@@ -958,7 +958,21 @@ __device__ __forceinline__ void face_body(const KParams<real>& P, const int blk)
       // FP64 limiter reads)
       if (need_lo && !(blend && gt0(alpha_f))) {
         high_only = true;
-        if ((m.limiter & kLimFlux) && EQ::K > 0) high_only = limiter_idle(uL, uR, FHO);
+        if ((m.limiter & kLimFlux) && EQ::K > 0) {
+          const bool fL = is_f32_face_data(uL[0]), fR = is_f32_face_data(uR[0]);
+          if (fL) uL[0] = -uL[0];
+          if (fR) uR[0] = -uR[0];
+          high_only = limiter_idle(uL, uR, FHO);
+          if (!high_only && (fL || fR)) {  // left open: the FP64 face data after all
+            if (fL) exact_face_data<N, EQ>(P, P.tb, eL, sL, j, dtd);
+            if (fR) exact_face_data<N, EQ>(P, P.tb, eR, sR, j, dtd);
+#pragma unroll
+            for (int v = 0; v < M; ++v) {
+              uL[v] = fld(1 + 2 * M + v, sL, eL);
+              uR[v] = fld(1 + 2 * M + v, sR, eR);
+            }
+          }
+        }
       }
     }
     if (need_lo && !high_only) rusanov<EQ>(uL, uR, dir, fLO, P.ph, xf);

@@ -19,8 +19,17 @@
 //   - reciprocals and square roots by one third-order and two Newton steps from
 //     the hardware's approximations (recip, sqrt_pos), and factors that depend
 //     on the step or the node row alone formed once per block.
-// Measured (k_local, the same workload): 612 FP64 instructions per point, 12.57
-// -> 8.42 ms; ten-moment N = 3 at 256 x 256 2.61 -> 2.03 ms.
+//   - an element that is neither blended nor beside a blended face or a boundary
+//     needs its low-order scheme only for the flux limiter's inequality, which
+//     the face kernel decides in FP32: there the MUSCL-Hancock states and the
+//     subcell fluxes next to the faces are formed in FP32 (hancock_states_f32),
+//     and the face kernel forms the FP64 data itself where the inequality is not
+//     clear (exact_face_data).  The update is the same: alpha = 0 leaves the
+//     high-order part alone, and theta is decided as in FP64.
+// Measured (k_local, the same workload): the contractions and the first two
+// groups of decisions 12.57 -> 8.42 ms (612 FP64 instructions per point), the
+// low-order scheme in FP32 -> 5.60 ms; ten-moment N = 3 at 256 x 256 2.61 -> 2.03
+// -> 1.56 ms.
 #pragma once
 #include "cr_common.cuh"
 #include "cr_fixed.cuh"
@@ -108,12 +117,202 @@ __device__ __forceinline__ bool clearly_admissible(const float* s, const float* 
   return true;
 }
 
+// MUSCL-Hancock states of one node (Sec. 4.2): the evolved states at the four
+// subcell faces, or the node value where one of them is not admissible.  nb(v,
+// dir, up) is the neighbour node's value along the line; hx, hy = dt / (2 w h).
+template <int N, class EQ, class Nb>
+__device__ __forceinline__ void hancock_states(const Mesh& m, const Phys<double>& ph, const Tab<double>& tb,
+                                               const double (&un)[EQ::M], double alpha, int p, int q, double hx,
+                                               double hy, Nb nb, double (&xm)[EQ::M], double (&xp)[EQ::M],
+                                               double (&ym)[EQ::M], double (&yp)[EQ::M]) {
+  constexpr int M = EQ::M;
+#pragma unroll
+  for (int v = 0; v < M; ++v) xm[v] = xp[v] = ym[v] = yp[v] = un[v];
+  if (!(m.limiter & kLimMH)) return;
+  const double beta = 2.0 - alpha;
+  double sx[M], sy[M];
+  auto slopes = [&](double (&sl)[M], int c, int dir) {
+    const double bm = beta * tb.ihm[c], bc = tb.ihc[c], bp = beta * tb.ihp[c];
+    const float fm = trunc_f32(bm), fc = trunc_f32(bc), fp = trunc_f32(bp);
+#pragma unroll
+    for (int v = 0; v < M; ++v) {
+      const double um = nb(v, dir, 0), up = nb(v, dir, 1);
+      sl[v] = minmod_scaled(un[v] - um, up - um, up - un[v], bm, bc, bp, fm, fc, fp);
+    }
+  };
+  slopes(sx, p, 0);
+  slopes(sy, q, 1);
+  double fxm[M], fxp[M], fym[M], fyp[M], Fm[M], Fp[M], ex[M];
+  vfma(fxm, tb.dm[p], sx, un);
+  vfma(fxp, tb.dp[p], sx, un);
+  vfma(fym, tb.dm[q], sy, un);
+  vfma(fyp, tb.dp[q], sy, un);
+  EQ::flux(fxm, 0, Fm, ph);
+  EQ::flux(fxp, 0, Fp, ph);
+  vsub(ex, Fp, Fm);
+  vmul(ex, ex, hx);
+  EQ::flux(fym, 1, Fm, ph);
+  EQ::flux(fyp, 1, Fp, ph);
+  vsub(Fp, Fp, Fm);
+  vfma(ex, hy, Fp);
+  bool ok = true;
+  if constexpr (EQ::K > 0) {
+    float uf[M], xf[M], yf[M], ef[M], A[M], st[M];
+    const float dmx = trunc_f32(tb.dm[p]), dpx = trunc_f32(tb.dp[p]);
+    const float dmy = trunc_f32(tb.dm[q]), dpy = trunc_f32(tb.dp[q]);
+#pragma unroll
+    for (int v = 0; v < M; ++v) {
+      uf[v] = trunc_f32(un[v]);
+      xf[v] = trunc_f32(sx[v]);
+      yf[v] = trunc_f32(sy[v]);
+      ef[v] = trunc_f32(ex[v]);
+      A[v] = fabsf(uf[v]) + fabsf(xf[v]) + fabsf(yf[v]) + fabsf(ef[v]);
+    }
+#pragma unroll
+    for (int c = 0; c < 8; ++c) {  // four face states, then evolved
+      const float d = (c & 3) == 0 ? dmx : (c & 3) == 1 ? dpx : (c & 3) == 2 ? dmy : dpy;
+#pragma unroll
+      for (int v = 0; v < M; ++v) {
+        st[v] = fmaf(d, (c & 2) ? yf[v] : xf[v], uf[v]);
+        if (c & 4) st[v] -= ef[v];
+      }
+      ok = ok && clearly_admissible<EQ>(st, A);
+    }
+  }
+  double exm[M], exp_[M], eym[M], eyp[M];
+  vsub(exm, fxm, ex);
+  vsub(exp_, fxp, ex);
+  vsub(eym, fym, ex);
+  vsub(eyp, fyp, ex);
+  if (!ok)
+    ok = EQ::admissible_fast(fxm, ph) && EQ::admissible_fast(fxp, ph) && EQ::admissible_fast(exm, ph) &&
+         EQ::admissible_fast(exp_, ph) && EQ::admissible_fast(fym, ph) && EQ::admissible_fast(fyp, ph) &&
+         EQ::admissible_fast(eym, ph) && EQ::admissible_fast(eyp, ph);
+  if (ok) {
+#pragma unroll
+    for (int v = 0; v < M; ++v) {
+      xm[v] = exm[v];
+      xp[v] = exp_[v];
+      ym[v] = eym[v];
+      yp[v] = eyp[v];
+    }
+  }
+}
+
+// The same in FP32, for elements whose low-order scheme only feeds the screen of
+// the flux limiter (see the body).  Returns false where admissibility is not
+// clear in FP32 (the FP64 form then decides).
+template <int N, class EQ, class Nb>
+__device__ __forceinline__ bool hancock_states_f32(const Mesh& m, const Phys<float>& ph, const Tab<double>& tb,
+                                                   const float (&un)[EQ::M], float alpha, int p, int q, float hx,
+                                                   float hy, Nb nb, float (&xm)[EQ::M], float (&xp)[EQ::M],
+                                                   float (&ym)[EQ::M], float (&yp)[EQ::M]) {
+  constexpr int M = EQ::M;
+#pragma unroll
+  for (int v = 0; v < M; ++v) xm[v] = xp[v] = ym[v] = yp[v] = un[v];
+  if (!(m.limiter & kLimMH)) return EQ::K == 0 || un[0] > 1e-30f;
+  const float beta = 2.0f - alpha;
+  float sx[M], sy[M], A[M];
+  auto slopes = [&](float (&sl)[M], int c, int dir) {
+    const float bm = beta * trunc_f32(tb.ihm[c]), bc = trunc_f32(tb.ihc[c]), bp = beta * trunc_f32(tb.ihp[c]);
+#pragma unroll
+    for (int v = 0; v < M; ++v) {
+      const float um = nb(v, dir, 0), up = nb(v, dir, 1);
+      sl[v] = minmod3((un[v] - um) * bm, (up - um) * bc, (up - un[v]) * bp);
+    }
+  };
+  slopes(sx, p, 0);
+  slopes(sy, q, 1);
+  float Fm[M], Fp[M], ex[M], vn, c2;
+  vfma(xm, trunc_f32(tb.dm[p]), sx, un);
+  vfma(xp, trunc_f32(tb.dp[p]), sx, un);
+  vfma(ym, trunc_f32(tb.dm[q]), sy, un);
+  vfma(yp, trunc_f32(tb.dp[q]), sy, un);
+  flux_c2_f32<EQ>(xm, 0, Fm, &vn, &c2, ph);
+  flux_c2_f32<EQ>(xp, 0, Fp, &vn, &c2, ph);
+  vsub(ex, Fp, Fm);
+  vmul(ex, ex, hx);
+  flux_c2_f32<EQ>(ym, 1, Fm, &vn, &c2, ph);
+  flux_c2_f32<EQ>(yp, 1, Fp, &vn, &c2, ph);
+  vsub(Fp, Fp, Fm);
+  vfma(ex, hy, Fp);
+#pragma unroll
+  for (int v = 0; v < M; ++v) A[v] = fabsf(un[v]) + fabsf(sx[v]) + fabsf(sy[v]) + fabsf(ex[v]);
+  bool ok = clearly_admissible<EQ>(xm, A) && clearly_admissible<EQ>(xp, A) && clearly_admissible<EQ>(ym, A) &&
+            clearly_admissible<EQ>(yp, A);
+  vsub(xm, xm, ex);
+  vsub(xp, xp, ex);
+  vsub(ym, ym, ex);
+  vsub(yp, yp, ex);
+  return ok && clearly_admissible<EQ>(xm, A) && clearly_admissible<EQ>(xp, A) && clearly_admissible<EQ>(ym, A) &&
+         clearly_admissible<EQ>(yp, A);
+}
+
+// FP32 face data carry their density negated (their states are clearly
+// admissible); a widened FP32 number also has 29 zero low bits.
+__device__ __forceinline__ bool is_f32_face_data(double density) {
+  return __double2hiint(density) < 0 && (__double2loint(density) & 0x1fffffff) == 0;
+}
+
+// FP64 face data in the place of FP32 ones (hancock_states_f32): the evolved
+// boundary state and the limiter base of face node (side, j) of element e, from
+// the state in memory into the slots.  For the face kernel, where the screen of
+// the limiter leaves a face open; rare, so kept out of line.  Elements beside a
+// boundary always have FP64 data and are left as they are.
+template <int N, class EQ>
+__device__ __noinline__ void exact_face_data(const KParams<double>& P, const Tab<double>& tb, int e, int side, int j,
+                                             double dt) {
+  constexpr int n = N + 1, NP = n * n, M = EQ::M;
+  const Mesh& m = P.m;
+#pragma unroll
+  for (int f = 0; f < 4; ++f)
+    if (neighbour(m, e, f) < 0) return;
+  const double alpha = P.b.alpha[e];
+  const int dir = side >> 1;
+  double st[4][M];  // evolved states towards the face and inwards, of the boundary node and the next one
+  double ub[M];
+  for (int in = 0; in < 2; ++in) {
+    const int c = (side & 1) ? N - in : in;
+    const int p = dir == 0 ? c : j, q = dir == 0 ? j : c, k = p + n * q;
+    double un[M], xm[M], xp[M], ym[M], yp[M];
+#pragma unroll
+    for (int v = 0; v < M; ++v) un[v] = P.b.u[((size_t)v * m.ne + e) * NP + k];
+    auto nb = [&](int v, int d, int up) {
+      const int cc = d == 0 ? p : q, step = d == 0 ? 1 : n;
+      int ee = e, kk = k + (up ? step : -step);
+      if (cc == (up ? N : 0)) {
+        ee = neighbour(m, e, 2 * d + up);
+        kk = k + (up ? -N : N) * step;
+      }
+      return P.b.u[((size_t)v * m.ne + ee) * NP + kk];
+    };
+    const double hx = dt * (0.5 * tb.invw[p] * P.ph.invdx), hy = dt * (0.5 * tb.invw[q] * P.ph.invdy);
+    hancock_states<N, EQ>(m, P.ph, tb, un, alpha, p, q, hx, hy, nb, xm, xp, ym, yp);
+#pragma unroll
+    for (int v = 0; v < M; ++v) {
+      const double lo = dir == 0 ? xm[v] : ym[v], hi = dir == 0 ? xp[v] : yp[v];
+      st[2 * in][v] = (side & 1) ? hi : lo;
+      st[2 * in + 1][v] = (side & 1) ? lo : hi;
+      if (in == 0) ub[v] = un[v];
+    }
+  }
+  double f[M];  // twice the subcell flux between the two nodes
+  if (side & 1) rusanov_twice<EQ>(st[2], st[1], dir, f, P.ph);
+  else rusanov_twice<EQ>(st[1], st[2], dir, f, P.ph);
+  const double c = 0.5 * dt * ((side & 1) ? P.ph.cflim[side] : -P.ph.cflim[side]);
+#pragma unroll
+  for (int v = 0; v < M; ++v) {
+    P.b.slot[slot_index(1 + 2 * M + v, side, e, j, 4, m.ne, n)] = st[0][v];
+    P.b.slot[slot_index(1 + 3 * M + v, side, e, j, 4, m.ne, n)] = fma(c, f[v], ub[v]);
+  }
+}
+
 // Shared memory of the body beyond the five node arrays, in bytes.
 template <int N, class EQ>
 __host__ __device__ constexpr size_t local64_extra(int epb) {
   constexpr int n = N + 1, S = Tableau<N>::S;
   return (size_t)epb * sizeof(double) + (size_t)(4 * n * n) * sizeof(int2) + (size_t)(S * S + 4 * n) * sizeof(double) +
-         (size_t)epb * (4 + 2 * n * EQ::M) * sizeof(int);
+         (size_t)epb * (5 + 2 * n * EQ::M) * sizeof(int);
 }
 
 template <int N, class EQ, int T>
@@ -159,6 +358,7 @@ __device__ __forceinline__ void local_body_f64(const KParams<double>& P, const T
   int* sNbr = reinterpret_cast<int*>(sWy + n);                // [epb][4]
   int* sKx = sNbr + epb * 4;                                  // line keys [epb][n][M]
   int* sKy = sKx + epb * n * M;
+  int* sFull = sKy + epb * n * M;                             // [epb] low-order scheme in FP64
 
   double un[M];
 #pragma unroll
@@ -182,6 +382,26 @@ __device__ __forceinline__ void local_body_f64(const KParams<double>& P, const T
     }
     sAlpha[e2] = al;
     if (v2) P.b.alpha[eg] = al;
+    // An element needs its low-order scheme in FP64 when it is blended, when one
+    // of its faces is (a face neighbour is blended: alpha_raw > 0 in it or in a
+    // neighbour of it), or beside a boundary (those faces take the FP64 limiter
+    // as it stands).  Everywhere else that scheme feeds only the flux limiter's
+    // test, which FP32 answers (cr_screen.cuh; the face kernel forms the FP64
+    // data itself where it does not).
+    bool full = gt0(al);
+#pragma unroll
+    for (int f = 0; f < 4; ++f) {
+      if (nbs[f] < 0) full = true;
+      else if (!full && m.alpha_mode != 1 && (m.limiter & kLimBlend)) {
+        full = gt0(P.b.alpha_raw[nbs[f]]);
+#pragma unroll
+        for (int g = 0; g < 4; ++g) {
+          const int n2 = neighbour(m, nbs[f], g);
+          full = full || (n2 >= 0 && gt0(P.b.alpha_raw[n2]));
+        }
+      }
+    }
+    sFull[e2] = full;
   }
   for (int t = tid; t < n * n; t += T) {
     tDx[t] = P.ds.fDx[t];
@@ -422,100 +642,65 @@ __device__ __forceinline__ void local_body_f64(const KParams<double>& P, const T
 #pragma unroll
   for (int v = 0; v < M; ++v) LO[v] = 0.0;
   if (need_lo) {
-    double xm[M], xp[M], ym[M], yp[M];
-#pragma unroll
-    for (int v = 0; v < M; ++v) xm[v] = xp[v] = ym[v] = yp[v] = un[v];
-    if (m.limiter & kLimMH) {
-      const double beta = 2.0 - alpha;
-      double sx[M], sy[M];
-      // slopes along one direction: the neighbour nodes of the line, across a
-      // face the neighbour element's, at a boundary the side's ghost node
-      // (outflow: the own node; wall: its reflection; Dirichlet, inflow: given)
-      auto slopes = [&](double (&sl)[M], int c, int step, int side0, int far_lo, int far_hi, int mom) {
-        const int nbl = c == 0 ? sNbr[el * 4 + side0] : -1, nbr = c == N ? sNbr[el * 4 + side0 + 1] : -1;
-        const int sg = c == 0 ? side0 : side0 + 1, bc = m.bcs[sg];
-        double gv[M];
-#pragma unroll
-        for (int v = 0; v < M; ++v) gv[v] = un[v];
-        if (bc == kBcDirichlet || bc == kBcInflow) ghost_at<M>(m, sg, P.b.ctl->t, gv);
-        else if (bc == kBcWall && M > 1) gv[M > 1 ? mom : 0] = -un[M > 1 ? mom : 0];
-        const double bm = beta * tb.ihm[c], bc0 = tb.ihc[c], bp = beta * tb.ihp[c];
-        const float fm = trunc_f32(bm), fc = trunc_f32(bc0), fp = trunc_f32(bp);
-#pragma unroll
-        for (int v = 0; v < M; ++v) {
-          const double um = c > 0 ? s0[v * stride + tid - step]
-                                  : (nbl >= 0 ? P.b.u[((size_t)v * m.ne + nbl) * NP + far_lo] : gv[v]);
-          const double up = c < N ? s0[v * stride + tid + step]
-                                  : (nbr >= 0 ? P.b.u[((size_t)v * m.ne + nbr) * NP + far_hi] : gv[v]);
-          sl[v] = minmod_scaled(un[v] - um, up - um, up - un[v], bm, bc0, bp, fm, fc, fp);
-        }
-      };
-      slopes(sx, p, 1, 0, N + n * q, n * q, 1);
-      slopes(sy, q, n, 2, p + n * N, p, 2);
-      double fxm[M], fxp[M], fym[M], fyp[M], Fm[M], Fp[M], ex[M];
-      vfma(fxm, tb.dm[p], sx, un);
-      vfma(fxp, tb.dp[p], sx, un);
-      vfma(fym, tb.dm[q], sy, un);
-      vfma(fyp, tb.dp[q], sy, un);
-      EQ::flux(fxm, 0, Fm, ph);
-      EQ::flux(fxp, 0, Fp, ph);
-      vsub(ex, Fp, Fm);
-      vmul(ex, ex, sHx[p]);
-      EQ::flux(fym, 1, Fm, ph);
-      EQ::flux(fyp, 1, Fp, ph);
-      vsub(Fp, Fp, Fm);
-      vfma(ex, sHy[q], Fp);
-      bool ok = true;
-      if constexpr (EQ::K > 0) {
-        float uf[M], xf[M], yf[M], ef[M], A[M], st[M];
-        const float dmx = trunc_f32(tb.dm[p]), dpx = trunc_f32(tb.dp[p]);
-        const float dmy = trunc_f32(tb.dm[q]), dpy = trunc_f32(tb.dp[q]);
-#pragma unroll
-        for (int v = 0; v < M; ++v) {
-          uf[v] = trunc_f32(un[v]);
-          xf[v] = trunc_f32(sx[v]);
-          yf[v] = trunc_f32(sy[v]);
-          ef[v] = trunc_f32(ex[v]);
-          A[v] = fabsf(uf[v]) + fabsf(xf[v]) + fabsf(yf[v]) + fabsf(ef[v]);
-        }
-#pragma unroll
-        for (int c = 0; c < 8; ++c) {  // four face states, then evolved
-          const float d = (c & 3) == 0 ? dmx : (c & 3) == 1 ? dpx : (c & 3) == 2 ? dmy : dpy;
-#pragma unroll
-          for (int v = 0; v < M; ++v) {
-            st[v] = fmaf(d, (c & 2) ? yf[v] : xf[v], uf[v]);
-            if (c & 4) st[v] -= ef[v];
-          }
-          ok = ok && clearly_admissible<EQ>(st, A);
-        }
+    // neighbour nodes of the line: across a face the neighbour element's, at a
+    // boundary the side's ghost node (outflow: the own node; wall: its
+    // reflection; Dirichlet, inflow: given)
+    auto nb = [&](int v, int dir, int up) -> double {
+      const int c = dir == 0 ? p : q, step = dir == 0 ? 1 : n;
+      if (c != (up ? N : 0)) return s0[v * stride + tid + (up ? step : -step)];
+      const int side = 2 * dir + up, e2 = sNbr[el * 4 + side];
+      if (e2 >= 0) return P.b.u[((size_t)v * m.ne + e2) * NP + k + (up ? -N : N) * step];
+      const int bc = m.bcs[side];
+      if (bc == kBcDirichlet || bc == kBcInflow) {
+        double g[M];
+        ghost_at<M>(m, side, P.b.ctl->t, g);
+        return g[v];
       }
-      double exm[M], exp_[M], eym[M], eyp[M];
-      vsub(exm, fxm, ex);
-      vsub(exp_, fxp, ex);
-      vsub(eym, fym, ex);
-      vsub(eyp, fyp, ex);
-      if (!ok)
-        ok = EQ::admissible_fast(fxm, ph) && EQ::admissible_fast(fxp, ph) && EQ::admissible_fast(exm, ph) &&
-             EQ::admissible_fast(exp_, ph) && EQ::admissible_fast(fym, ph) && EQ::admissible_fast(fyp, ph) &&
-             EQ::admissible_fast(eym, ph) && EQ::admissible_fast(eyp, ph);
-      if (ok) {
+      return bc == kBcWall && v == 1 + dir ? -un[v] : un[v];
+    };
+    auto put_exact = [&]() {
+      double xm[M], xp[M], ym[M], yp[M];
+      hancock_states<N, EQ>(m, ph, tb, un, alpha, p, q, sHx[p], sHy[q], nb, xm, xp, ym, yp);
+      vst_sh<M, stride>(sA + tid, xm);
+      vst_sh<M, stride>(sB + tid, xp);
+      vst_sh<M, stride>(sC + tid, ym);
+      vst_sh<M, stride>(sD + tid, yp);
+    };
+    // FP32 states sit in the low words of the same slots
+    auto low = [&](double* base, int v) -> float& { return *reinterpret_cast<float*>(base + v * stride); };
+    Phys<float> phf;
+    phf.gamma = trunc_f32(ph.gamma);
+    phf.gm1 = trunc_f32(ph.gm1);
+    phf.ax = trunc_f32(ph.ax);
+    phf.ay = trunc_f32(ph.ay);
+    const bool full0 = sFull[el] != 0;
+    bool unclear = false;
+    if (full0) {
+      put_exact();
+    } else {
+      float uf[M], xm[M], xp[M], ym[M], yp[M];
 #pragma unroll
-        for (int v = 0; v < M; ++v) {
-          xm[v] = exm[v];
-          xp[v] = exp_[v];
-          ym[v] = eym[v];
-          yp[v] = eyp[v];
-        }
+      for (int v = 0; v < M; ++v) uf[v] = trunc_f32(un[v]);
+      auto nbf = [&](int v, int dir, int up) { return trunc_f32(nb(v, dir, up)); };
+      unclear = !hancock_states_f32<N, EQ>(m, phf, tb, uf, trunc_f32(alpha), p, q, trunc_f32(sHx[p]), trunc_f32(sHy[q]),
+                                           nbf, xm, xp, ym, yp);
+#pragma unroll
+      for (int v = 0; v < M; ++v) {
+        low(sA + tid, v) = xm[v];
+        low(sB + tid, v) = xp[v];
+        low(sC + tid, v) = ym[v];
+        low(sD + tid, v) = yp[v];
       }
+      if (unclear) sFull[el] = 1;  // the whole element goes to FP64
     }
-    vst_sh<M, stride>(sA + tid, xm);
-    vst_sh<M, stride>(sB + tid, xp);
-    vst_sh<M, stride>(sC + tid, ym);
-    vst_sh<M, stride>(sD + tid, yp);
-    __syncthreads();
+    if (__syncthreads_or(unclear)) {
+      if (!full0 && sFull[el]) put_exact();
+      __syncthreads();
+    }
     // subcell fluxes (twice their value), numbered across the block: element r /
     // NSF, its N n x-subfaces, then its n N y-subfaces; the flux right of (above)
-    // node (p2, q2) overwrites that node's x+ (y+) state, which no other reads
+    // node (p2, q2) overwrites that node's x+ (y+) state, which no other reads.
+    // FP32 elements need only those next to the element faces.
     constexpr int NSX = N * n, NSF = 2 * N * n;
     for (int gs = tid; gs < epr * NSF; gs += T) {
       const int el2 = gs / NSF, r = gs - el2 * NSF;
@@ -524,16 +709,31 @@ __device__ __forceinline__ void local_body_f64(const KParams<double>& P, const T
       const int p2 = isx ? rr % N : rr % n, q2 = isx ? rr / N : rr / n;
       const int node = el2 * NP + p2 + n * q2;
       double* sL = (isx ? sB : sD) + node;
-      const double* sR = (isx ? sA : sC) + node + (isx ? 1 : n);
-      double uL[M], uR[M], fr[M];
-      vld_sh<M, stride>(uL, sL);
-      vld_sh<M, stride>(uR, sR);
-      rusanov_twice<EQ>(uL, uR, isx ? 0 : 1, fr, ph);
-      vst_sh<M, stride>(sL, fr);
+      double* sR = (isx ? sA : sC) + node + (isx ? 1 : n);
+      if (sFull[el2]) {
+        double uL[M], uR[M], fr[M];
+        vld_sh<M, stride>(uL, sL);
+        vld_sh<M, stride>(uR, sR);
+        rusanov_twice<EQ>(uL, uR, isx ? 0 : 1, fr, ph);
+        vst_sh<M, stride>(sL, fr);
+      } else if (const int c = isx ? p2 : q2; c == 0 || c == N - 1) {
+        float uL[M], uR[M], fL[M], fR[M], vL, vR, cL, cR;
+#pragma unroll
+        for (int v = 0; v < M; ++v) {
+          uL[v] = low(sL, v);
+          uR[v] = low(sR, v);
+        }
+        flux_c2_f32<EQ>(uL, isx ? 0 : 1, fL, &vL, &cL, phf);
+        flux_c2_f32<EQ>(uR, isx ? 0 : 1, fR, &vR, &cR, phf);
+        const float lam = fmaxf(fabsf(vL) + sqrt_f32(cL), fabsf(vR) + sqrt_f32(cR));
+#pragma unroll
+        for (int v = 0; v < M; ++v) low(sL, v) = fL[v] + fR[v] - lam * (uR[v] - uL[v]);
+      }
     }
     __syncthreads();
-    // low-order residual of the interior subfaces (eq. (low.order.update))
-    {
+    // low-order residual of the interior subfaces (eq. (low.order.update)); 0
+    // times alpha where the element is not blended
+    if (gt0(a)) {
       double fr[M], fl[M];
 #pragma unroll
       for (int v = 0; v < M; ++v) fr[v] = fl[v] = 0.0;
@@ -559,14 +759,25 @@ __device__ __forceinline__ void local_body_f64(const KParams<double>& P, const T
         const int side = fs.side, j = fs.j, base = fs.el * NP;
         const int nb_node = base + (side == 0 ? n * j : side == 1 ? N + n * j : side == 2 ? j : j + n * N);
         const int adj_node = nb_node - (side == 1 ? 1 : side == 3 ? n : 0);
-        const double* ust = side == 0 ? sA : side == 1 ? sB : side == 2 ? sC : sD;
-        const double* adj = side < 2 ? sB : sD;
+        double* ust = (side == 0 ? sA : side == 1 ? sB : side == 2 ? sC : sD) + nb_node;
+        double* adj = (side < 2 ? sB : sD) + adj_node;
         const double c = hdt * ((side & 1) ? ph.cflim[side] : -ph.cflim[side]);
-        double us[M], ub[M], fa[M];
-        vld_sh<M, stride>(us, ust + nb_node);
-        vld_sh<M, stride>(ub, s0 + nb_node);
-        vld_sh<M, stride>(fa, adj + adj_node);
-        vfma(ub, c, fa);
+        double us[M], ub[M];
+        if (sFull[fs.el]) {
+          double fa[M];
+          vld_sh<M, stride>(us, ust);
+          vld_sh<M, stride>(ub, s0 + nb_node);
+          vld_sh<M, stride>(fa, adj);
+          vfma(ub, c, fa);
+        } else {
+          const float cf = trunc_f32(c);
+#pragma unroll
+          for (int v = 0; v < M; ++v) {
+            us[v] = widen_f32(low(ust, v));
+            ub[v] = widen_f32(fmaf(cf, low(adj, v), trunc_f32(s0[v * stride + nb_node])));
+          }
+          if (EQ::K > 0) us[0] = -us[0];  // a negative density marks FP32 face data
+        }
 #pragma unroll
         for (int v = 0; v < M; ++v) {
           P.b.slot[slot_index(1 + 2 * M + v, side, eg, j, 4, m.ne, n)] = us[v];

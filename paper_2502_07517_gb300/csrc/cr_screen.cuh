@@ -28,6 +28,19 @@ __device__ __forceinline__ float trunc_f32(double x) {
 }
 __device__ __forceinline__ float trunc_f32(float x) { return x; }
 
+// x as FP64 from the bit pattern (below FP32's normal range: a signed 0).
+__device__ __forceinline__ double widen_f32(float x) {
+  const unsigned b = __float_as_uint(x), m = b & 0x7fffffffu;
+  const unsigned hi = (m >> 3) + (896u << 20);
+  return m < 0x00800000u ? __hiloint2double(int(b & 0x80000000u), 0)
+                         : __hiloint2double(int(hi | (b & 0x80000000u)), int(b << 29));
+}
+__device__ __forceinline__ float rcp_f32(float x) {
+  float r;
+  asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(x));
+  return r;
+}
+
 __device__ __forceinline__ bool finite_bits(double x) { return (__double2hiint(x) & 0x7ff00000) != 0x7ff00000; }
 __device__ __forceinline__ bool finite_bits(float x) { return isfinite(x); }
 
@@ -35,6 +48,29 @@ __device__ __forceinline__ float sqrt_f32(float x) {
   float r;
   asm("sqrt.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(fmaxf(x, 0.0f)));
   return r;
+}
+
+// Flux in direction dir, normal velocity and squared sound speed in FP32 (see
+// flux_c2; equations without a sound speed: vn is the wave speed).
+template <class EQ>
+__device__ __forceinline__ void flux_c2_f32(const float* u, int dir, float* f, float* vn, float* c2,
+                                            const Phys<float>& ph) {
+  if constexpr (IsEuler<EQ>::value) {
+    const float rinv = rcp_f32(u[0]);
+    float p;
+    EQ::flux_r(u, dir, rinv, f, &p, ph);
+    *vn = u[1 + dir] * rinv;
+    *c2 = ph.gamma * p * rinv;
+  } else if constexpr (EQ::M == 6) {
+    const float rinv = rcp_f32(u[0]);
+    EQ::flux_r(u, dir, rinv, f, ph);
+    *vn = u[1 + dir] * rinv;
+    *c2 = 3.0f * (2.0f * u[3 + 2 * dir] - u[1 + dir] * *vn) * rinv;
+  } else {
+    EQ::flux(u, dir, f, ph);
+    *vn = EQ::speed(u, dir, ph);
+    *c2 = 0.0f;
+  }
 }
 
 // Constraint k of the state s in FP32 and the bound of its error, A[v] bounding
