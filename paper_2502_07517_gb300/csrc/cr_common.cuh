@@ -162,14 +162,17 @@ struct DiffScaled {
 };
 
 // FP64: also as fixed-point coefficients (cr_fixed.cuh) for the integer-pipe
-// contractions, with the exponent offsets (fix_exp) of the x and y matrices.
+// contractions, with the exponent offsets (fix_exp) of the x and y matrices: oD
+// of Dx and Dy; oDt is what a sum with Dtx, Dty taken times b_i (fix_scaled) adds
+// to them, the same in both directions; and the trace coefficients l(0), l(1).
 template <>
 struct DiffScaled<double> {
   double Dx[kMaxNodes1 * kMaxNodes1], Dy[kMaxNodes1 * kMaxNodes1];
   double Dtx[kMaxNodes1 * kMaxNodes1], Dty[kMaxNodes1 * kMaxNodes1];
   int2 fDx[kMaxNodes1 * kMaxNodes1], fDy[kMaxNodes1 * kMaxNodes1];
   int2 fDtx[kMaxNodes1 * kMaxNodes1], fDty[kMaxNodes1 * kMaxNodes1];
-  int oD[2], oDt[2];
+  int2 fL[2 * kMaxNodes1];
+  int oD[2], oDt, oL;
 };
 
 template <typename real>
@@ -203,15 +206,26 @@ inline void fill_scaled(const double* D, const double* w, const double* l0, cons
       ds->Dty[i * n + j] = real(dt * invdy);
     }
   if constexpr (sizeof(real) == 8) {
-    auto fixed = [&](const double* A, int2* F) {
-      const int scale = fix_scale(A, n * n);
+    auto fixed = [&](const double* A, int scale, int2* F) {
       for (int i = 0; i < kMaxNodes1 * kMaxNodes1; ++i) F[i] = i < n * n ? fix_coef(A[i], scale) : make_int2(0, 0);
-      return fix_exp(scale);
     };
-    ds->oD[0] = fixed(ds->Dx, ds->fDx);
-    ds->oD[1] = fixed(ds->Dy, ds->fDy);
-    ds->oDt[0] = fixed(ds->Dtx, ds->fDtx);
-    ds->oDt[1] = fixed(ds->Dty, ds->fDty);
+    const int sx = fix_scale(ds->Dx, n * n), sy = fix_scale(ds->Dy, n * n);
+    const int tx = fix_scale(ds->Dtx, n * n) - sx, ty = fix_scale(ds->Dty, n * n) - sy, t = tx < ty ? tx : ty;
+    fixed(ds->Dx, sx, ds->fDx);
+    fixed(ds->Dy, sy, ds->fDy);
+    fixed(ds->Dtx, sx + t, ds->fDtx);
+    fixed(ds->Dty, sy + t, ds->fDty);
+    ds->oD[0] = fix_exp(sx);
+    ds->oD[1] = fix_exp(sy);
+    ds->oDt = 1 - t;
+    double l[2 * kMaxNodes1];
+    for (int i = 0; i < n; ++i) {
+      l[i] = l0[i];
+      l[n + i] = l1[i];
+    }
+    const int scale = fix_scale(l, 2 * n);
+    for (int i = 0; i < 2 * kMaxNodes1; ++i) ds->fL[i] = i < 2 * n ? fix_coef(l[i], scale) : make_int2(0, 0);
+    ds->oL = fix_exp(scale);
   }
 }
 

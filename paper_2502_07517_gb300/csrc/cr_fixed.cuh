@@ -3,14 +3,15 @@
 // GB300 has two FP64 FMA lanes per SM (16 cycles per warp instruction) and
 // half-rate 32 x 32 + 64 bit integer multiply-adds (0.5 cycles), so a short dot
 // product with constant coefficients is several times cheaper in fixed point:
-// the values of a line share one exponent E (the largest biased FP64 exponent
-// among them) and become 59-bit integers, the coefficients 58-bit integers
-// with a common scale, both as two signed limbs of about 30 bits; three integer
-// multiply-adds per term (the product of the low limbs is dropped) and one
-// rounding at the end.  Per term, truncating the value costs at most 2^-57 of
-// max|a| max|x|, rounding the coefficient 2^-58 and the dropped product 2^-57;
-// an FMA chain rounds every partial sum to 2^-53.  Against exact rational
-// arithmetic the mean error is half of the FMA chain's
+// the values that enter a sum share an exponent E and become 59-bit integers,
+// the coefficients of a matrix 58-bit integers with a common scale, both as two
+// signed limbs of about 30 bits; three integer multiply-adds per term (the
+// product of the low limbs is dropped) and one rounding at the end.  A sum over
+// two lines with matrices A and B takes the exponents so that |A| |x| and |B| |y|
+// have one scale, and needs no alignment.  Per term, truncating the value costs
+// at most 2^-56 of the largest max|a| max|x|, rounding the coefficient 2^-57 and
+// the dropped product 2^-56; an FMA chain rounds every partial sum to 2^-53.
+// Against exact rational arithmetic the mean error is half of the FMA chain's
 // (tests/test_fixed_point.py).
 //
 // Conversions between FP64 and integers or FP32 run on the same FP64 pipe (18
@@ -53,24 +54,19 @@ CRK_HD double from_bits(uint64_t b) {
 #endif
 }
 
-// Magnitude key of a value: its high word without the sign; keys order as the
-// magnitudes, and key >> 20 is the biased exponent (0x7ff: not finite).
-CRK_HD int mag_key(double x) { return hi_word(x) & 0x7fffffff; }
+// Biased exponent (0x7ff: not finite).
+CRK_HD int exp_of(double x) { return (hi_word(x) & 0x7fffffff) >> 20; }
 
-// Line exponents are kept at or above kMinLineExp, which keeps every exponent
-// below in the normal range; lines with larger magnitudes than 2^(kMaxLineExp -
-// 1022) are given up as not finite (NaN results).
+// Shared exponents are kept at or above kMinLineExp (a zero then truncates to 0
+// in spite of its implicit bit); values with larger ones than kMaxLineExp are
+// given up as not finite (NaN results).
 constexpr int kMinLineExp = 64, kMaxLineExp = 2000;
-CRK_HD int line_exp(int key) {
-  const int e = key >> 20;
-  return e < kMinLineExp ? kMinLineExp : e;
-}
 
 constexpr int kLimb = 29;  // bits of a low limb
 
 // x as a fixed-point number (hi 2^29 + lo) 2^(E - 1080), truncated towards
-// zero; wants an exponent of x of at most E + 1 (one bit of headroom, so that a
-// line keeps its exponent when its values grow less than twofold).
+// zero; wants an exponent of x of at most E + 1 (one bit of headroom, so that E stays
+// when the values grow less than twofold).
 CRK_HD int2 to_fixed(double x, int E) {
   const int h = hi_word(x);
   const uint32_t l = lo_word(x);
@@ -117,20 +113,27 @@ CRK_HD double from_fixed(long long r, int e) {
   return (f < 0 || a == 0) ? 0.0 : from_bits(b | (s << 63));
 }
 
-// Sum of two dot products with their own scales: r1 2^(e1 - 1023) + r2 2^(e2 -
-// 1023) (the smaller scale is shifted down).
-CRK_HD double from_fixed2(long long r1, int e1, long long r2, int e2) {
-  const int d = e1 - e2;
-  const int d1 = d < 0 ? (d < -63 ? 63 : -d) : 0, d2 = d > 0 ? (d > 63 ? 63 : d) : 0;
-  return from_fixed((r1 >> d1) + (r2 >> d2), d > 0 ? e1 : e2);
-}
-
 // Coefficients with |a| 2^scale <= 2^58 as a 30-bit and a 29-bit signed limb.
 inline int2 fix_coef(double a, int scale) {
   const long long v = llrint(ldexp(a, scale));
   const long long lo = ((v + (1ll << (kLimb - 1))) & ((1ll << kLimb) - 1)) - (1ll << (kLimb - 1));
   return make_int2(int((v - lo) >> kLimb), int(lo));
 }
+// A coefficient times b in [0, 1], with a scale one less (truncated towards
+// zero): several such sums, sum b <= 1, add up without overflow.
+CRK_HD int2 fix_scaled(int2 a, double b) {
+  const long long v = ((long long)a.x << kLimb) + a.y;
+  const uint64_t m = uint64_t(v < 0 ? -v : v), f = uint64_t(b * 9223372036854775808.0);  // b 2^63
+#ifdef __CUDA_ARCH__
+  const long long t = (long long)__umul64hi(m, f);
+#else
+  const long long t = (long long)((unsigned __int128)m * f >> 64);
+#endif
+  const long long w = v < 0 ? -t : t;
+  const long long lo = ((w + (1ll << (kLimb - 1))) & ((1ll << kLimb) - 1)) - (1ll << (kLimb - 1));
+  return make_int2(int((w - lo) >> kLimb), int(lo));
+}
+
 // The scale for coefficients a[0..n): the largest is at least 2^57.
 inline int fix_scale(const double* a, int n) {
   double m = 0.0;

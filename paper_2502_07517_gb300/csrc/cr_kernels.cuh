@@ -820,8 +820,8 @@ __device__ __forceinline__ void local_phase(const KParams<real>& P, const Tab<re
 // Resident blocks per SM the step kernels ask for (measured on GB300,
 // 2D Euler N = 4, 512x512): FP32_BULK blocks are latency bound and gain from
 // four 256-thread blocks per SM (64 registers; k_local 1.39 -> 1.05 ms,
-// k_update 0.91 -> 0.60 ms); the FP64 k_local is bound by the FP64 pipe and
-// gains 3% from two blocks (128 registers instead of 130); the FP64 k_update
+// k_update 0.91 -> 0.60 ms); the FP64 k_local takes two (in two dimensions
+// LocalBlocks); the FP64 k_update
 // is bound by its barriers and gains from more resident blocks: 2.15 ms at
 // one (106 registers), 1.91 at three (85), 1.75 at four (64).
 template <bool MIXED> struct MinBlocks {
@@ -838,8 +838,18 @@ template <int NP, int THREADS = 256> struct BlockShape {
 };
 template <int NP, bool MIXED> using UpdateShape = BlockShape<NP, MIXED ? 128 : 256>;
 
+// Blocks of the element kernel.  FP64 in two dimensions (cr_local64.cuh): three
+// resident blocks (80 registers) so that one block's integer phases overlap
+// another's FP64 phases: 4.91 ms at two, 4.51 at three, although the compiler
+// spills 0.7 kB per thread there (2D Euler N = 4, 512 x 512); blocks of 128
+// threads 4.84 ms (per-block tables and neighbours), of 352 4.44.  The ten-moment
+// equations (six variables) keep two.
+template <int DIM, class EQ, bool MIXED> struct LocalBlocks {
+  static constexpr int value = DIM == 2 && !MIXED && EQ::M <= 4 ? 3 : MinBlocks<MIXED>::local;
+};
+
 template <int DIM, int N, class EQ, typename real, bool MIXED>
-__global__ void __launch_bounds__(256, MinBlocks<MIXED>::local) k_local(const __grid_constant__ KParams<real> P) {
+__global__ void __launch_bounds__(256, LocalBlocks<DIM, EQ, MIXED>::value) k_local(const __grid_constant__ KParams<real> P) {
   local_phase<DIM, N, EQ, real, MIXED, BlockShape<DIM == 2 ? (N + 1) * (N + 1) : N + 1>::T>(P, P.tb, blockIdx.x);
 }
 

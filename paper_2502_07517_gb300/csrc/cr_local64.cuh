@@ -7,11 +7,12 @@
 // at 10% of the issue slots (2D Euler N = 4, 512 x 512: 12.57 ms, 1,031 FP64
 // instructions per solution point).  So every FP64 instruction that integer or
 // FP32 work can replace without touching the result is worth 30 of those:
-//   - the D contractions (a third of the FP64 work) run in fixed point on the
-//     integer pipe (cr_fixed.cuh);
+//   - the D contractions and the face traces (40% of the FP64 work) run in
+//     fixed point on the integer pipe (cr_fixed.cuh); the FR volume term takes
+//     each stage's fluxes with b_i in its matrices and accumulates in fixed
+//     point, so the time-averaged fluxes are never formed;
 //   - the trace of the time-averaged solution is the average of the stage
-//     traces, which the face-node threads form anyway, and the wave speed of
-//     the u^n trace shares the first stage's flux;
+//     traces, and the wave speed of the u^n trace shares the first stage's flux;
 //   - which of the three slopes minmod takes, which of two wave speeds is the
 //     larger and whether the MUSCL-Hancock states are admissible are decided in
 //     FP32 where the answer is clear by a margin above the FP32 rounding, and
@@ -26,10 +27,13 @@
 //     and the face kernel forms the FP64 data itself where the inequality is not
 //     clear (exact_face_data).  The update is the same: alpha = 0 leaves the
 //     high-order part alone, and theta is decided as in FP64.
-// Measured (k_local, the same workload): the contractions and the first two
-// groups of decisions 12.57 -> 8.42 ms (612 FP64 instructions per point), the
-// low-order scheme in FP32 -> 5.60 ms; ten-moment N = 3 at 256 x 256 2.61 -> 2.03
-// -> 1.56 ms.
+// Measured (k_local, the same workload): the contractions and the first decisions
+// 12.57 -> 8.42 ms (612 FP64 instructions per point), the low-order scheme in FP32
+// -> 5.60 ms, traces and volume term on the integer pipe as well (251 FP64
+// instructions, 56% of the pipe, 28% of the issue slots: latency bound) -> 5.03
+// ms, the stage residuals in shared memory and a third resident block -> 4.51 ms,
+// neighbour data and tables loaded by all threads at once -> 4.35 ms; ten-moment
+// N = 3 at 256 x 256 2.61 -> 1.42 ms.
 #pragma once
 #include "cr_common.cuh"
 #include "cr_fixed.cuh"
@@ -199,6 +203,48 @@ __device__ __forceinline__ void hancock_states(const Mesh& m, const Phys<double>
   }
 }
 
+// Value of variable v at the neighbour of node k = (p, q) of a block's element
+// along direction dir: from the block's nodes (u points at this node's slot),
+// across a face from the neighbour element (nbr: the element's face neighbours),
+// at a boundary the side's ghost node (outflow: the own node; wall: its
+// reflection; Dirichlet, inflow: given).
+template <int N, class EQ, int STRIDE>
+__device__ __forceinline__ double line_neighbour(const KParams<double>& P, const double* u, const int* nbr, int k, int p,
+                                                 int q, int v, int dir, int up) {
+  constexpr int n = N + 1, NP = n * n, M = EQ::M;
+  const Mesh& m = P.m;
+  const int c = dir == 0 ? p : q, step = dir == 0 ? 1 : n;
+  if (c != (up ? N : 0)) return u[v * STRIDE + (up ? step : -step)];
+  const int side = 2 * dir + up, e2 = nbr[side];
+  if (e2 >= 0) return P.b.u[((size_t)v * m.ne + e2) * NP + k + (up ? -N : N) * step];
+  const int bc = m.bcs[side];
+  if (bc == kBcDirichlet || bc == kBcInflow) {
+    double g[M];
+    ghost_at<M>(m, side, P.b.ctl->t, g);
+    return g[v];
+  }
+  const double x = u[v * STRIDE];
+  return bc == kBcWall && v == 1 + dir ? -x : x;
+}
+
+// hancock_states of a block's node into the four node arrays at st (M STRIDE
+// apart).  Out of line: only blended elements, their neighbours and those beside
+// a boundary come here, and the element kernel keeps its registers.
+template <int N, class EQ, int STRIDE>
+__device__ __noinline__ void put_hancock_states(const KParams<double>& P, const Tab<double>& tb, const double* u,
+                                                const int* nbr, int k, double alpha, double hx, double hy, double* st) {
+  constexpr int M = EQ::M;
+  const int p = k % (N + 1), q = k / (N + 1);
+  double un[M], xm[M], xp[M], ym[M], yp[M];
+  vld_sh<M, STRIDE>(un, u);
+  auto nb = [&](int v, int dir, int up) { return line_neighbour<N, EQ, STRIDE>(P, u, nbr, k, p, q, v, dir, up); };
+  hancock_states<N, EQ>(P.m, P.ph, tb, un, alpha, p, q, hx, hy, nb, xm, xp, ym, yp);
+  vst_sh<M, STRIDE>(st, xm);
+  vst_sh<M, STRIDE>(st + M * STRIDE, xp);
+  vst_sh<M, STRIDE>(st + 2 * M * STRIDE, ym);
+  vst_sh<M, STRIDE>(st + 3 * M * STRIDE, yp);
+}
+
 // The same in FP32, for elements whose low-order scheme only feeds the screen of
 // the flux limiter (see the body).  Returns false where admissibility is not
 // clear in FP32 (the FP64 form then decides).
@@ -311,8 +357,10 @@ __device__ __noinline__ void exact_face_data(const KParams<double>& P, const Tab
 template <int N, class EQ>
 __host__ __device__ constexpr size_t local64_extra(int epb) {
   constexpr int n = N + 1, S = Tableau<N>::S;
-  return (size_t)epb * sizeof(double) + (size_t)(4 * n * n) * sizeof(int2) + (size_t)(S * S + 4 * n) * sizeof(double) +
-         (size_t)epb * (5 + 2 * n * EQ::M) * sizeof(int);
+  constexpr size_t src = (EQ::M == 6 || HasGravity<EQ>::value ? EQ::M * n * n : 0)  // the averaged source,
+                         + (N == 4 ? 3 * EQ::M * n * n : 0);                      // stage residuals
+  return (size_t)epb * (1 + src) * sizeof(double) + (size_t)(2 * (1 + S) * n * n + 2 * n) * sizeof(int2) +
+         (size_t)(S * S + 4 * n) * sizeof(double) + (size_t)epb * (5 + 2 * EQ::M) * sizeof(int);
 }
 
 template <int N, class EQ, int T>
@@ -333,9 +381,8 @@ __device__ __forceinline__ void local_body_f64(const KParams<double>& P, const T
   const double dt = P.b.ctl->dt_step;
   if (!gt0(dt)) return;
 
-  // node arrays [M][epb][NP]: u^n; the stage state, then the MUSCL-Hancock
-  // states; the stage fluxes in fixed point; the time-averaged solution (for a
-  // source), then the y+ states
+  // node arrays [M][epb][NP]: u^n; in fixed point the stage state and fluxes,
+  // then the MUSCL-Hancock states; for a source its time average
   extern __shared__ __align__(16) unsigned char smem_raw[];
   constexpr int stride = epb * NP, arr = M * stride;
   double* s0 = reinterpret_cast<double*>(smem_raw);
@@ -343,74 +390,80 @@ __device__ __forceinline__ void local_body_f64(const KParams<double>& P, const T
   double* sB = sA + arr;
   double* sC = sB + arr;
   double* sD = sC + arr;
+  constexpr bool SRC = EQ::M == 6 || HasGravity<EQ>::value;
+  constexpr bool kShL = N == 4;  // four residuals are live at a time
+  double* sS = sD + arr;
+  double* sL = sS + (SRC ? arr : 0);  // stage residuals 0..2 (kept in shared memory at N = 4; 3: sD)
+  int2* xA = reinterpret_cast<int2*>(sA);
   int2* xB = reinterpret_cast<int2*>(sB);
   int2* xC = reinterpret_cast<int2*>(sC);
-  double* sAlpha = sD + arr;                                  // [epb]
+  double* sAlpha = sL + (kShL ? 3 * arr : 0);                 // [epb]
   int2* tDx = reinterpret_cast<int2*>(sAlpha + epb);          // [n][n] each
   int2* tDy = tDx + n * n;
-  int2* tDtx = tDy + n * n;
-  int2* tDty = tDtx + n * n;
-  double* sAdt = reinterpret_cast<double*>(tDty + n * n);     // dt a_ij
+  int2* tB = tDy + n * n;                                     // b_i times the FR matrices [S][2][n][n]
+  int2* tL = tB + 2 * S * n * n;                              // l(0), l(1) [2][n]
+  double* sAdt = reinterpret_cast<double*>(tL + 2 * n);       // dt a_ij
   double* sHx = sAdt + S * S;                                 // dt / (2 w_p dx), dt / (2 w_q dy)
   double* sHy = sHx + n;
   double* sWx = sHy + n;                                      // 1 / (2 w_p dx), 1 / (2 w_q dy)
   double* sWy = sWx + n;
   int* sNbr = reinterpret_cast<int*>(sWy + n);                // [epb][4]
-  int* sKx = sNbr + epb * 4;                                  // line keys [epb][n][M]
-  int* sKy = sKx + epb * n * M;
-  int* sFull = sKy + epb * n * M;                             // [epb] low-order scheme in FP64
+  int* sKey = sNbr + epb * 4;                                 // exponents [fluxes, state][epb][M]
+  int* sFull = sKey + 2 * epb * M;                            // [epb] low-order scheme in FP64
 
   double un[M];
 #pragma unroll
   for (int v = 0; v < M; ++v) un[v] = P.b.u[((size_t)v * m.ne + ee) * NP + k];
-  for (int t = tid; t < 2 * epb * n * M; t += T) sKx[t] = 0;
-  for (int e2 = tid; e2 < epb; e2 += T) {
-    const int eg0 = blk * epr + e2;
-    const bool v2 = e2 < epr && eg0 < m.ne;
-    const int eg = v2 ? eg0 : m.ne - 1;
-    int nbs[4];
-#pragma unroll
-    for (int f = 0; f < 4; ++f) sNbr[e2 * 4 + f] = nbs[f] = neighbour(m, eg, f);
-    double al = 0.0;
-    if (m.alpha_mode == 1) {
-      al = m.alpha_fixed;
-    } else if (m.limiter & kLimBlend) {
-      al = P.b.alpha_raw[eg];
-#pragma unroll
-      for (int f = 0; f < 4; ++f)
-        if (nbs[f] >= 0) al = fmax(al, 0.5 * P.b.alpha_raw[nbs[f]]);
+  for (int t = tid; t < 2 * epb * M; t += T) sKey[t] = 0;
+  for (int t = tid; t < epb; t += T) {
+    sFull[t] = 0;
+    sAlpha[t] = m.alpha_mode == 1 ? m.alpha_fixed : 0.0;
+  }
+  __syncthreads();
+  // alpha_e, smoothed with the face neighbours, and which elements need their
+  // low-order scheme in FP64: the blended ones, those with a blended face (a face
+  // neighbour is blended: alpha_raw > 0 in it or in a neighbour of it) and those
+  // beside a boundary (those faces take the FP64 limiter as it stands).
+  // Everywhere else that scheme feeds only the flux limiter's test, which FP32
+  // answers (cr_screen.cuh; the face kernel forms the FP64 data itself where it
+  // does not).  One thread per element and cell of the 13 within two steps, so
+  // that their loads go out together.
+  for (int t = T - 1 - tid; t < epb * 13; t += T) {
+    const int e2 = t / 13, c = t - e2 * 13;
+    const int eg0 = blk * epr + e2, eg = e2 < epr && eg0 < m.ne ? eg0 : m.ne - 1;
+    // cell offsets: the face neighbours (x-, x+, y-, y+), the element, the second ring
+    // plus 2, three bits each
+    const int iy = eg / m.nx;
+    int cx = eg - iy * m.nx + int(0x32ca502499ull >> (3 * c) & 7) - 2, cy = iy + int(0x364c092652ull >> (3 * c) & 7) - 2;
+    bool in = true;
+    if (m.bcx == 0) cx = (cx % m.nx + m.nx) % m.nx;
+    else in = cx >= 0 && cx < m.nx;
+    if (m.bcy == 0) cy = (cy % m.ny + m.ny) % m.ny;
+    else in = in && cy >= 0 && cy < m.ny;
+    const int ec = in ? cx + m.nx * cy : -1;
+    if (c < 4) {
+      sNbr[e2 * 4 + c] = ec;
+      if (ec < 0) sFull[e2] = 1;
     }
-    sAlpha[e2] = al;
-    if (v2) P.b.alpha[eg] = al;
-    // An element needs its low-order scheme in FP64 when it is blended, when one
-    // of its faces is (a face neighbour is blended: alpha_raw > 0 in it or in a
-    // neighbour of it), or beside a boundary (those faces take the FP64 limiter
-    // as it stands).  Everywhere else that scheme feeds only the flux limiter's
-    // test, which FP32 answers (cr_screen.cuh; the face kernel forms the FP64
-    // data itself where it does not).
-    bool full = gt0(al);
-#pragma unroll
-    for (int f = 0; f < 4; ++f) {
-      if (nbs[f] < 0) full = true;
-      else if (!full && m.alpha_mode != 1 && (m.limiter & kLimBlend)) {
-        full = gt0(P.b.alpha_raw[nbs[f]]);
-#pragma unroll
-        for (int g = 0; g < 4; ++g) {
-          const int n2 = neighbour(m, nbs[f], g);
-          full = full || (n2 >= 0 && gt0(P.b.alpha_raw[n2]));
-        }
+    if (m.alpha_mode != 1 && (m.limiter & kLimBlend) && ec >= 0) {
+      const double raw = P.b.alpha_raw[ec];
+      if (gt0(raw)) {
+        sFull[e2] = 1;
+        if (c <= 4)  // bit patterns of positive numbers order as the values
+          atomicMax(reinterpret_cast<unsigned long long*>(sAlpha + e2),
+                    (unsigned long long)__double_as_longlong(c == 4 ? raw : 0.5 * raw));
       }
     }
-    sFull[e2] = full;
   }
-  for (int t = tid; t < n * n; t += T) {
-    tDx[t] = P.ds.fDx[t];
-    tDy[t] = P.ds.fDy[t];
-    tDtx[t] = P.ds.fDtx[t];
-    tDty[t] = P.ds.fDty[t];
+  // tables: D / dx, D / dy, b_i times the FR matrices, the trace coefficients
+  for (int t = tid; t < 2 * (1 + S) * n * n; t += T) {
+    const int i = t / (n * n), r = t - i * (n * n), st = i / 2 - 1;
+    if (i < 2) tDx[t] = (i == 0 ? P.ds.fDx : P.ds.fDy)[r];
+    else tDx[t] = fix_scaled((i & 1 ? P.ds.fDty : P.ds.fDtx)[r], TB::b(st));
   }
-  // (per-block factors by threads of the last warps: the first ones smooth alpha)
-  for (int t = T - 1 - tid; t < S * S + 2 * n; t += T) {
+  for (int t = tid; t < 2 * n; t += T) tL[t] = P.ds.fL[t];
+  // factors of the step and the node row
+  for (int t = tid; t < S * S + 2 * n; t += T) {
     if (t < S * S) {
       sAdt[t] = dt * TB::a(t / S, t % S);
     } else {
@@ -422,12 +475,16 @@ __device__ __forceinline__ void local_body_f64(const KParams<double>& P, const T
   }
   vst_sh<M, stride>(s0 + tid, un);
   __syncthreads();
+  if (m.alpha_mode == 1 && gt0(m.alpha_fixed)) {
+    for (int t = tid; t < epb; t += T) sFull[t] = 1;  // (read after the stages' barriers)
+  }
+  for (int t = tid; t < epr; t += T)
+    if (blk * epr + t < m.ne) P.b.alpha[blk * epr + t] = sAlpha[t];
   const double alpha = sAlpha[el];
   const bool blend = (m.limiter & kLimBlend) || m.alpha_mode == 1;
   const bool need_lo = blend || (m.limiter & kLimFlux);
   const double a = blend ? alpha : 0.0;
 
-  constexpr bool SRC = EQ::M == 6 || HasGravity<EQ>::value;
   const bool has_src = (EQ::M == 6 && m.source == 1) || (HasGravity<EQ>::value && m.source == 2);
   double dWx = 0.0, dWy = 0.0;
   if (HasGravity<EQ>::value && has_src) {
@@ -439,119 +496,162 @@ __device__ __forceinline__ void local_body_f64(const KParams<double>& P, const T
   }
 
   // ---------------- local cRK stages -----------------------------------
-  double Lst[S > 1 ? S - 1 : 1][M], Fa[M], Ga[M];
+  double Lst[S > 1 ? S - 1 : 1][M];
   double ea[SPT][M], Ut[SPT][M];
+  long long ho[M];  // sum_i b_i (FR volume part of the stage fluxes), fixed point
 #pragma unroll
   for (int v = 0; v < M; ++v) {
-    Fa[v] = Ga[v] = 0.0;
+    ho[v] = 0;
 #pragma unroll
     for (int mm = 0; mm < SPT; ++mm) ea[mm][v] = Ut[mm][v] = 0.0;
   }
-  int* const kx = sKx + (el * n + q) * M;  // this node's x-line and y-line
-  int* const ky = sKy + (el * n + p) * M;
   const int line_x = el * NP + n * q, line_y = el * NP + p;
+  // Exponents of the element's values in fixed point, per variable: kf is the
+  // exponent of the products |D/dx| |f|, |D/dy| |g| (the x and y fluxes so carry
+  // exponents kf - oD[0], kf - oD[1], and their sums need no alignment), ku the
+  // exponent of the stage state.
+  int* const kf = sKey + el * M;
+  int* const ku = kf + epb * M;
+  const int o0 = P.ds.oD[0], o1 = P.ds.oD[1];
+  const int kmin = kMinLineExp + max(o0, o1), kmax = kMaxLineExp + min(o0, o1);
 
-  // The x and y fluxes of this node into the line arrays in fixed point, and a
-  // barrier.  A line keeps its exponent from the first stage until a value
-  // needs two more bits; then (rarely: the vote) the line takes the larger one.
-  auto put_lines = [&](const double (&f)[M], const double (&g)[M], bool first) {
+  // The fluxes of this node, and where its traces are wanted the stage state,
+  // into the node arrays in fixed point, and a barrier.  An element keeps its
+  // exponents from the first stage until a value needs two more bits; then
+  // (rarely: the vote) it takes the larger ones.
+  auto put_nodes = [&](const double (&f)[M], const double (&g)[M], const double (&u)[M], bool first, bool traces) {
     if (first) {
 #pragma unroll
       for (int v = 0; v < M; ++v) {
-        atomicMax(kx + v, mag_key(f[v]));
-        atomicMax(ky + v, mag_key(g[v]));
+        atomicMax(kf + v, max(max(exp_of(f[v]) + o0, exp_of(g[v]) + o1), kmin));
+        atomicMax(ku + v, max(exp_of(u[v]), kMinLineExp));
       }
       __syncthreads();
     }
-    unsigned over = 0u;  // bit 2v: f[v] outgrew its line's exponent, bit 2v + 1: g[v]
+    unsigned over = 0u;  // bit 2v: f[v] or g[v] outgrew the exponent, 2v + 1: u[v]
+    auto put_all = [&]() {
 #pragma unroll
-    for (int v = 0; v < M; ++v) {
-      const int ex = line_exp(kx[v]), ey = line_exp(ky[v]);
-      over |= (unsigned((mag_key(f[v]) >> 20) > ex + 1) << (2 * v)) | (unsigned((mag_key(g[v]) >> 20) > ey + 1) << (2 * v + 1));
-      xB[v * stride + tid] = to_fixed(f[v], ex);
-      xC[v * stride + tid] = to_fixed(g[v], ey);
-    }
+      for (int v = 0; v < M; ++v) {
+        const int E = kf[v];
+        over |= unsigned(max(exp_of(f[v]) + o0, exp_of(g[v]) + o1) > E + 1) << (2 * v);
+        xB[v * stride + tid] = to_fixed(f[v], E - o0);
+        xC[v * stride + tid] = to_fixed(g[v], E - o1);
+        if (traces) {
+          const int Eu = ku[v];
+          over |= unsigned(exp_of(u[v]) > Eu + 1) << (2 * v + 1);
+          xA[v * stride + tid] = to_fixed(u[v], Eu);
+        }
+      }
+    };
+    put_all();
     if (first) {
       __syncthreads();
     } else if (__syncthreads_or(valid && over)) {
+      int before[M];
 #pragma unroll
-      for (int v = 0; v < M; ++v) {
-        if ((over >> (2 * v)) & 1u) atomicMax(kx + v, mag_key(f[v]));
-        if ((over >> (2 * v + 1)) & 1u) atomicMax(ky + v, mag_key(g[v]));
-      }
+      for (int v = 0; v < M; ++v) before[v] = kf[v];
       __syncthreads();
 #pragma unroll
       for (int v = 0; v < M; ++v) {
-        xB[v * stride + tid] = to_fixed(f[v], line_exp(kx[v]));
-        xC[v * stride + tid] = to_fixed(g[v], line_exp(ky[v]));
+        if ((over >> (2 * v)) & 1u) atomicMax(kf + v, max(exp_of(f[v]) + o0, exp_of(g[v]) + o1));
+        if ((over >> (2 * v + 1)) & 1u) atomicMax(ku + v, exp_of(u[v]));
       }
+      __syncthreads();
+      put_all();
+#pragma unroll
+      for (int v = 0; v < M; ++v) ho[v] >>= min(63, kf[v] - before[v]);
       __syncthreads();
     }
   };
-  // sum_r Ax[p][r] f(line_x, r) + Ay[q][r] g(line_y, r) of variable v
-  auto line_dot = [&](int v, const int2* Ax, const int2* Ay, int ox, int oy) -> double {
-    FixAcc ax{0, 0}, ay{0, 0};
+  const double kNaN = __longlong_as_double(0x7ff8000000000000ll);
+  // Trace along the line (base, step) of node values X with exponent E.
+  auto trace_dot = [&](const int2* X, int E, int base, int step, const int2* l) -> double {
+    FixAcc acc{0, 0};
 #pragma unroll
-    for (int r = 0; r < n; ++r) {
-      fix_mad(ax, xB[v * stride + line_x + r], Ax[p * n + r]);
-      fix_mad(ay, xC[v * stride + line_y + n * r], Ay[q * n + r]);
-    }
-    const int ex = line_exp(kx[v]), ey = line_exp(ky[v]);
-    if (max(ex, ey) > kMaxLineExp) return __longlong_as_double(0x7ff8000000000000ll);
-    return from_fixed2(fix_sum(ax), ex + ox, fix_sum(ay), ey + oy);
+    for (int r = 0; r < n; ++r) fix_mad(acc, X[base + step * r], l[r]);
+    return E > kMaxLineExp ? kNaN : from_fixed(fix_sum(acc), E + P.ds.oL);
   };
 
 #pragma unroll
   for (int i = 0; i < S; ++i) {
+    constexpr bool kSrcEq = SRC;
+    const bool avg = TB::b(i) != 0.0;           // the stage enters the time averages
+    const bool traces = i == 0 || avg;
     double ui[M], f[M], g[M];
+    vld_sh<M, stride>(ui, s0 + tid);
 #pragma unroll
-    for (int v = 0; v < M; ++v) ui[v] = un[v];
-#pragma unroll
-    for (int j = 0; j < i; ++j)
-      if (TB::a(i, j) != 0.0) vfma(ui, -sAdt[i * S + j], Lst[j]);
+    for (int j = 0; j < i; ++j) {
+      if (TB::a(i, j) == 0.0) continue;
+      if (kShL && j < 4) vfma_sh<M, stride>(ui, -sAdt[i * S + j], (j == 3 ? sD : sL + j * arr) + tid);
+      else vfma(ui, -sAdt[i * S + j], Lst[j]);
+    }
     EQ::flux_xy(ui, f, g, ph);
-    if (TB::b(i) != 0.0) {
-      vfma(Fa, TB::b(i), f);
-      vfma(Ga, TB::b(i), g);
-    }
-    if (SRC && has_src) {  // the time-averaged solution, for its source
+    double src[M];
+    if (kSrcEq && has_src) {
+      source_eval<EQ>(ui, dWx, dWy, src);
 #pragma unroll
-      for (int v = 0; v < M; ++v) {
-        double* ua = sD + v * stride + tid;
-        if (i == 0) *ua = TB::b(0) * ui[v];
-        else if (TB::b(i) != 0.0) *ua = fma(TB::b(i), ui[v], *ua);
+      for (int v = 0; v < M; ++v) {  // the time-averaged source, sum_i b_i s(u^(i))
+        double* sa = sS + v * stride + tid;
+        if (i == 0) *sa = TB::b(0) * src[v];
+        else if (avg) *sa = fma(TB::b(i), src[v], *sa);
       }
     }
-    vst_sh<M, stride>(sA + tid, ui);
-    if (i < S - 1) put_lines(f, g, i == 0);
-    else __syncthreads();
-    if (i < S - 1) {
+    if (i < S - 1 || avg) put_nodes(f, g, ui, i == 0, traces);
+    // one pass over the two lines for the stage residual D f / dx + D g / dy and
+    // the stage's part of the FR volume term (its matrices hold the factor b_i),
+    // two variables at a time (one load of a coefficient for both)
+    const int2* const bx = tB + 2 * i * n * n;
+    const int2* const by = bx + n * n;
 #pragma unroll
-      for (int v = 0; v < M; ++v) Lst[i < S - 1 ? i : 0][v] = line_dot(v, tDx, tDy, P.ds.oD[0], P.ds.oD[1]);
-      if (SRC && has_src) {
-        double us[M], s[M];
-        vld_sh<M, stride>(us, sA + tid);
-        source_eval<EQ>(us, dWx, dWy, s);
+    for (int v0 = 0; v0 < M; v0 += 2) {
+      constexpr int W = M > 1 ? 2 : 1;
+      FixAcc lo[W], hi[W];
 #pragma unroll
-        for (int v = 0; v < M; ++v) Lst[i < S - 1 ? i : 0][v] -= s[v];
+      for (int w = 0; w < W; ++w) lo[w] = hi[w] = FixAcc{0, 0};
+#pragma unroll
+      for (int d = 0; d < 2; ++d) {
+#pragma unroll
+        for (int r = 0; r < n; ++r) {
+          const int c = (d == 0 ? p : q) * n + r;
+          int2 cl, ch;
+          if (i < S - 1) cl = (d == 0 ? tDx : tDy)[c];
+          if (avg) ch = (d == 0 ? bx : by)[c];
+#pragma unroll
+          for (int w = 0; w < W; ++w) {
+            const int2 x = d == 0 ? xB[(v0 + w) * stride + line_x + r] : xC[(v0 + w) * stride + line_y + n * r];
+            if (i < S - 1) fix_mad(lo[w], x, cl);
+            if (avg) fix_mad(hi[w], x, ch);
+          }
+        }
+      }
+#pragma unroll
+      for (int w = 0; w < W; ++w) {
+        const int v = v0 + w;
+        if (avg) ho[v] += fix_sum(hi[w]);
+        if (i < S - 1) {
+          const int E = kf[v];
+          double L = E > kmax ? kNaN : from_fixed(fix_sum(lo[w]), E);
+          if (kSrcEq && has_src) L -= src[v];
+          if (kShL && i < 4) (i == 3 ? sD : sL + i * arr)[v * stride + tid] = L;
+          else Lst[i < S - 1 ? i : 0][v] = L;
+        }
       }
     }
-    if (i == 0 || TB::b(i) != 0.0) {
+    if (traces) {
 #pragma unroll
       for (int mm = 0; mm < SPT; ++mm) {
         const FaceSlot fs = face_slot<NSLOT, n>(tid + mm * T);
         const int eg = blk * epr + fs.el;
         if (fs.el < epr && eg < m.ne) {
           const int side = fs.side, j = fs.j;
+          const bool isx = side < 2;
+          const int base = fs.el * NP + (isx ? n * j : j), step = isx ? 1 : n;
+          const int* key = sKey + fs.el * M;
+          const int2* l = tL + (side & 1) * n;
           double ut[M];
 #pragma unroll
-          for (int v = 0; v < M; ++v) ut[v] = 0.0;
-#pragma unroll
-          for (int r = 0; r < n; ++r) {
-            const double l = (side & 1) ? tb.l1[r] : tb.l0[r];
-            vfma_sh<M, stride>(ut, l, sA + fs.el * NP + (side < 2 ? r + n * j : j + n * r));
-          }
-          if (TB::b(i) != 0.0) {
+          for (int v = 0; v < M; ++v) ut[v] = trace_dot(xA + v * stride, key[epb * M + v], base, step, l);
+          if (avg) {
             vfma(Ut[mm], TB::b(i), ut);
             if (m.dissipation == 2) {  // D-CSX: the stage trace, for the face kernel
 #pragma unroll
@@ -562,7 +662,7 @@ __device__ __forceinline__ void local_body_f64(const KParams<double>& P, const T
           if (i == 0 || m.central == 0) {
             double fn[M], vn, c2;
             flux_c2<EQ>(ut, side >> 1, fn, &vn, &c2, ph);
-            if (TB::b(i) != 0.0 && m.central == 0) vfma(ea[mm], TB::b(i), fn);  // EA, eq. (evaluate)
+            if (avg && m.central == 0) vfma(ea[mm], TB::b(i), fn);  // EA, eq. (evaluate)
             if (i == 0) {  // u^n trace: its wave speed, and the trace itself for D1
               P.b.slot[slot_index(0, side, eg, j, 4, m.ne, n)] = EQ::K > 0 ? fabs(vn) + sqrt_pos(c2) : vn;
               if (m.dissipation == 1) {
@@ -571,29 +671,29 @@ __device__ __forceinline__ void local_body_f64(const KParams<double>& P, const T
               }
             }
           }
+          if (avg && m.central == 1) {  // AE, eq. (extrapolate): the trace of the flux itself
+#pragma unroll
+            for (int v = 0; v < M; ++v)
+              ea[mm][v] = fma(TB::b(i), trace_dot((isx ? xB : xC) + v * stride, key[v] - (isx ? o0 : o1), base, step, l), ea[mm][v]);
+          }
         }
       }
     }
-    __syncthreads();
+    if (i < S - 1) __syncthreads();
   }
 
-  // ---------------- time averages: high-order volume part, face data ----
-  if (m.central == 1) {  // AE: the averages themselves, for their traces
-    vst_sh<M, stride>(sA + tid, Fa);
-  }
-  put_lines(Fa, Ga, false);
-  double HO[M];
+  // ---------------- high-order part of the update, face data -------------
+  // HO = u^n - dt (1 - a) sum_i b_i (FR volume part) + dt (time-averaged source)
+  // (into memory at once: the low-order part is added where alpha > 0)
+  {
+    const double dho = dt * (1.0 - a);
 #pragma unroll
-  for (int v = 0; v < M; ++v) HO[v] = line_dot(v, tDtx, tDty, P.ds.oDt[0], P.ds.oDt[1]);
-  // HO becomes the high-order part of the update, u^n - dt (1 - a) HO + dt S,
-  // with the source of the time-averaged solution (linear in u)
-  const double dho = dt * (1.0 - a);
-  vfma(HO, -dho, HO, un);
-  if (SRC && has_src) {
-    double us[M], Sa[M];
-    vld_sh<M, stride>(us, sD + tid);
-    source_eval<EQ>(us, dWx, dWy, Sa);
-    vfma(HO, dt, Sa);
+    for (int v = 0; v < M; ++v) {
+      const int E = kf[v];
+      double h = E > kmax ? kNaN : fma(-dho, from_fixed(ho[v], E + P.ds.oDt), s0[v * stride + tid]);
+      if (SRC && has_src) h = fma(dt, sS[v * stride + tid], h);
+      if (valid) P.b.P[((size_t)v * m.ne + e) * NP + k] = h;
+    }
   }
 #pragma unroll
   for (int mm = 0; mm < SPT; ++mm) {
@@ -601,70 +701,21 @@ __device__ __forceinline__ void local_body_f64(const KParams<double>& P, const T
     const int eg = blk * epr + fs.el;
     if (fs.el < epr && eg < m.ne) {
       // slots 1..M: the trace the dissipation jumps over (U; D1 stored u^n's);
-      // slots 1+M..: the EA average (AE: below)
+      // slots 1+M..: the central part (EA or AE average)
 #pragma unroll
       for (int v = 0; v < M; ++v) {
         if (m.dissipation != 1) P.b.slot[slot_index(1 + v, fs.side, eg, fs.j, 4, m.ne, n)] = Ut[mm][v];
-        if (m.central == 0) P.b.slot[slot_index(1 + M + v, fs.side, eg, fs.j, 4, m.ne, n)] = ea[mm][v];
-      }
-    }
-  }
-  if (m.central == 1) {  // AE, eq. (extrapolate): the trace of F on x faces, of G on y faces
-    for (int dir = 0; dir < 2; ++dir) {
-      if (dir == 1) {
-        __syncthreads();
-        vst_sh<M, stride>(sA + tid, Ga);
-        __syncthreads();
-      }
-#pragma unroll
-      for (int mm = 0; mm < SPT; ++mm) {
-        const FaceSlot fs = face_slot<NSLOT, n>(tid + mm * T);
-        const int eg = blk * epr + fs.el;
-        if (fs.el < epr && eg < m.ne && (fs.side >> 1) == dir) {
-          double Ft[M];
-#pragma unroll
-          for (int v = 0; v < M; ++v) Ft[v] = 0.0;
-#pragma unroll
-          for (int r = 0; r < n; ++r) {
-            const double l = (fs.side & 1) ? tb.l1[r] : tb.l0[r];
-            vfma_sh<M, stride>(Ft, l, sA + fs.el * NP + (dir == 0 ? r + n * fs.j : fs.j + n * r));
-          }
-#pragma unroll
-          for (int v = 0; v < M; ++v) P.b.slot[slot_index(1 + M + v, fs.side, eg, fs.j, 4, m.ne, n)] = Ft[v];
-        }
+        P.b.slot[slot_index(1 + M + v, fs.side, eg, fs.j, 4, m.ne, n)] = ea[mm][v];
       }
     }
   }
   __syncthreads();
 
   // ---------------- MUSCL-Hancock / first-order subcells -----------------
-  double LO[M];
-#pragma unroll
-  for (int v = 0; v < M; ++v) LO[v] = 0.0;
   if (need_lo) {
-    // neighbour nodes of the line: across a face the neighbour element's, at a
-    // boundary the side's ghost node (outflow: the own node; wall: its
-    // reflection; Dirichlet, inflow: given)
-    auto nb = [&](int v, int dir, int up) -> double {
-      const int c = dir == 0 ? p : q, step = dir == 0 ? 1 : n;
-      if (c != (up ? N : 0)) return s0[v * stride + tid + (up ? step : -step)];
-      const int side = 2 * dir + up, e2 = sNbr[el * 4 + side];
-      if (e2 >= 0) return P.b.u[((size_t)v * m.ne + e2) * NP + k + (up ? -N : N) * step];
-      const int bc = m.bcs[side];
-      if (bc == kBcDirichlet || bc == kBcInflow) {
-        double g[M];
-        ghost_at<M>(m, side, P.b.ctl->t, g);
-        return g[v];
-      }
-      return bc == kBcWall && v == 1 + dir ? -un[v] : un[v];
-    };
+    auto nb = [&](int v, int dir, int up) { return line_neighbour<N, EQ, stride>(P, s0 + tid, sNbr + el * 4, k, p, q, v, dir, up); };
     auto put_exact = [&]() {
-      double xm[M], xp[M], ym[M], yp[M];
-      hancock_states<N, EQ>(m, ph, tb, un, alpha, p, q, sHx[p], sHy[q], nb, xm, xp, ym, yp);
-      vst_sh<M, stride>(sA + tid, xm);
-      vst_sh<M, stride>(sB + tid, xp);
-      vst_sh<M, stride>(sC + tid, ym);
-      vst_sh<M, stride>(sD + tid, yp);
+      put_hancock_states<N, EQ, stride>(P, tb, s0 + tid, sNbr + el * 4, k, alpha, sHx[p], sHy[q], sA + tid);
     };
     // FP32 states sit in the low words of the same slots
     auto low = [&](double* base, int v) -> float& { return *reinterpret_cast<float*>(base + v * stride); };
@@ -680,7 +731,7 @@ __device__ __forceinline__ void local_body_f64(const KParams<double>& P, const T
     } else {
       float uf[M], xm[M], xp[M], ym[M], yp[M];
 #pragma unroll
-      for (int v = 0; v < M; ++v) uf[v] = trunc_f32(un[v]);
+      for (int v = 0; v < M; ++v) uf[v] = trunc_f32(s0[v * stride + tid]);
       auto nbf = [&](int v, int dir, int up) { return trunc_f32(nb(v, dir, up)); };
       unclear = !hancock_states_f32<N, EQ>(m, phf, tb, uf, trunc_f32(alpha), p, q, trunc_f32(sHx[p]), trunc_f32(sHy[q]),
                                            nbf, xm, xp, ym, yp);
@@ -731,10 +782,9 @@ __device__ __forceinline__ void local_body_f64(const KParams<double>& P, const T
       }
     }
     __syncthreads();
-    // low-order residual of the interior subfaces (eq. (low.order.update)); 0
-    // times alpha where the element is not blended
-    if (gt0(a)) {
-      double fr[M], fl[M];
+    // low-order residual of the interior subfaces (eq. (low.order.update))
+    if (valid && gt0(a)) {
+      double LO[M], fr[M], fl[M];
 #pragma unroll
       for (int v = 0; v < M; ++v) fr[v] = fl[v] = 0.0;
       if (p < N) vld_sh<M, stride>(fr, sB + tid);
@@ -747,6 +797,11 @@ __device__ __forceinline__ void local_body_f64(const KParams<double>& P, const T
       if (q > 0) vld_sh<M, stride>(fl, sD + tid - n);
       vsub(fr, fr, fl);
       vfma(LO, sWy[q], fr);
+#pragma unroll
+      for (int v = 0; v < M; ++v) {
+        double* val = P.b.P + ((size_t)v * m.ne + e) * NP + k;
+        *val = fma(-(dt * a), LO[v], *val);
+      }
     }
     // face-node data for the face kernel: evolved boundary state u* and the
     // candidate base of the flux limiter, u_b -+ c f_adj
@@ -785,14 +840,6 @@ __device__ __forceinline__ void local_body_f64(const KParams<double>& P, const T
         }
       }
     }
-  }
-
-  // ---------------- partial update --------------------------------------
-  if (valid) {
-    double val[M];
-    vfma(val, -(dt * a), LO, HO);
-#pragma unroll
-    for (int v = 0; v < M; ++v) P.b.P[((size_t)v * m.ne + e) * NP + k] = val[v];
   }
 }
 

@@ -1,13 +1,12 @@
 """The fixed-point dot products of the FP64 element kernel (csrc/cr_fixed.cuh),
 compiled for the host and compared with exact rational arithmetic.
 
-Bound of one sum over two lines of n terms, from the format: per term the
-value's truncation (2^-57 of max|a| max|x|, doubled when the line uses its bit
-of headroom), the coefficient's rounding (2^-58, likewise) and the dropped
-product of the low limbs (2^-57), the two shifts at the end (2^-57 together),
-and one rounding of the result (2^-53 of it).  Lines below 2^-959 keep the unit
-2^-1016 of the smallest line exponent, and results below 2^-1022 become 0 (FP64
-itself has nothing finer than 2^-1074 there).
+Bound of one sum over two lines of n terms with a common product scale, from the
+format: per term the value's truncation (2^-56 of the larger max|a| max|x| of the
+two lines), the coefficient's rounding (2^-57) and the dropped product of the low
+limbs (2^-56), the shift at the end (2^-57), and one rounding of the result (2^-53
+of it).  Values below 2^-959 keep the unit 2^-1016 of the smallest exponent, and
+results below 2^-1022 become 0 (FP64 itself has nothing finer than 2^-1074 there).
 """
 import ctypes
 import os
@@ -26,15 +25,15 @@ SRC = r"""
 using namespace crk;
 extern "C" double two_lines(const double* A, const double* x, int nx, const double* B, const double* y, int ny,
                             const double* whole_a, const double* whole_b, int nw, int below) {
-  int kx = 0, ky = 0;
-  for (int i = 0; i < nx; ++i) if (mag_key(x[i]) > kx) kx = mag_key(x[i]);
-  for (int i = 0; i < ny; ++i) if (mag_key(y[i]) > ky) ky = mag_key(y[i]);
-  const int ex = line_exp(kx) - below, ey = line_exp(ky) - below;
-  const int sa = fix_scale(whole_a, nw), sb = fix_scale(whole_b, nw);
-  FixAcc a{0, 0}, b{0, 0};
-  for (int i = 0; i < nx; ++i) fix_mad(a, to_fixed(x[i], ex), fix_coef(A[i], sa));
-  for (int i = 0; i < ny; ++i) fix_mad(b, to_fixed(y[i], ey), fix_coef(B[i], sb));
-  return from_fixed2(fix_sum(a), ex + fix_exp(sa), fix_sum(b), ey + fix_exp(sb));
+  const int sa = fix_scale(whole_a, nw), sb = fix_scale(whole_b, nw), oa = fix_exp(sa), ob = fix_exp(sb);
+  int k = kMinLineExp + (oa > ob ? oa : ob);
+  for (int i = 0; i < nx; ++i) if (exp_of(x[i]) + oa > k) k = exp_of(x[i]) + oa;
+  for (int i = 0; i < ny; ++i) if (exp_of(y[i]) + ob > k) k = exp_of(y[i]) + ob;
+  if (k - below - (oa > ob ? oa : ob) >= kMinLineExp) k -= below;
+  FixAcc acc{0, 0};
+  for (int i = 0; i < nx; ++i) fix_mad(acc, to_fixed(x[i], k - oa), fix_coef(A[i], sa));
+  for (int i = 0; i < ny; ++i) fix_mad(acc, to_fixed(y[i], k - ob), fix_coef(B[i], sb));
+  return from_fixed(fix_sum(acc), k);
 }
 """
 
@@ -90,8 +89,9 @@ def test_two_line_dot_products(two_lines, N, kind, below):
                 Fraction(float(np.abs(DB).max())) * Fraction(float(np.abs(y).max()))
             top = max(tops)
             amax = Fraction(float(max(np.abs(DA).max(), np.abs(DB).max())))
-            bound = top * Fraction(4 * 2 * n + 4, 2 ** 57) + abs(want) / 2 ** 53 \
-                + (2 * n * amax + 1) / Fraction(2 ** 1016)
+            tops_scale = amax / Fraction(float(min(np.abs(DA).max(), np.abs(DB).max())))
+            bound = top * Fraction(5 * 2 * n + 1, 2 ** 57) + abs(want) / 2 ** 53 \
+                + (2 * n * amax * max(tops_scale, 1) + 1) / Fraction(2 ** 1016)
             e = abs(Fraction(got) - want)
             assert e <= bound, (it, p, float(e), float(bound))
             if kind in ("smooth", "rough") and top > 0:
