@@ -836,7 +836,7 @@ template <int NP, int THREADS = 256> struct BlockShape {
   static constexpr int EPB = (THREADS / NP) > 0 ? (THREADS / NP) : 1;
   static constexpr int T = EPB * NP;
 };
-template <int NP, bool MIXED> using UpdateShape = BlockShape<NP, MIXED ? 128 : 256>;
+template <int NP, bool MIXED, int THREADS = 256> using UpdateShape = BlockShape<NP, (MIXED && THREADS > 128 ? 128 : THREADS)>;
 
 // Blocks of the element kernel.  FP64 in two dimensions (cr_local64.cuh): three
 // resident blocks (80 registers) so that one block's integer phases overlap
@@ -848,9 +848,9 @@ template <int DIM, class EQ, bool MIXED> struct LocalBlocks {
   static constexpr int value = DIM == 2 && !MIXED && EQ::M <= 4 ? 3 : MinBlocks<MIXED>::local;
 };
 
-template <int DIM, int N, class EQ, typename real, bool MIXED>
-__global__ void __launch_bounds__(256, LocalBlocks<DIM, EQ, MIXED>::value) k_local(const __grid_constant__ KParams<real> P) {
-  local_phase<DIM, N, EQ, real, MIXED, BlockShape<DIM == 2 ? (N + 1) * (N + 1) : N + 1>::T>(P, P.tb, blockIdx.x);
+template <int DIM, int N, class EQ, typename real, bool MIXED, int THREADS = 256>
+__global__ void __launch_bounds__(THREADS, LocalBlocks<DIM, EQ, MIXED>::value * (256 / THREADS)) k_local(const __grid_constant__ KParams<real> P) {
+  local_phase<DIM, N, EQ, real, MIXED, BlockShape<DIM == 2 ? (N + 1) * (N + 1) : N + 1, THREADS>::T>(P, P.tb, blockIdx.x);
 }
 
 // ===========================================================================
@@ -2091,9 +2091,9 @@ __device__ __forceinline__ void update_body(const KParams<real>& P, const Tab<re
 #undef RED0
 }
 
-template <int DIM, int N, class EQ, typename real, bool MIXED>
-__global__ void __launch_bounds__(256, MinBlocks<MIXED>::update) k_update(const __grid_constant__ KParams<real> P) {
-  update_body<DIM, N, EQ, real, MIXED, UpdateShape<DIM == 2 ? (N + 1) * (N + 1) : N + 1, MIXED>::T>(
+template <int DIM, int N, class EQ, typename real, bool MIXED, int THREADS = 256>
+__global__ void __launch_bounds__(THREADS, MinBlocks<MIXED>::update * (256 / THREADS)) k_update(const __grid_constant__ KParams<real> P) {
+  update_body<DIM, N, EQ, real, MIXED, UpdateShape<DIM == 2 ? (N + 1) * (N + 1) : N + 1, MIXED, THREADS>::T>(
       P, P.tb, P.td, blockIdx.x, gridDim.x, true);  // k_finish_step ends the step
 }
 

@@ -28,8 +28,8 @@ struct Impl {
   // variables per node in the element kernel's shared arrays (VarPack pads FP32 to pairs)
   static constexpr int MV = (M + VarPack<real>::VL - 1) / VarPack<real>::VL * VarPack<real>::VL;
 
-  // elements per block: about 256 threads per block (at least one element);
-  // the FP32-bulk update kernel takes UpdateShape's (128 threads)
+  // elements of a 256-thread block (at least one); the FP32-bulk update kernel
+  // takes UpdateShape's (128 threads), small 1D meshes kSmallThreads
   static constexpr int EPB = BlockShape<NP>::EPB;
 
   static size_t smem_local(int epb) {
@@ -57,24 +57,47 @@ struct Impl {
                                 cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem_update(EPB));
   }
 
+  // One-dimensional FP64 meshes with fewer than kSmallNodes solution points:
+  // blocks of kSmallThreads threads.  The kernels are bound by the FP64 pipe of the
+  // SMs that have work, and 256-thread blocks leave SMs idle (1D Euler N = 4, us
+  // per step: 4,000 elements 62 -> 53, 10,000 92 -> 76, but 20,000 133 -> 137 and
+  // 30,000 166 -> 188).  FP32 bulk is latency bound: the same within 1%.
+  static constexpr bool kHasSmall = DIM == 1 && !MIXED;
+  static constexpr int kSmallThreads = 64;
+  static constexpr long long kSmallNodes = 152ll * 512;
+  static bool small(const KParams<real>& P) { return kHasSmall && (long long)P.m.ne * NP < kSmallNodes; }
+
+  template <int THREADS>
+  static cudaError_t local_in(const KParams<real>& P, cudaStream_t s) {
+    constexpr int E = BlockShape<NP, THREADS>::EPB;
+    k_local<DIM, N, EQ, real, MIXED, THREADS><<<(P.m.ne + E - 1) / E, E * NP, smem_local(E), s>>>(P);
+    return cudaGetLastError();
+  }
+  template <int THREADS>
+  static cudaError_t update_in(const KParams<real>& P, cudaStream_t s) {
+    constexpr int E = UpdateShape<NP, MIXED, THREADS>::EPB;
+    k_update<DIM, N, EQ, real, MIXED, THREADS><<<(P.m.ne + E - 1) / E, E * NP, smem_update(E), s>>>(P);
+    return cudaGetLastError();
+  }
   static cudaError_t launch_local(const void* pv, cudaStream_t s) {
     const KParams<real>& P = *static_cast<const KParams<real>*>(pv);
-    const int grid = (P.m.ne + EPB - 1) / EPB;
-    k_local<DIM, N, EQ, real, MIXED><<<grid, EPB * NP, smem_local(EPB), s>>>(P);
-    return cudaGetLastError();
+    if constexpr (kHasSmall)
+      if (small(P)) return local_in<kSmallThreads>(P, s);
+    return local_in<256>(P, s);
   }
   static cudaError_t launch_face(const void* pv, cudaStream_t s) {
     const KParams<real>& P = *static_cast<const KParams<real>*>(pv);
     const int nfaces = P.m.ny * P.m.nfx * NFN + (DIM == 2 ? P.m.nfy * P.m.nx * n : 0);
-    k_face<DIM, N, EQ, real><<<(nfaces + 255) / 256, 256, 0, s>>>(P);
+    // few face nodes: one warp per block, so that every SM has some
+    const int threads = nfaces < 152 * 4 * 32 ? 32 : 256;
+    k_face<DIM, N, EQ, real><<<(nfaces + threads - 1) / threads, threads, 0, s>>>(P);
     return cudaGetLastError();
   }
   static cudaError_t launch_update(const void* pv, cudaStream_t s) {
     const KParams<real>& P = *static_cast<const KParams<real>*>(pv);
-    constexpr int EU = UpdateShape<NP, MIXED>::EPB;
-    const int grid = (P.m.ne + EU - 1) / EU;
-    k_update<DIM, N, EQ, real, MIXED><<<grid, EU * NP, smem_update(EU), s>>>(P);
-    return cudaGetLastError();
+    if constexpr (kHasSmall)
+      if (small(P)) return update_in<kSmallThreads>(P, s);
+    return update_in<256>(P, s);
   }
   static cudaError_t launch_finish(const void* pv, cudaStream_t s) {
     const KParams<real>& P = *static_cast<const KParams<real>*>(pv);
@@ -91,8 +114,8 @@ struct Impl {
 
   static cudaError_t prologue(const void* pv, cudaStream_t s) {
     const KParams<real>& P = *static_cast<const KParams<real>*>(pv);
-    const int grid = (P.m.ne + EPB - 1) / EPB;
-    k_prologue<DIM, N, EQ, real, MIXED><<<grid, EPB * NP, smem_update(EPB), s>>>(P);
+    const int E = small(P) ? BlockShape<NP, kSmallThreads>::EPB : EPB;
+    k_prologue<DIM, N, EQ, real, MIXED><<<(P.m.ne + E - 1) / E, E * NP, smem_update(E), s>>>(P);
     return cudaGetLastError();
   }
 
