@@ -33,8 +33,8 @@ struct Impl {
   static constexpr int EPB = BlockShape<NP>::EPB;
 
   static size_t smem_local(int epb) {
-    if constexpr (DIM == 2 && !MIXED)
-      return (size_t)5 * M * epb * NP * sizeof(double) + local64_extra<N, EQ>(epb);
+    if constexpr (HasLocal64<DIM, EQ, MIXED>::value)
+      return (size_t)5 * M * epb * NP * sizeof(double) + local64_extra<DIM, N, EQ>(epb);
     return (((size_t)5 * MV * epb * NP * sizeof(real) + 15) & ~(size_t)15) + (size_t)epb * sizeof(double) +
            (size_t)4 * n * n * sizeof(real) + (size_t)epb * 4 * sizeof(int);
   }

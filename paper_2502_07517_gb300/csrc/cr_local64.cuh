@@ -1,6 +1,6 @@
-// The FP64 element kernel in two dimensions (the body that k_local and the
-// batched kernels run for real = double, DIM = 2): the same phases and the same
-// outputs as local_body, arranged for the FP64 pipe.
+// The FP64 element kernel (the body that k_local and the batched kernels run for
+// real = double, except for scalar equations in one dimension): the same phases
+// and the same outputs as local_body, arranged for the FP64 pipe.
 //
 // What bounds it: GB300 issues one FP64 warp instruction per SM every 16
 // cycles, against two integer or FP32 ones per cycle, and the pipe was 90% busy
@@ -33,7 +33,8 @@
 // instructions, 56% of the pipe, 28% of the issue slots: latency bound) -> 5.03
 // ms, the stage residuals in shared memory and a third resident block -> 4.51 ms,
 // neighbour data and tables loaded by all threads at once -> 4.35 ms; ten-moment
-// N = 3 at 256 x 256 2.61 -> 1.42 ms.
+// N = 3 at 256 x 256 2.61 -> 1.42 ms; 1D Euler N = 4, whole step, 4,000 elements 53
+// -> 49 us, 60,000 elements 314 -> 163 us.
 #pragma once
 #include "cr_common.cuh"
 #include "cr_fixed.cuh"
@@ -97,7 +98,7 @@ __device__ __forceinline__ void rusanov_twice(const double* uL, const double* uR
   flux_c2<EQ>(uL, dir, fL, &vL, &cL, ph);
   flux_c2<EQ>(uR, dir, fR, &vR, &cR, ph);
   if constexpr (EQ::K > 0) lam = wave_max(vL, cL, vR, cR);
-  else lam = vL;  // linear advection: the speed does not depend on the state
+  else lam = __longlong_as_double(max(__double_as_longlong(vL), __double_as_longlong(vR)));  // (speeds are not negative)
 #pragma unroll
   for (int v = 0; v < EQ::M; ++v) out[v] = fma(-lam, uR[v] - uL[v], fL[v] + fR[v]);
 }
@@ -110,8 +111,9 @@ __device__ __forceinline__ bool clearly_admissible(const float* s, const float* 
   if constexpr (EQ::K == 0) return true;
   if (!(s[0] > kMarginF * A[0])) return false;
   if constexpr (IsEuler<EQ>::value) {
-    const float q = s[3] * s[0] - 0.5f * (s[1] * s[1] + s[2] * s[2]);
-    return q > kMarginF * (A[3] * A[0] + A[1] * A[1] + A[2] * A[2]);
+    constexpr int E = EQ::M - 1;
+    const float k2 = E == 3 ? s[1] * s[1] + s[2] * s[2] : s[1] * s[1], a2 = E == 3 ? A[1] * A[1] + A[2] * A[2] : A[1] * A[1];
+    return s[E] * s[0] - 0.5f * k2 > kMarginF * (A[E] * A[0] + a2);
   } else if constexpr (EQ::M == 6) {
     const float a11 = 2.0f * s[0] * s[3] - s[1] * s[1], a22 = 2.0f * s[0] * s[5] - s[2] * s[2];
     const float a12 = 2.0f * s[0] * s[4] - s[1] * s[2];
@@ -121,10 +123,10 @@ __device__ __forceinline__ bool clearly_admissible(const float* s, const float* 
   return true;
 }
 
-// MUSCL-Hancock states of one node (Sec. 4.2): the evolved states at the four
-// subcell faces, or the node value where one of them is not admissible.  nb(v,
+// MUSCL-Hancock states of one node (Sec. 4.2): the evolved states at its
+// subcell faces (in one dimension the y states are not formed), or the node value where one of them is not admissible.  nb(v,
 // dir, up) is the neighbour node's value along the line; hx, hy = dt / (2 w h).
-template <int N, class EQ, class Nb>
+template <int DIM, int N, class EQ, class Nb>
 __device__ __forceinline__ void hancock_states(const Mesh& m, const Phys<double>& ph, const Tab<double>& tb,
                                                const double (&un)[EQ::M], double alpha, int p, int q, double hx,
                                                double hy, Nb nb, double (&xm)[EQ::M], double (&xp)[EQ::M],
@@ -145,20 +147,24 @@ __device__ __forceinline__ void hancock_states(const Mesh& m, const Phys<double>
     }
   };
   slopes(sx, p, 0);
-  slopes(sy, q, 1);
+  if (DIM == 2) slopes(sy, q, 1);
   double fxm[M], fxp[M], fym[M], fyp[M], Fm[M], Fp[M], ex[M];
   vfma(fxm, tb.dm[p], sx, un);
   vfma(fxp, tb.dp[p], sx, un);
-  vfma(fym, tb.dm[q], sy, un);
-  vfma(fyp, tb.dp[q], sy, un);
+  if (DIM == 2) {
+    vfma(fym, tb.dm[q], sy, un);
+    vfma(fyp, tb.dp[q], sy, un);
+  }
   EQ::flux(fxm, 0, Fm, ph);
   EQ::flux(fxp, 0, Fp, ph);
   vsub(ex, Fp, Fm);
   vmul(ex, ex, hx);
-  EQ::flux(fym, 1, Fm, ph);
-  EQ::flux(fyp, 1, Fp, ph);
-  vsub(Fp, Fp, Fm);
-  vfma(ex, hy, Fp);
+  if (DIM == 2) {
+    EQ::flux(fym, 1, Fm, ph);
+    EQ::flux(fyp, 1, Fp, ph);
+    vsub(Fp, Fp, Fm);
+    vfma(ex, hy, Fp);
+  }
   bool ok = true;
   if constexpr (EQ::K > 0) {
     float uf[M], xf[M], yf[M], ef[M], A[M], st[M];
@@ -168,12 +174,13 @@ __device__ __forceinline__ void hancock_states(const Mesh& m, const Phys<double>
     for (int v = 0; v < M; ++v) {
       uf[v] = trunc_f32(un[v]);
       xf[v] = trunc_f32(sx[v]);
-      yf[v] = trunc_f32(sy[v]);
+      yf[v] = DIM == 2 ? trunc_f32(sy[v]) : 0.0f;
       ef[v] = trunc_f32(ex[v]);
       A[v] = fabsf(uf[v]) + fabsf(xf[v]) + fabsf(yf[v]) + fabsf(ef[v]);
     }
 #pragma unroll
-    for (int c = 0; c < 8; ++c) {  // four face states, then evolved
+    for (int c = 0; c < 8; ++c) {  // the face states, then evolved
+      if (DIM == 1 && (c & 2)) continue;
       const float d = (c & 3) == 0 ? dmx : (c & 3) == 1 ? dpx : (c & 3) == 2 ? dmy : dpy;
 #pragma unroll
       for (int v = 0; v < M; ++v) {
@@ -186,19 +193,26 @@ __device__ __forceinline__ void hancock_states(const Mesh& m, const Phys<double>
   double exm[M], exp_[M], eym[M], eyp[M];
   vsub(exm, fxm, ex);
   vsub(exp_, fxp, ex);
-  vsub(eym, fym, ex);
-  vsub(eyp, fyp, ex);
-  if (!ok)
+  if (DIM == 2) {
+    vsub(eym, fym, ex);
+    vsub(eyp, fyp, ex);
+  }
+  if (!ok) {
     ok = EQ::admissible_fast(fxm, ph) && EQ::admissible_fast(fxp, ph) && EQ::admissible_fast(exm, ph) &&
-         EQ::admissible_fast(exp_, ph) && EQ::admissible_fast(fym, ph) && EQ::admissible_fast(fyp, ph) &&
-         EQ::admissible_fast(eym, ph) && EQ::admissible_fast(eyp, ph);
+         EQ::admissible_fast(exp_, ph);
+    if (DIM == 2)
+      ok = ok && EQ::admissible_fast(fym, ph) && EQ::admissible_fast(fyp, ph) && EQ::admissible_fast(eym, ph) &&
+           EQ::admissible_fast(eyp, ph);
+  }
   if (ok) {
 #pragma unroll
     for (int v = 0; v < M; ++v) {
       xm[v] = exm[v];
       xp[v] = exp_[v];
-      ym[v] = eym[v];
-      yp[v] = eyp[v];
+      if (DIM == 2) {
+        ym[v] = eym[v];
+        yp[v] = eyp[v];
+      }
     }
   }
 }
@@ -208,10 +222,10 @@ __device__ __forceinline__ void hancock_states(const Mesh& m, const Phys<double>
 // across a face from the neighbour element (nbr: the element's face neighbours),
 // at a boundary the side's ghost node (outflow: the own node; wall: its
 // reflection; Dirichlet, inflow: given).
-template <int N, class EQ, int STRIDE>
+template <int DIM, int N, class EQ, int STRIDE>
 __device__ __forceinline__ double line_neighbour(const KParams<double>& P, const double* u, const int* nbr, int k, int p,
                                                  int q, int v, int dir, int up) {
-  constexpr int n = N + 1, NP = n * n, M = EQ::M;
+  constexpr int n = N + 1, NP = DIM == 2 ? n * n : n, M = EQ::M;
   const Mesh& m = P.m;
   const int c = dir == 0 ? p : q, step = dir == 0 ? 1 : n;
   if (c != (up ? N : 0)) return u[v * STRIDE + (up ? step : -step)];
@@ -230,25 +244,27 @@ __device__ __forceinline__ double line_neighbour(const KParams<double>& P, const
 // hancock_states of a block's node into the four node arrays at st (M STRIDE
 // apart).  Out of line: only blended elements, their neighbours and those beside
 // a boundary come here, and the element kernel keeps its registers.
-template <int N, class EQ, int STRIDE>
+template <int DIM, int N, class EQ, int STRIDE>
 __device__ __noinline__ void put_hancock_states(const KParams<double>& P, const Tab<double>& tb, const double* u,
                                                 const int* nbr, int k, double alpha, double hx, double hy, double* st) {
   constexpr int M = EQ::M;
-  const int p = k % (N + 1), q = k / (N + 1);
+  const int p = DIM == 2 ? k % (N + 1) : k, q = DIM == 2 ? k / (N + 1) : 0;
   double un[M], xm[M], xp[M], ym[M], yp[M];
   vld_sh<M, STRIDE>(un, u);
-  auto nb = [&](int v, int dir, int up) { return line_neighbour<N, EQ, STRIDE>(P, u, nbr, k, p, q, v, dir, up); };
-  hancock_states<N, EQ>(P.m, P.ph, tb, un, alpha, p, q, hx, hy, nb, xm, xp, ym, yp);
+  auto nb = [&](int v, int dir, int up) { return line_neighbour<DIM, N, EQ, STRIDE>(P, u, nbr, k, p, q, v, dir, up); };
+  hancock_states<DIM, N, EQ>(P.m, P.ph, tb, un, alpha, p, q, hx, hy, nb, xm, xp, ym, yp);
   vst_sh<M, STRIDE>(st, xm);
   vst_sh<M, STRIDE>(st + M * STRIDE, xp);
-  vst_sh<M, STRIDE>(st + 2 * M * STRIDE, ym);
-  vst_sh<M, STRIDE>(st + 3 * M * STRIDE, yp);
+  if (DIM == 2) {
+    vst_sh<M, STRIDE>(st + 2 * M * STRIDE, ym);
+    vst_sh<M, STRIDE>(st + 3 * M * STRIDE, yp);
+  }
 }
 
 // The same in FP32, for elements whose low-order scheme only feeds the screen of
 // the flux limiter (see the body).  Returns false where admissibility is not
 // clear in FP32 (the FP64 form then decides).
-template <int N, class EQ, class Nb>
+template <int DIM, int N, class EQ, class Nb>
 __device__ __forceinline__ bool hancock_states_f32(const Mesh& m, const Phys<float>& ph, const Tab<double>& tb,
                                                    const float (&un)[EQ::M], float alpha, int p, int q, float hx,
                                                    float hy, Nb nb, float (&xm)[EQ::M], float (&xp)[EQ::M],
@@ -268,30 +284,37 @@ __device__ __forceinline__ bool hancock_states_f32(const Mesh& m, const Phys<flo
     }
   };
   slopes(sx, p, 0);
-  slopes(sy, q, 1);
+  if (DIM == 2) slopes(sy, q, 1);
   float Fm[M], Fp[M], ex[M], vn, c2;
   vfma(xm, trunc_f32(tb.dm[p]), sx, un);
   vfma(xp, trunc_f32(tb.dp[p]), sx, un);
-  vfma(ym, trunc_f32(tb.dm[q]), sy, un);
-  vfma(yp, trunc_f32(tb.dp[q]), sy, un);
+  if (DIM == 2) {
+    vfma(ym, trunc_f32(tb.dm[q]), sy, un);
+    vfma(yp, trunc_f32(tb.dp[q]), sy, un);
+  }
   flux_c2_f32<EQ>(xm, 0, Fm, &vn, &c2, ph);
   flux_c2_f32<EQ>(xp, 0, Fp, &vn, &c2, ph);
   vsub(ex, Fp, Fm);
   vmul(ex, ex, hx);
-  flux_c2_f32<EQ>(ym, 1, Fm, &vn, &c2, ph);
-  flux_c2_f32<EQ>(yp, 1, Fp, &vn, &c2, ph);
-  vsub(Fp, Fp, Fm);
-  vfma(ex, hy, Fp);
+  if (DIM == 2) {
+    flux_c2_f32<EQ>(ym, 1, Fm, &vn, &c2, ph);
+    flux_c2_f32<EQ>(yp, 1, Fp, &vn, &c2, ph);
+    vsub(Fp, Fp, Fm);
+    vfma(ex, hy, Fp);
+  }
 #pragma unroll
-  for (int v = 0; v < M; ++v) A[v] = fabsf(un[v]) + fabsf(sx[v]) + fabsf(sy[v]) + fabsf(ex[v]);
-  bool ok = clearly_admissible<EQ>(xm, A) && clearly_admissible<EQ>(xp, A) && clearly_admissible<EQ>(ym, A) &&
-            clearly_admissible<EQ>(yp, A);
+  for (int v = 0; v < M; ++v) A[v] = fabsf(un[v]) + fabsf(sx[v]) + (DIM == 2 ? fabsf(sy[v]) : 0.0f) + fabsf(ex[v]);
+  bool ok = clearly_admissible<EQ>(xm, A) && clearly_admissible<EQ>(xp, A);
   vsub(xm, xm, ex);
   vsub(xp, xp, ex);
-  vsub(ym, ym, ex);
-  vsub(yp, yp, ex);
-  return ok && clearly_admissible<EQ>(xm, A) && clearly_admissible<EQ>(xp, A) && clearly_admissible<EQ>(ym, A) &&
-         clearly_admissible<EQ>(yp, A);
+  ok = ok && clearly_admissible<EQ>(xm, A) && clearly_admissible<EQ>(xp, A);
+  if (DIM == 2) {
+    ok = ok && clearly_admissible<EQ>(ym, A) && clearly_admissible<EQ>(yp, A);
+    vsub(ym, ym, ex);
+    vsub(yp, yp, ex);
+    ok = ok && clearly_admissible<EQ>(ym, A) && clearly_admissible<EQ>(yp, A);
+  }
+  return ok;
 }
 
 // FP32 face data carry their density negated (their states are clearly
@@ -305,13 +328,13 @@ __device__ __forceinline__ bool is_f32_face_data(double density) {
 // the state in memory into the slots.  For the face kernel, where the screen of
 // the limiter leaves a face open; rare, so kept out of line.  Elements beside a
 // boundary always have FP64 data and are left as they are.
-template <int N, class EQ>
+template <int DIM, int N, class EQ>
 __device__ __noinline__ void exact_face_data(const KParams<double>& P, const Tab<double>& tb, int e, int side, int j,
                                              double dt) {
-  constexpr int n = N + 1, NP = n * n, M = EQ::M;
+  constexpr int n = N + 1, NP = DIM == 2 ? n * n : n, M = EQ::M;
   const Mesh& m = P.m;
 #pragma unroll
-  for (int f = 0; f < 4; ++f)
+  for (int f = 0; f < 2 * DIM; ++f)
     if (neighbour(m, e, f) < 0) return;
   const double alpha = P.b.alpha[e];
   const int dir = side >> 1;
@@ -332,8 +355,8 @@ __device__ __noinline__ void exact_face_data(const KParams<double>& P, const Tab
       }
       return P.b.u[((size_t)v * m.ne + ee) * NP + kk];
     };
-    const double hx = dt * (0.5 * tb.invw[p] * P.ph.invdx), hy = dt * (0.5 * tb.invw[q] * P.ph.invdy);
-    hancock_states<N, EQ>(m, P.ph, tb, un, alpha, p, q, hx, hy, nb, xm, xp, ym, yp);
+    const double hx = dt * (0.5 * tb.invw[p] * P.ph.invdx), hy = DIM == 2 ? dt * (0.5 * tb.invw[q] * P.ph.invdy) : 0.0;
+    hancock_states<DIM, N, EQ>(m, P.ph, tb, un, alpha, p, q, hx, hy, nb, xm, xp, ym, yp);
 #pragma unroll
     for (int v = 0; v < M; ++v) {
       const double lo = dir == 0 ? xm[v] : ym[v], hi = dir == 0 ? xp[v] : yp[v];
@@ -348,31 +371,32 @@ __device__ __noinline__ void exact_face_data(const KParams<double>& P, const Tab
   const double c = 0.5 * dt * ((side & 1) ? P.ph.cflim[side] : -P.ph.cflim[side]);
 #pragma unroll
   for (int v = 0; v < M; ++v) {
-    P.b.slot[slot_index(1 + 2 * M + v, side, e, j, 4, m.ne, n)] = st[0][v];
-    P.b.slot[slot_index(1 + 3 * M + v, side, e, j, 4, m.ne, n)] = fma(c, f[v], ub[v]);
+    P.b.slot[slot_index(1 + 2 * M + v, side, e, j, 2 * DIM, m.ne, DIM == 2 ? n : 1)] = st[0][v];
+    P.b.slot[slot_index(1 + 3 * M + v, side, e, j, 2 * DIM, m.ne, DIM == 2 ? n : 1)] = fma(c, f[v], ub[v]);
   }
 }
 
 // Shared memory of the body beyond the five node arrays, in bytes.
-template <int N, class EQ>
+template <int DIM, int N, class EQ>
 __host__ __device__ constexpr size_t local64_extra(int epb) {
   constexpr int n = N + 1, S = Tableau<N>::S;
-  constexpr size_t src = (EQ::M == 6 || HasGravity<EQ>::value ? EQ::M * n * n : 0)  // the averaged source,
-                         + (N == 4 ? 3 * EQ::M * n * n : 0);                      // stage residuals
+  constexpr size_t src = (EQ::M == 6 || HasGravity<EQ>::value ? EQ::M * (DIM == 2 ? n * n : n) : 0)  // the averaged source,
+                         + (N == 4 ? 3 * EQ::M * (DIM == 2 ? n * n : n) : 0);                      // stage residuals
   return (size_t)epb * (1 + src) * sizeof(double) + (size_t)(2 * (1 + S) * n * n + 2 * n) * sizeof(int2) +
          (size_t)(S * S + 4 * n) * sizeof(double) + (size_t)epb * (5 + 2 * EQ::M) * sizeof(int);
 }
 
-template <int N, class EQ, int T>
+template <int DIM, int N, class EQ, int T>
 __device__ __forceinline__ void local_body_f64(const KParams<double>& P, const Tab<double>& tb, const int blk) {
-  constexpr int n = N + 1, NP = n * n, M = EQ::M, S = Tableau<N>::S, NSLOT = 4 * n;
+  constexpr int n = N + 1, NP = DIM == 2 ? n * n : n, M = EQ::M, S = Tableau<N>::S;
+  constexpr int NSIDE = 2 * DIM, NFN = DIM == 2 ? n : 1, NSLOT = NSIDE * NFN;
   constexpr int SPT = (NSLOT + NP - 1) / NP;
   using TB = Tableau<N>;
   const Mesh& m = P.m;
   const Phys<double>& ph = P.ph;
   constexpr int epb = (T + NP - 1) / NP, epr = T / NP;
   const int tid = threadIdx.x;
-  const int el = tid / NP, k = tid - el * NP, p = k % n, q = k / n;
+  const int el = tid / NP, k = tid - el * NP, p = DIM == 2 ? k % n : k, q = DIM == 2 ? k / n : 0;
   const int e = blk * epr + el;
   const bool valid = el < epr && e < m.ne;
   const int ee = valid ? e : m.ne - 1;
@@ -428,8 +452,9 @@ __device__ __forceinline__ void local_body_f64(const KParams<double>& P, const T
   // answers (cr_screen.cuh; the face kernel forms the FP64 data itself where it
   // does not).  One thread per element and cell of the 13 within two steps, so
   // that their loads go out together.
-  for (int t = T - 1 - tid; t < epb * 13; t += T) {
-    const int e2 = t / 13, c = t - e2 * 13;
+  constexpr int NC = DIM == 2 ? 13 : 5;
+  for (int t = T - 1 - tid; t < epb * NC; t += T) {
+    const int e2 = t / NC, c = DIM == 2 ? t - e2 * NC : (0x65410 >> (4 * (t - e2 * NC))) & 15;
     const int eg0 = blk * epr + e2, eg = e2 < epr && eg0 < m.ne ? eg0 : m.ne - 1;
     // cell offsets: the face neighbours (x-, x+, y-, y+), the element, the second ring
     // plus 2, three bits each
@@ -438,7 +463,8 @@ __device__ __forceinline__ void local_body_f64(const KParams<double>& P, const T
     bool in = true;
     if (m.bcx == 0) cx = (cx % m.nx + m.nx) % m.nx;
     else in = cx >= 0 && cx < m.nx;
-    if (m.bcy == 0) cy = (cy % m.ny + m.ny) % m.ny;
+    if (DIM == 1) cy = 0;
+    else if (m.bcy == 0) cy = (cy % m.ny + m.ny) % m.ny;
     else in = in && cy >= 0 && cy < m.ny;
     const int ec = in ? cx + m.nx * cy : -1;
     if (c < 4) {
@@ -489,10 +515,10 @@ __device__ __forceinline__ void local_body_f64(const KParams<double>& P, const T
   double dWx = 0.0, dWy = 0.0;
   if (HasGravity<EQ>::value && has_src) {
     dWx = m.grav[0];
-    dWy = m.grav[1];
+    dWy = DIM == 2 ? m.grav[1] : 0.0;
   } else if (SRC && has_src) {
-    const double x = m.x0 + (ix + tb.xi[p]) * m.dx, y = m.y0 + (iy + tb.xi[q]) * m.dy;
-    source_grad<2, double>(m, x - m.src_cx, y - m.src_cy, &dWx, &dWy);
+    const double x = m.x0 + (ix + tb.xi[p]) * m.dx, y = DIM == 2 ? m.y0 + (iy + tb.xi[q]) * m.dy : 0.0;
+    source_grad<DIM, double>(m, x - m.src_cx, DIM == 2 ? y - m.src_cy : 0.0, &dWx, &dWy);
   }
 
   // ---------------- local cRK stages -----------------------------------
@@ -512,7 +538,7 @@ __device__ __forceinline__ void local_body_f64(const KParams<double>& P, const T
   // exponent of the stage state.
   int* const kf = sKey + el * M;
   int* const ku = kf + epb * M;
-  const int o0 = P.ds.oD[0], o1 = P.ds.oD[1];
+  const int o0 = P.ds.oD[0], o1 = DIM == 2 ? P.ds.oD[1] : o0;
   const int kmin = kMinLineExp + max(o0, o1), kmax = kMaxLineExp + min(o0, o1);
 
   // The fluxes of this node, and where its traces are wanted the stage state,
@@ -523,7 +549,7 @@ __device__ __forceinline__ void local_body_f64(const KParams<double>& P, const T
     if (first) {
 #pragma unroll
       for (int v = 0; v < M; ++v) {
-        atomicMax(kf + v, max(max(exp_of(f[v]) + o0, exp_of(g[v]) + o1), kmin));
+        atomicMax(kf + v, max((DIM == 2 ? max(exp_of(f[v]) + o0, exp_of(g[v]) + o1) : exp_of(f[v]) + o0), kmin));
         atomicMax(ku + v, max(exp_of(u[v]), kMinLineExp));
       }
       __syncthreads();
@@ -533,9 +559,9 @@ __device__ __forceinline__ void local_body_f64(const KParams<double>& P, const T
 #pragma unroll
       for (int v = 0; v < M; ++v) {
         const int E = kf[v];
-        over |= unsigned(max(exp_of(f[v]) + o0, exp_of(g[v]) + o1) > E + 1) << (2 * v);
+        over |= unsigned((DIM == 2 ? max(exp_of(f[v]) + o0, exp_of(g[v]) + o1) : exp_of(f[v]) + o0) > E + 1) << (2 * v);
         xB[v * stride + tid] = to_fixed(f[v], E - o0);
-        xC[v * stride + tid] = to_fixed(g[v], E - o1);
+        if (DIM == 2) xC[v * stride + tid] = to_fixed(g[v], E - o1);
         if (traces) {
           const int Eu = ku[v];
           over |= unsigned(exp_of(u[v]) > Eu + 1) << (2 * v + 1);
@@ -553,7 +579,7 @@ __device__ __forceinline__ void local_body_f64(const KParams<double>& P, const T
       __syncthreads();
 #pragma unroll
       for (int v = 0; v < M; ++v) {
-        if ((over >> (2 * v)) & 1u) atomicMax(kf + v, max(exp_of(f[v]) + o0, exp_of(g[v]) + o1));
+        if ((over >> (2 * v)) & 1u) atomicMax(kf + v, (DIM == 2 ? max(exp_of(f[v]) + o0, exp_of(g[v]) + o1) : exp_of(f[v]) + o0));
         if ((over >> (2 * v + 1)) & 1u) atomicMax(ku + v, exp_of(u[v]));
       }
       __syncthreads();
@@ -585,7 +611,8 @@ __device__ __forceinline__ void local_body_f64(const KParams<double>& P, const T
       if (kShL && j < 4) vfma_sh<M, stride>(ui, -sAdt[i * S + j], (j == 3 ? sD : sL + j * arr) + tid);
       else vfma(ui, -sAdt[i * S + j], Lst[j]);
     }
-    EQ::flux_xy(ui, f, g, ph);
+    if (DIM == 2) EQ::flux_xy(ui, f, g, ph);
+    else EQ::flux(ui, 0, f, ph);
     double src[M];
     if (kSrcEq && has_src) {
       source_eval<EQ>(ui, dWx, dWy, src);
@@ -604,12 +631,12 @@ __device__ __forceinline__ void local_body_f64(const KParams<double>& P, const T
     const int2* const by = bx + n * n;
 #pragma unroll
     for (int v0 = 0; v0 < M; v0 += 2) {
-      constexpr int W = M > 1 ? 2 : 1;
-      FixAcc lo[W], hi[W];
+      const int W = M - v0 < 2 ? M - v0 : 2;
+      FixAcc lo[2], hi[2];
 #pragma unroll
-      for (int w = 0; w < W; ++w) lo[w] = hi[w] = FixAcc{0, 0};
+      for (int w = 0; w < 2; ++w) lo[w] = hi[w] = FixAcc{0, 0};
 #pragma unroll
-      for (int d = 0; d < 2; ++d) {
+      for (int d = 0; d < DIM; ++d) {
 #pragma unroll
         for (int r = 0; r < n; ++r) {
           const int c = (d == 0 ? p : q) * n + r;
@@ -617,7 +644,8 @@ __device__ __forceinline__ void local_body_f64(const KParams<double>& P, const T
           if (i < S - 1) cl = (d == 0 ? tDx : tDy)[c];
           if (avg) ch = (d == 0 ? bx : by)[c];
 #pragma unroll
-          for (int w = 0; w < W; ++w) {
+          for (int w = 0; w < 2; ++w) {
+            if (w >= W) break;
             const int2 x = d == 0 ? xB[(v0 + w) * stride + line_x + r] : xC[(v0 + w) * stride + line_y + n * r];
             if (i < S - 1) fix_mad(lo[w], x, cl);
             if (avg) fix_mad(hi[w], x, ch);
@@ -625,7 +653,8 @@ __device__ __forceinline__ void local_body_f64(const KParams<double>& P, const T
         }
       }
 #pragma unroll
-      for (int w = 0; w < W; ++w) {
+      for (int w = 0; w < 2; ++w) {
+        if (w >= W) break;
         const int v = v0 + w;
         if (avg) ho[v] += fix_sum(hi[w]);
         if (i < S - 1) {
@@ -640,7 +669,7 @@ __device__ __forceinline__ void local_body_f64(const KParams<double>& P, const T
     if (traces) {
 #pragma unroll
       for (int mm = 0; mm < SPT; ++mm) {
-        const FaceSlot fs = face_slot<NSLOT, n>(tid + mm * T);
+        const FaceSlot fs = face_slot<NSLOT, NFN>(tid + mm * T);
         const int eg = blk * epr + fs.el;
         if (fs.el < epr && eg < m.ne) {
           const int side = fs.side, j = fs.j;
@@ -656,7 +685,7 @@ __device__ __forceinline__ void local_body_f64(const KParams<double>& P, const T
             if (m.dissipation == 2) {  // D-CSX: the stage trace, for the face kernel
 #pragma unroll
               for (int v = 0; v < M; ++v)
-                P.b.slot[slot_index(1 + 4 * M + i * M + v, side, eg, j, 4, m.ne, n)] = ut[v];
+                P.b.slot[slot_index(1 + 4 * M + i * M + v, side, eg, j, NSIDE, m.ne, NFN)] = ut[v];
             }
           }
           if (i == 0 || m.central == 0) {
@@ -664,10 +693,10 @@ __device__ __forceinline__ void local_body_f64(const KParams<double>& P, const T
             flux_c2<EQ>(ut, side >> 1, fn, &vn, &c2, ph);
             if (avg && m.central == 0) vfma(ea[mm], TB::b(i), fn);  // EA, eq. (evaluate)
             if (i == 0) {  // u^n trace: its wave speed, and the trace itself for D1
-              P.b.slot[slot_index(0, side, eg, j, 4, m.ne, n)] = EQ::K > 0 ? fabs(vn) + sqrt_pos(c2) : vn;
+              P.b.slot[slot_index(0, side, eg, j, NSIDE, m.ne, NFN)] = EQ::K > 0 ? fabs(vn) + sqrt_pos(c2) : vn;
               if (m.dissipation == 1) {
 #pragma unroll
-                for (int v = 0; v < M; ++v) P.b.slot[slot_index(1 + v, side, eg, j, 4, m.ne, n)] = ut[v];
+                for (int v = 0; v < M; ++v) P.b.slot[slot_index(1 + v, side, eg, j, NSIDE, m.ne, NFN)] = ut[v];
               }
             }
           }
@@ -697,15 +726,15 @@ __device__ __forceinline__ void local_body_f64(const KParams<double>& P, const T
   }
 #pragma unroll
   for (int mm = 0; mm < SPT; ++mm) {
-    const FaceSlot fs = face_slot<NSLOT, n>(tid + mm * T);
+    const FaceSlot fs = face_slot<NSLOT, NFN>(tid + mm * T);
     const int eg = blk * epr + fs.el;
     if (fs.el < epr && eg < m.ne) {
       // slots 1..M: the trace the dissipation jumps over (U; D1 stored u^n's);
       // slots 1+M..: the central part (EA or AE average)
 #pragma unroll
       for (int v = 0; v < M; ++v) {
-        if (m.dissipation != 1) P.b.slot[slot_index(1 + v, fs.side, eg, fs.j, 4, m.ne, n)] = Ut[mm][v];
-        P.b.slot[slot_index(1 + M + v, fs.side, eg, fs.j, 4, m.ne, n)] = ea[mm][v];
+        if (m.dissipation != 1) P.b.slot[slot_index(1 + v, fs.side, eg, fs.j, NSIDE, m.ne, NFN)] = Ut[mm][v];
+        P.b.slot[slot_index(1 + M + v, fs.side, eg, fs.j, NSIDE, m.ne, NFN)] = ea[mm][v];
       }
     }
   }
@@ -713,9 +742,9 @@ __device__ __forceinline__ void local_body_f64(const KParams<double>& P, const T
 
   // ---------------- MUSCL-Hancock / first-order subcells -----------------
   if (need_lo) {
-    auto nb = [&](int v, int dir, int up) { return line_neighbour<N, EQ, stride>(P, s0 + tid, sNbr + el * 4, k, p, q, v, dir, up); };
+    auto nb = [&](int v, int dir, int up) { return line_neighbour<DIM, N, EQ, stride>(P, s0 + tid, sNbr + el * 4, k, p, q, v, dir, up); };
     auto put_exact = [&]() {
-      put_hancock_states<N, EQ, stride>(P, tb, s0 + tid, sNbr + el * 4, k, alpha, sHx[p], sHy[q], sA + tid);
+      put_hancock_states<DIM, N, EQ, stride>(P, tb, s0 + tid, sNbr + el * 4, k, alpha, sHx[p], sHy[q], sA + tid);
     };
     // FP32 states sit in the low words of the same slots
     auto low = [&](double* base, int v) -> float& { return *reinterpret_cast<float*>(base + v * stride); };
@@ -733,14 +762,16 @@ __device__ __forceinline__ void local_body_f64(const KParams<double>& P, const T
 #pragma unroll
       for (int v = 0; v < M; ++v) uf[v] = trunc_f32(s0[v * stride + tid]);
       auto nbf = [&](int v, int dir, int up) { return trunc_f32(nb(v, dir, up)); };
-      unclear = !hancock_states_f32<N, EQ>(m, phf, tb, uf, trunc_f32(alpha), p, q, trunc_f32(sHx[p]), trunc_f32(sHy[q]),
+      unclear = !hancock_states_f32<DIM, N, EQ>(m, phf, tb, uf, trunc_f32(alpha), p, q, trunc_f32(sHx[p]), trunc_f32(sHy[q]),
                                            nbf, xm, xp, ym, yp);
 #pragma unroll
       for (int v = 0; v < M; ++v) {
         low(sA + tid, v) = xm[v];
         low(sB + tid, v) = xp[v];
-        low(sC + tid, v) = ym[v];
-        low(sD + tid, v) = yp[v];
+        if (DIM == 2) {
+          low(sC + tid, v) = ym[v];
+          low(sD + tid, v) = yp[v];
+        }
       }
       if (unclear) sFull[el] = 1;  // the whole element goes to FP64
     }
@@ -752,7 +783,7 @@ __device__ __forceinline__ void local_body_f64(const KParams<double>& P, const T
     // NSF, its N n x-subfaces, then its n N y-subfaces; the flux right of (above)
     // node (p2, q2) overwrites that node's x+ (y+) state, which no other reads.
     // FP32 elements need only those next to the element faces.
-    constexpr int NSX = N * n, NSF = 2 * N * n;
+    constexpr int NSX = N * NFN, NSF = DIM * NSX;
     for (int gs = tid; gs < epr * NSF; gs += T) {
       const int el2 = gs / NSF, r = gs - el2 * NSF;
       const bool isx = r < NSX;
@@ -791,12 +822,14 @@ __device__ __forceinline__ void local_body_f64(const KParams<double>& P, const T
       if (p > 0) vld_sh<M, stride>(fl, sB + tid - 1);
       vsub(fr, fr, fl);
       vmul(LO, fr, sWx[p]);
+      if (DIM == 2) {
 #pragma unroll
-      for (int v = 0; v < M; ++v) fr[v] = fl[v] = 0.0;
-      if (q < N) vld_sh<M, stride>(fr, sD + tid);
-      if (q > 0) vld_sh<M, stride>(fl, sD + tid - n);
-      vsub(fr, fr, fl);
-      vfma(LO, sWy[q], fr);
+        for (int v = 0; v < M; ++v) fr[v] = fl[v] = 0.0;
+        if (q < N) vld_sh<M, stride>(fr, sD + tid);
+        if (q > 0) vld_sh<M, stride>(fl, sD + tid - n);
+        vsub(fr, fr, fl);
+        vfma(LO, sWy[q], fr);
+      }
 #pragma unroll
       for (int v = 0; v < M; ++v) {
         double* val = P.b.P + ((size_t)v * m.ne + e) * NP + k;
@@ -808,11 +841,11 @@ __device__ __forceinline__ void local_body_f64(const KParams<double>& P, const T
     const double hdt = 0.5 * dt;
 #pragma unroll
     for (int mm = 0; mm < SPT; ++mm) {
-      const FaceSlot fs = face_slot<NSLOT, n>(tid + mm * T);
+      const FaceSlot fs = face_slot<NSLOT, NFN>(tid + mm * T);
       const int eg = blk * epr + fs.el;
       if (fs.el < epr && eg < m.ne) {
         const int side = fs.side, j = fs.j, base = fs.el * NP;
-        const int nb_node = base + (side == 0 ? n * j : side == 1 ? N + n * j : side == 2 ? j : j + n * N);
+        const int nb_node = base + (DIM == 1 ? side * N : side == 0 ? n * j : side == 1 ? N + n * j : side == 2 ? j : j + n * N);
         const int adj_node = nb_node - (side == 1 ? 1 : side == 3 ? n : 0);
         double* ust = (side == 0 ? sA : side == 1 ? sB : side == 2 ? sC : sD) + nb_node;
         double* adj = (side < 2 ? sB : sD) + adj_node;
@@ -835,8 +868,8 @@ __device__ __forceinline__ void local_body_f64(const KParams<double>& P, const T
         }
 #pragma unroll
         for (int v = 0; v < M; ++v) {
-          P.b.slot[slot_index(1 + 2 * M + v, side, eg, j, 4, m.ne, n)] = us[v];
-          P.b.slot[slot_index(1 + 3 * M + v, side, eg, j, 4, m.ne, n)] = ub[v];
+          P.b.slot[slot_index(1 + 2 * M + v, side, eg, j, NSIDE, m.ne, NFN)] = us[v];
+          P.b.slot[slot_index(1 + 3 * M + v, side, eg, j, NSIDE, m.ne, NFN)] = ub[v];
         }
       }
     }

@@ -126,7 +126,7 @@ __device__ __forceinline__ bool flux_limiter_idle(const float* uL, const float* 
   // (pressures are differences of energies) and those times the speeds
   float SL = 0.0f, SR = 0.0f;
 #pragma unroll
-  for (int v = 3; v < M; ++v) {
+  for (int v = M == 3 ? 2 : 3; v < M; ++v) {
     SL += fabsf(uL[v]);
     SR += fabsf(uR[v]);
   }
@@ -136,7 +136,7 @@ __device__ __forceinline__ bool flux_limiter_idle(const float* uL, const float* 
   for (int v = 0; v < M; ++v) {
     lo[v] = 0.5f * (fL[v] + fR[v]) - 0.5f * lam * (uR[v] - uL[v]);
     const float a = fabsf(fL[v]) + fabsf(fR[v]) + lam * (fabsf(uL[v]) + fabsf(uR[v])) + fabsf(F[v]) +
-                    (v == 0 ? 0.0f : v < 3 ? S : S * V);
+                    (v == 0 ? 0.0f : v < (M == 3 ? 2 : 3) ? S : S * V);
     aL[v] = fabsf(bL[v]) + cL * a;
     aR[v] = fabsf(bR[v]) + cR * a;
   }
