@@ -67,17 +67,31 @@ struct Impl {
   static constexpr long long kSmallNodes = 152ll * 512;
   static bool small(const KParams<real>& P) { return kHasSmall && (long long)P.m.ne * NP < kSmallNodes; }
 
+  // Launch behind the previous kernel of the step (wait_for_previous_kernel).
+  template <class... A>
+  static cudaError_t chain(void (*kernel)(A...), int grid, int threads, size_t smem, cudaStream_t s, const A&... args) {
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3(grid);
+    cfg.blockDim = dim3(threads);
+    cfg.dynamicSmemBytes = smem;
+    cfg.stream = s;
+    cudaLaunchAttribute at[1];
+    at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    at[0].val.programmaticStreamSerializationAllowed = 1;
+    cfg.attrs = at;
+    cfg.numAttrs = 1;
+    return cudaLaunchKernelEx(&cfg, kernel, args...);
+  }
+
   template <int THREADS>
   static cudaError_t local_in(const KParams<real>& P, cudaStream_t s) {
     constexpr int E = BlockShape<NP, THREADS>::EPB;
-    k_local<DIM, N, EQ, real, MIXED, THREADS><<<(P.m.ne + E - 1) / E, E * NP, smem_local(E), s>>>(P);
-    return cudaGetLastError();
+    return chain(&k_local<DIM, N, EQ, real, MIXED, THREADS>, (P.m.ne + E - 1) / E, E * NP, smem_local(E), s, P);
   }
   template <int THREADS>
   static cudaError_t update_in(const KParams<real>& P, cudaStream_t s) {
     constexpr int E = UpdateShape<NP, MIXED, THREADS>::EPB;
-    k_update<DIM, N, EQ, real, MIXED, THREADS><<<(P.m.ne + E - 1) / E, E * NP, smem_update(E), s>>>(P);
-    return cudaGetLastError();
+    return chain(&k_update<DIM, N, EQ, real, MIXED, THREADS>, (P.m.ne + E - 1) / E, E * NP, smem_update(E), s, P);
   }
   static cudaError_t launch_local(const void* pv, cudaStream_t s) {
     const KParams<real>& P = *static_cast<const KParams<real>*>(pv);
@@ -90,8 +104,7 @@ struct Impl {
     const int nfaces = P.m.ny * P.m.nfx * NFN + (DIM == 2 ? P.m.nfy * P.m.nx * n : 0);
     // few face nodes: one warp per block, so that every SM has some
     const int threads = nfaces < 152 * 4 * 32 ? 32 : 256;
-    k_face<DIM, N, EQ, real><<<(nfaces + threads - 1) / threads, threads, 0, s>>>(P);
-    return cudaGetLastError();
+    return chain(&k_face<DIM, N, EQ, real>, (nfaces + threads - 1) / threads, threads, 0, s, P);
   }
   static cudaError_t launch_update(const void* pv, cudaStream_t s) {
     const KParams<real>& P = *static_cast<const KParams<real>*>(pv);
@@ -101,8 +114,7 @@ struct Impl {
   }
   static cudaError_t launch_finish(const void* pv, cudaStream_t s) {
     const KParams<real>& P = *static_cast<const KParams<real>*>(pv);
-    k_finish_step<<<1, 32, 0, s>>>(P.b.ctl);
-    return cudaGetLastError();
+    return chain(&k_finish_step, 1, 32, 0, s, P.b.ctl);
   }
   static cudaError_t step(const void* pv, cudaStream_t s) {
     cudaError_t e = launch_local(pv, s);
