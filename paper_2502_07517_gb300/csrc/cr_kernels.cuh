@@ -159,6 +159,16 @@ struct OpMin {
   __device__ T operator()(T a, T b) const { return fmin(a, b); }
 };
 
+// Minimum of doubles on the integer pipe (a comparison on the FP64 pipe costs 19 SM
+// cycles per warp and its latency in a chain): bit patterns ordered as the values.
+struct OpMinBits {
+  __device__ double operator()(double a, double b) const {
+    const long long x = __double_as_longlong(a), y = __double_as_longlong(b);
+    const long long m = 0x7fffffffffffffffll;
+    return (x ^ ((x >> 63) & m)) <= (y ^ ((y >> 63) & m)) ? a : b;
+  }
+};
+
 // ---------------------------------------------------------------------------
 // Arithmetic over the M variables of a point.  In FP32 the variables go two at
 // a time through Blackwell's packed FP32 instructions (FFMA2, FADD2, FMUL2: one
@@ -1663,6 +1673,113 @@ __device__ __forceinline__ double scaling_root(const double* ubar, const double*
   return lo;
 }
 
+// The scaling limiter (Sec. 3.2) of a block in which some point needs it, in FP64:
+// theta_1 for the density, theta_2 for the second constraint (scaling_root), per
+// element.  Called by every thread of the block; node values come and go in the
+// rows of the reduction buffer behind the first ([M] ur, FP32 bulk then [M] fl; only
+// elements with a failing point change and do FP64 work), means and limiter scalars
+// in sEl.  Out of line: most blocks never come here, and the update kernel keeps its
+// registers.
+template <int DIM, int N, class EQ, typename real, bool MIXED, int T>
+__device__ __noinline__ void limit_block(const KParams<real>& P, const Tab<double>& td, double* sU, double* sRed,
+                                         const double* sEl, int need, bool mean_ok, bool traces) {
+  constexpr int n = N + 1;
+  constexpr int NP = DIM == 2 ? n * n : n;
+  constexpr int M = EQ::M;
+  constexpr int NSIDE = DIM == 2 ? 4 : 2;
+  constexpr int NFN = DIM == 2 ? n : 1;
+  constexpr int NSLOT = NSIDE * NFN;
+  constexpr int SPT = (NSLOT + NP - 1) / NP;
+  constexpr int epb = (T + NP - 1) / NP, stride = epb * NP;
+  const int el = threadIdx.x / NP, k = threadIdx.x - el * NP;
+  real* X = reinterpret_cast<real*>(sRed + stride) + threadIdx.x;
+  const double eps1 = sEl[el * 16 + 1], eps2 = sEl[el * 16 + 2];
+  double ubar[M];
+#pragma unroll
+  for (int v = 0; v < M; ++v) ubar[v] = sEl[el * 16 + 4 + v];
+#define ATU(v, node) sU[(v) * stride + el * NP + (node)]
+#define RED(w) sRed[((w) * epb + el) * NP + k]
+#define RED0(w) sRed[((w) * epb + el) * NP]
+  // (the threads of elements without a failing point only take part in the barriers)
+  double pts[1 + SPT][M];
+  int np2 = 1;
+  __syncthreads();
+  RED(0) = need ? 0.0 : 1.0;
+  elem_reduce<NP, 1>(sRed, epb, el, k, OpMinBits());
+  const bool elem_need = RED0(0) == 0.0;
+  __syncthreads();
+  double rmin = 0.0;
+  if (elem_need) {
+#pragma unroll
+    for (int v = 0; v < M; ++v) {
+      if constexpr (MIXED) pts[0][v] = ubar[v] + double(X[(M + v) * stride]);
+      else pts[0][v] = double(X[v * stride]);
+      ATU(v, k) = pts[0][v];
+    }
+    rmin = pts[0][0];
+  }
+  __syncthreads();
+  if (elem_need && traces) {
+#pragma unroll
+    for (int mm = 0; mm < SPT; ++mm) {
+      const int sl = k + mm * NP;
+      if (sl < NSLOT) {
+        const int side = sl / NFN, j = sl - side * NFN;
+#pragma unroll
+        for (int v = 0; v < M; ++v) {
+          double acc = 0.0;
+#pragma unroll
+          for (int r = 0; r < n; ++r) {
+            const double l = (side & 1) ? td.l1[r] : td.l0[r];
+            acc += l * ATU(v, side < 2 ? r + n * j : j + n * r);
+          }
+          pts[np2][v] = acc;
+        }
+        rmin = OpMinBits()(rmin, pts[np2][0]);
+        ++np2;
+      }
+    }
+  }
+  RED(0) = rmin;
+  elem_reduce<NP, 1>(sRed, epb, el, k, OpMinBits());
+  rmin = RED0(0);
+  __syncthreads();
+  double tmin = 1.0;
+  if (elem_need && mean_ok) {
+    if (rmin < eps1) {
+      const double th1 = (ubar[0] - eps1) / (ubar[0] - rmin);
+      for (int t = 0; t < np2; ++t) pts[t][0] = ubar[0] + th1 * (pts[t][0] - ubar[0]);
+    }
+    for (int t = 0; t < np2; ++t) {
+      const double g1 = EQ::constraint(pts[t], 1, P.phd) - eps2;
+      if (g1 >= 0.0) continue;
+      const double lo = scaling_root<EQ>(ubar, pts[t], g1, eps2, P.phd);
+      tmin = OpMinBits()(tmin, lo);
+    }
+  }
+  RED(0) = tmin;
+  elem_reduce<NP, 1>(sRed, epb, el, k, OpMinBits());
+  const double th2 = RED0(0);
+  __syncthreads();
+  if (elem_need && th2 < 1.0) {
+#pragma unroll
+    for (int v = 0; v < M; ++v) pts[0][v] = ubar[v] + th2 * (pts[0][v] - ubar[v]);
+  }
+  // status tests only the mean (above): the limited points are admissible
+  // in exact arithmetic, and a tiny constraint value at a face trace is
+  // below the rounding of its interpolation
+  if (elem_need) {
+#pragma unroll
+    for (int v = 0; v < M; ++v) {
+      if constexpr (MIXED) X[(M + v) * stride] = real(pts[0][v] - ubar[v]);
+      X[v * stride] = real(pts[0][v]);
+    }
+  }
+#undef ATU
+#undef RED
+#undef RED0
+}
+
 // ===========================================================================
 // k_update.  Shared memory (doubles): sU [MU][epb][NP] node values, sRed
 // [RW][epb][NP] reduction buffer, sEl [epb][16] per-element values.
@@ -1989,76 +2106,96 @@ __device__ __forceinline__ void update_body(const KParams<real>& P, const Tab<re
     // with a failing point takes the FP64 result below: the others keep their
     // values bit for bit, whichever elements share their block.
     if (__syncthreads_or(valid && need)) {
-      // FP64 path (oracle's limiter): points in FP64
-      double pts[1 + SPT][M];
-      int np2 = 1;
-      __syncthreads();
-      RED(0) = need ? 0.0 : 1.0;
-      elem_reduce<NP, 1>(sRed, epb, el, k, OpMin());
-      const bool elem_need = RED0(0) == 0.0;
-      __syncthreads();
-#pragma unroll
-      for (int v = 0; v < M; ++v) {
-        if constexpr (MIXED) pts[0][v] = ubar[v] + double(fl[v]);
-        else pts[0][v] = double(ur[v]);
-      }
-#pragma unroll
-      for (int v = 0; v < M; ++v) ATU(v, k) = pts[0][v];
-      __syncthreads();
-      if (traces) {
-#pragma unroll
-        for (int mm = 0; mm < SPT; ++mm) {
-          const int sl = k + mm * NP;
-          if (sl < NSLOT) {
-            const int side = sl / NFN, j = sl - side * NFN;
-#pragma unroll
-            for (int v = 0; v < M; ++v) {
-              double acc = 0.0;
-#pragma unroll
-              for (int r = 0; r < n; ++r) {
-                const double l = (side & 1) ? td.l1[r] : td.l0[r];
-                acc += l * ATU(v, side < 2 ? r + n * j : j + n * r);
-              }
-              pts[np2][v] = acc;
-            }
-            ++np2;
-          }
-        }
-      }
-      double rmin = pts[0][0];
-      for (int t = 1; t < np2; ++t) rmin = fmin(rmin, pts[t][0]);
-      RED(0) = rmin;
-      elem_reduce<NP, 1>(sRed, epb, el, k, OpMin());
-      rmin = RED0(0);
-      __syncthreads();
-      if (mean_ok && rmin < eps1) {
-        const double th1 = (ubar[0] - eps1) / (ubar[0] - rmin);
-        for (int t = 0; t < np2; ++t) pts[t][0] = ubar[0] + th1 * (pts[t][0] - ubar[0]);
-      }
-      double tmin = 1.0;
-      if (mean_ok)
-        for (int t = 0; t < np2; ++t) {
-          const double g1 = EQ::constraint(pts[t], 1, P.phd) - eps2;
-          if (g1 >= 0.0) continue;
-          const double lo = scaling_root<EQ>(ubar, pts[t], g1, eps2, P.phd);
-          tmin = fmin(tmin, lo);
-        }
-      RED(0) = tmin;
-      elem_reduce<NP, 1>(sRed, epb, el, k, OpMin());
-      const double th2 = RED0(0);
-      __syncthreads();
-      if (th2 < 1.0)
-        for (int t = 0; t < np2; ++t)
-#pragma unroll
-          for (int v = 0; v < M; ++v) pts[t][v] = ubar[v] + th2 * (pts[t][v] - ubar[v]);
-      // status tests only the mean (above): the limited points are admissible
-      // in exact arithmetic, and a tiny constraint value at a face trace is
-      // below the rounding of its interpolation
-      if (elem_need) {
+      // (the limiter out of line: ten-moment FP32 bulk, 211 x 173 elements, k_update
+      // 0.123 -> 0.106 ms, FP64 256 x 256 0.254 -> 0.221; FP32-bulk Euler, where few
+      // blocks limit, keeps it inline: 0.305 against 0.315 ms at 512 x 512)
+      if constexpr (!MIXED || M == 6) {
+        // node values through the free rows of the reduction buffer, so that they
+        // can stay in registers here
+        real* X = reinterpret_cast<real*>(sRed + stride);
 #pragma unroll
         for (int v = 0; v < M; ++v) {
-          if constexpr (MIXED) fl[v] = real(pts[0][v] - ubar[v]);
-          ur[v] = real(pts[0][v]);
+          X[v * stride + tid] = ur[v];
+          if constexpr (MIXED) X[(M + v) * stride + tid] = fl[v];
+        }
+        limit_block<DIM, N, EQ, real, MIXED, T>(P, td, sU, sRed, sEl, need, mean_ok, traces);
+#pragma unroll
+        for (int v = 0; v < M; ++v) {
+          ur[v] = X[v * stride + tid];
+          if constexpr (MIXED) fl[v] = X[(M + v) * stride + tid];
+        }
+      } else {
+        // FP64 path (oracle's limiter): points in FP64
+        double pts[1 + SPT][M];
+        int np2 = 1;
+        __syncthreads();
+        RED(0) = need ? 0.0 : 1.0;
+        elem_reduce<NP, 1>(sRed, epb, el, k, OpMin());
+        const bool elem_need = RED0(0) == 0.0;
+        __syncthreads();
+#pragma unroll
+        for (int v = 0; v < M; ++v) {
+          if constexpr (MIXED) pts[0][v] = ubar[v] + double(fl[v]);
+          else pts[0][v] = double(ur[v]);
+        }
+#pragma unroll
+        for (int v = 0; v < M; ++v) ATU(v, k) = pts[0][v];
+        __syncthreads();
+        if (traces) {
+#pragma unroll
+          for (int mm = 0; mm < SPT; ++mm) {
+            const int sl = k + mm * NP;
+            if (sl < NSLOT) {
+              const int side = sl / NFN, j = sl - side * NFN;
+#pragma unroll
+              for (int v = 0; v < M; ++v) {
+                double acc = 0.0;
+#pragma unroll
+                for (int r = 0; r < n; ++r) {
+                  const double l = (side & 1) ? td.l1[r] : td.l0[r];
+                  acc += l * ATU(v, side < 2 ? r + n * j : j + n * r);
+                }
+                pts[np2][v] = acc;
+              }
+              ++np2;
+            }
+          }
+        }
+        double rmin = pts[0][0];
+        for (int t = 1; t < np2; ++t) rmin = fmin(rmin, pts[t][0]);
+        RED(0) = rmin;
+        elem_reduce<NP, 1>(sRed, epb, el, k, OpMin());
+        rmin = RED0(0);
+        __syncthreads();
+        if (mean_ok && rmin < eps1) {
+          const double th1 = (ubar[0] - eps1) / (ubar[0] - rmin);
+          for (int t = 0; t < np2; ++t) pts[t][0] = ubar[0] + th1 * (pts[t][0] - ubar[0]);
+        }
+        double tmin = 1.0;
+        if (mean_ok)
+          for (int t = 0; t < np2; ++t) {
+            const double g1 = EQ::constraint(pts[t], 1, P.phd) - eps2;
+            if (g1 >= 0.0) continue;
+            const double lo = scaling_root<EQ>(ubar, pts[t], g1, eps2, P.phd);
+            tmin = fmin(tmin, lo);
+          }
+        RED(0) = tmin;
+        elem_reduce<NP, 1>(sRed, epb, el, k, OpMin());
+        const double th2 = RED0(0);
+        __syncthreads();
+        if (th2 < 1.0)
+          for (int t = 0; t < np2; ++t)
+#pragma unroll
+            for (int v = 0; v < M; ++v) pts[t][v] = ubar[v] + th2 * (pts[t][v] - ubar[v]);
+        // status tests only the mean (above): the limited points are admissible
+        // in exact arithmetic, and a tiny constraint value at a face trace is
+        // below the rounding of its interpolation
+        if (elem_need) {
+#pragma unroll
+          for (int v = 0; v < M; ++v) {
+            if constexpr (MIXED) fl[v] = real(pts[0][v] - ubar[v]);
+            ur[v] = real(pts[0][v]);
+          }
         }
       }
     }
@@ -2140,8 +2277,15 @@ __device__ __forceinline__ void update_body(const KParams<real>& P, const Tab<re
 #undef RED0
 }
 
+// Resident blocks of the update kernel: FP64 in two dimensions five (48 registers,
+// 140 B of spills): with the screens it waits at barriers more than for the FP64
+// pipe, 0.600 ms at four, 0.564 at five (2D Euler N = 4, 512 x 512).
+template <int DIM, bool MIXED> struct UpdateBlocks {
+  static constexpr int value = DIM == 2 && !MIXED ? 5 : MinBlocks<MIXED>::update;
+};
+
 template <int DIM, int N, class EQ, typename real, bool MIXED, int THREADS = 256>
-__global__ void __launch_bounds__(THREADS, MinBlocks<MIXED>::update * (256 / THREADS)) k_update(const __grid_constant__ KParams<real> P) {
+__global__ void __launch_bounds__(THREADS, UpdateBlocks<DIM, MIXED>::value * (256 / THREADS)) k_update(const __grid_constant__ KParams<real> P) {
   wait_for_previous_kernel();
   update_body<DIM, N, EQ, real, MIXED, UpdateShape<DIM == 2 ? (N + 1) * (N + 1) : N + 1, MIXED, THREADS>::T>(
       P, P.tb, P.td, blockIdx.x, gridDim.x, true);  // k_finish_step ends the step
