@@ -32,7 +32,8 @@
 // -> 5.60 ms, traces and volume term on the integer pipe as well (251 FP64
 // instructions, 56% of the pipe, 28% of the issue slots: latency bound) -> 5.03
 // ms, the stage residuals in shared memory and a third resident block -> 4.51 ms,
-// neighbour data and tables loaded by all threads at once -> 4.35 ms; ten-moment
+// neighbour data and tables loaded by all threads at once -> 4.35 ms, the N = 4
+// stage sums in integers -> 4.15 ms; ten-moment
 // N = 3 at 256 x 256 2.61 -> 1.42 ms; 1D Euler N = 4, whole step, 4,000 elements 53
 // -> 49 us, 60,000 elements 314 -> 163 us.
 #pragma once
@@ -376,6 +377,21 @@ __device__ __noinline__ void exact_face_data(const KParams<double>& P, const Tab
   }
 }
 
+// Stage sums of the N = 4 method over residuals R_j in fixed point: sum_j a_ij R_j
+// = m_i sum_j c_ij R_j with small whole c_ij.  |R| stays below 2^61.4 (the rows of D
+// sum to at most 2.51 of its largest entry, Gauss-Legendre and Gauss-Lobatto), so
+// the sums of stages 1 to 3 (weights up to 3) fit 63 bits as they are; those of 4
+// and 5 (12 and 37) are taken 4 bits down.
+struct StageSums {
+  static __host__ __device__ constexpr int c(int i, int j) {
+    return i == 4 ? (j == 0 ? 3 : j == 3 ? 9 : 0)
+         : i == 5 ? (j == 0 ? -3 : j == 1 ? 2 : j == 2 ? 12 : j == 3 ? -12 : j == 4 ? 8 : 0) : 0;
+  }
+  static __host__ __device__ constexpr double m(int i) {
+    return i == 1 ? 0.25 : i == 2 ? 0.125 : i == 3 ? 0.5 : i == 4 ? 0.0625 : 1.0 / 7.0;
+  }
+};
+
 // Shared memory of the body beyond the five node arrays, in bytes.
 template <int DIM, int N, class EQ>
 __host__ __device__ constexpr size_t local64_extra(int epb) {
@@ -490,7 +506,9 @@ __device__ __forceinline__ void local_body_f64(const KParams<double>& P, const T
   for (int t = tid; t < 2 * n; t += T) tL[t] = P.ds.fL[t];
   // factors of the step and the node row
   for (int t = tid; t < S * S + 2 * n; t += T) {
-    if (t < S * S) {
+    if (t < S) {  // (row 0 of the tableau is empty: the factors of the integer sums)
+      sAdt[t] = N == 4 && t > 0 ? dt * StageSums::m(t) : 0.0;
+    } else if (t < S * S) {
       sAdt[t] = dt * TB::a(t / S, t % S);
     } else {
       const int r = t - S * S, pp = r % n;
@@ -523,6 +541,8 @@ __device__ __forceinline__ void local_body_f64(const KParams<double>& P, const T
 
   // ---------------- local cRK stages -----------------------------------
   double Lst[S > 1 ? S - 1 : 1][M];
+  constexpr bool kIntSums = N == 4 && !SRC;  // the residuals stay in fixed point
+  long long Rlast[M];                        // (the last one, in registers)
   double ea[SPT][M], Ut[SPT][M];
   long long ho[M];  // sum_i b_i (FR volume part of the stage fluxes), fixed point
 #pragma unroll
@@ -545,7 +565,8 @@ __device__ __forceinline__ void local_body_f64(const KParams<double>& P, const T
   // into the node arrays in fixed point, and a barrier.  An element keeps its
   // exponents from the first stage until a value needs two more bits; then
   // (rarely: the vote) it takes the larger ones.
-  auto put_nodes = [&](const double (&f)[M], const double (&g)[M], const double (&u)[M], bool first, bool traces) {
+  auto put_nodes = [&](const double (&f)[M], const double (&g)[M], const double (&u)[M], int i, bool traces) {
+    const bool first = i == 0;
     if (first) {
 #pragma unroll
       for (int v = 0; v < M; ++v) {
@@ -585,7 +606,14 @@ __device__ __forceinline__ void local_body_f64(const KParams<double>& P, const T
       __syncthreads();
       put_all();
 #pragma unroll
-      for (int v = 0; v < M; ++v) ho[v] >>= min(63, kf[v] - before[v]);
+      for (int v = 0; v < M; ++v) {
+        const int d = min(63, kf[v] - before[v]);
+        ho[v] >>= d;
+        if (kIntSums) {
+          for (int j = 0; j < i && j < 4; ++j)
+            reinterpret_cast<long long*>(j == 3 ? sD : sL + j * arr)[v * stride + tid] >>= d;
+        }
+      }
       __syncthreads();
     }
   };
@@ -605,11 +633,40 @@ __device__ __forceinline__ void local_body_f64(const KParams<double>& P, const T
     const bool traces = i == 0 || avg;
     double ui[M], f[M], g[M];
     vld_sh<M, stride>(ui, s0 + tid);
+    if (kIntSums && i > 0) {
+      // u^n - dt m_i sum_j c_ij R_j (StageSums): the sum is exact in integers, one
+      // FP64 instruction per variable
 #pragma unroll
-    for (int j = 0; j < i; ++j) {
-      if (TB::a(i, j) == 0.0) continue;
-      if (kShL && j < 4) vfma_sh<M, stride>(ui, -sAdt[i * S + j], (j == 3 ? sD : sL + j * arr) + tid);
-      else vfma(ui, -sAdt[i * S + j], Lst[j]);
+      for (int v = 0; v < M; ++v) {
+        auto R = [&](int j) {
+          return j == 4 ? Rlast[v] : reinterpret_cast<long long*>(j == 3 ? sD : sL + j * arr)[v * stride + tid];
+        };
+        constexpr int low = 4;  // of the sums that need headroom, the low bits are summed apart
+        long long sum = 0, rest = 0;
+        if (i == 1) sum = R(0);
+        if (i == 2) sum = R(0) + R(1);
+        if (i == 3) sum = 2 * R(2) - R(1);
+        if (i >= 4) {
+#pragma unroll
+          for (int j = 0; j < i; ++j) {
+            const int c = StageSums::c(i, j);
+            if (c == 0) continue;
+            const long long r = R(j);
+            sum += c * (r >> low);
+            rest += c * (r & ((1 << low) - 1));
+          }
+          sum += rest >> low;
+        }
+        const int E = kf[v];
+        ui[v] = E > kmax ? kNaN : fma(-sAdt[i], from_fixed(sum, E + (i >= 4 ? low : 0)), ui[v]);
+      }
+    } else {
+#pragma unroll
+      for (int j = 0; j < i; ++j) {
+        if (TB::a(i, j) == 0.0) continue;
+        if (kShL && j < 4) vfma_sh<M, stride>(ui, -sAdt[i * S + j], (j == 3 ? sD : sL + j * arr) + tid);
+        else vfma(ui, -sAdt[i * S + j], Lst[j]);
+      }
     }
     if (DIM == 2) EQ::flux_xy(ui, f, g, ph);
     else EQ::flux(ui, 0, f, ph);
@@ -623,7 +680,7 @@ __device__ __forceinline__ void local_body_f64(const KParams<double>& P, const T
         else if (avg) *sa = fma(TB::b(i), src[v], *sa);
       }
     }
-    if (i < S - 1 || avg) put_nodes(f, g, ui, i == 0, traces);
+    if (i < S - 1 || avg) put_nodes(f, g, ui, i, traces);
     // one pass over the two lines for the stage residual D f / dx + D g / dy and
     // the stage's part of the FR volume term (its matrices hold the factor b_i),
     // two variables at a time (one load of a coefficient for both)
@@ -658,6 +715,12 @@ __device__ __forceinline__ void local_body_f64(const KParams<double>& P, const T
         const int v = v0 + w;
         if (avg) ho[v] += fix_sum(hi[w]);
         if (i < S - 1) {
+          if (kIntSums) {
+            const long long r = fix_sum(lo[w]);
+            if (i == 4) Rlast[v] = r;
+            else reinterpret_cast<long long*>(i == 3 ? sD : sL + i * arr)[v * stride + tid] = r;
+            continue;
+          }
           const int E = kf[v];
           double L = E > kmax ? kNaN : from_fixed(fix_sum(lo[w]), E);
           if (kSrcEq && has_src) L -= src[v];
