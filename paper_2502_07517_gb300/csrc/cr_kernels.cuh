@@ -874,10 +874,8 @@ __device__ __forceinline__ void local_phase(const KParams<real>& P, const Tab<re
 // Resident blocks per SM the step kernels ask for (measured on GB300,
 // 2D Euler N = 4, 512x512): FP32_BULK blocks are latency bound and gain from
 // four 256-thread blocks per SM (64 registers; k_local 1.39 -> 1.05 ms,
-// k_update 0.91 -> 0.60 ms); the FP64 k_local takes two (in two dimensions
-// LocalBlocks); the FP64 k_update
-// is bound by its barriers and gains from more resident blocks: 2.15 ms at
-// one (106 registers), 1.91 at three (85), 1.75 at four (64).
+// k_update 0.91 -> 0.60 ms); FP64 k_local takes two and k_update four in one
+// dimension (in two: LocalBlocks, UpdateBlocks).
 template <bool MIXED> struct MinBlocks {
   static constexpr int local = MIXED ? 4 : 2, update = 4;
 };
@@ -885,17 +883,20 @@ template <bool MIXED> struct MinBlocks {
 // Threads per block of the single-problem step kernels: the whole elements
 // that fit in 256 threads (at least one); the FP32-bulk update kernel in 128
 // (barrier bound: smaller blocks wait less at each barrier, 0.482 -> 0.411 ms
-// at 512x512 N = 4; the FP64 update was slower so, 1.75 -> 1.88 ms).
+// at 512x512 N = 4; the FP64 update was slower so, 1.75 -> 1.88 ms before its
+// screens, and stays at 256).
 template <int NP, int THREADS = 256> struct BlockShape {
   static constexpr int EPB = (THREADS / NP) > 0 ? (THREADS / NP) : 1;
   static constexpr int T = EPB * NP;
 };
-template <int NP, bool MIXED, int THREADS = 256> using UpdateShape = BlockShape<NP, (MIXED && THREADS > 128 ? 128 : THREADS)>;
+template <int NP, bool MIXED, int THREADS = 256>
+using UpdateShape = BlockShape<NP, (MIXED && THREADS > 128 ? 128 : THREADS)>;
 
 // Blocks of the element kernel.  FP64 in two dimensions (cr_local64.cuh): three
 // resident blocks (80 registers) so that one block's integer phases overlap
 // another's FP64 phases: 4.91 ms at two, 4.51 at three, although the compiler
-// spills 0.7 kB per thread there (2D Euler N = 4, 512 x 512); blocks of 128
+// spills 0.7 kB per thread there (2D Euler N = 4, 512 x 512; 4.14 ms with the
+// integer stage sums, which came after these); blocks of 128
 // threads 4.84 ms (per-block tables and neighbours), of 352 4.44.  The ten-moment
 // equations (six variables) keep two.
 template <int DIM, class EQ, bool MIXED> struct LocalBlocks {
@@ -903,9 +904,11 @@ template <int DIM, class EQ, bool MIXED> struct LocalBlocks {
 };
 
 template <int DIM, int N, class EQ, typename real, bool MIXED, int THREADS = 256>
-__global__ void __launch_bounds__(THREADS, LocalBlocks<DIM, EQ, MIXED>::value * (256 / THREADS)) k_local(const __grid_constant__ KParams<real> P) {
+__global__ void __launch_bounds__(THREADS, LocalBlocks<DIM, EQ, MIXED>::value * (256 / THREADS))
+    k_local(const __grid_constant__ KParams<real> P) {
   wait_for_previous_kernel();
-  local_phase<DIM, N, EQ, real, MIXED, BlockShape<DIM == 2 ? (N + 1) * (N + 1) : N + 1, THREADS>::T>(P, P.tb, blockIdx.x);
+  local_phase<DIM, N, EQ, real, MIXED, BlockShape<DIM == 2 ? (N + 1) * (N + 1) : N + 1, THREADS>::T>(
+      P, P.tb, blockIdx.x);
 }
 
 // ===========================================================================
@@ -1303,8 +1306,8 @@ __device__ __forceinline__ void face_body(const KParams<real>& P, const int blk)
 }
 
 // Resident blocks per SM of the face kernel (measured at 512x512 N = 4): FP32
-// bulk 0.161 -> 0.108 ms at four (64 registers instead of 82), FP64 1.00 ->
-// 0.99 ms at three (85 instead of 96).
+// bulk 0.161 -> 0.108 ms at four (64 registers instead of 82), FP64 three (80;
+// 0.202 ms).
 template <int DIM, int N, class EQ, typename real>
 __global__ void __launch_bounds__(256, sizeof(real) == 4 ? 4 : 3) k_face(const __grid_constant__ KParams<real> P) {
   wait_for_previous_kernel();
@@ -1644,7 +1647,9 @@ __device__ __forceinline__ void rate_and_finish(const Mesh& m, const Phys<T>& ph
 // line, so 7 to 10 evaluations do what a bisection does in 50; the evaluations
 // were most of the update kernel on steep ten-moment data (FP32 bulk, 211 x 173
 // elements, N = 3: 293 -> 125 us with the shorter reciprocals and square roots
-// of the constraint).
+// of the constraint).  Both end where the rounding of P_2 decides its sign: against
+// 80-bit arithmetic, on 6,893 random 1D Euler segments, the mean error of theta is
+// 6.8e-16, a bisection's 8.4e-16.
 template <class EQ>
 __device__ __forceinline__ double scaling_root(const double* ubar, const double* pt, double g1, double eps,
                                                const Phys<double>& ph) {
@@ -2285,7 +2290,8 @@ template <int DIM, bool MIXED> struct UpdateBlocks {
 };
 
 template <int DIM, int N, class EQ, typename real, bool MIXED, int THREADS = 256>
-__global__ void __launch_bounds__(THREADS, UpdateBlocks<DIM, MIXED>::value * (256 / THREADS)) k_update(const __grid_constant__ KParams<real> P) {
+__global__ void __launch_bounds__(THREADS, UpdateBlocks<DIM, MIXED>::value * (256 / THREADS))
+    k_update(const __grid_constant__ KParams<real> P) {
   wait_for_previous_kernel();
   update_body<DIM, N, EQ, real, MIXED, UpdateShape<DIM == 2 ? (N + 1) * (N + 1) : N + 1, MIXED, THREADS>::T>(
       P, P.tb, P.td, blockIdx.x, gridDim.x, true);  // k_finish_step ends the step
@@ -2330,12 +2336,22 @@ __global__ void k_prologue(const __grid_constant__ KParams<real> P) {
         u[v] = double(P.b.u[gi]);
       }
     } else {
-      u[v] = double(P.b.u[gi]) + P.b.umean[(size_t)v * m.ne + ee];
+      u[v] = to_double(P.b.u[gi]) + P.b.umean[(size_t)v * m.ne + ee];
     }
-    if (!isfinite(u[v])) bad = kStInvalidInput;
+    if (!finite_bits(u[v])) bad = kStInvalidInput;
     sRed[(v * epb + el) * NP + k] = W * u[v];
   }
-  if (!admissible<EQ>(u, P.phd)) bad = kStInvalidInput;
+  {  // admissible, in FP64 where FP32 does not show it clearly (512 x 512, N = 4:
+     // 0.505 -> 0.354 ms, FP32 bulk 0.555 -> 0.404)
+    float s[M], A[M];
+#pragma unroll
+    for (int v = 0; v < M; ++v) {
+      s[v] = trunc_f32(u[v]);
+      A[v] = fabsf(s[v]);
+    }
+    if (!clearly_above_eps<EQ>(s, A, trunc_f32(P.phd.gm1)) && !admissible<EQ>(u, P.phd))
+      bad = kStInvalidInput;
+  }
   if (valid && bad) {
     atomicOr(&P.b.ctl->status, bad);
     atomicMin(&P.b.ctl->bad_elem, e);
@@ -2365,41 +2381,70 @@ __global__ void k_prologue(const __grid_constant__ KParams<real> P) {
                                        0, 0.0, 0, gridDim.x, P.td.xi);
 }
 
+// Rows (variable, element) per block of the two kernels below, and the stride of a
+// row in shared memory (odd, so that threads reading one row each hit all banks).
+constexpr int kRowsPerBlock = 128;
+template <int NP> struct RowStride { static constexpr int value = NP | 1; };
+
+// The block's rows of in [rows][NP] into shared memory, coalesced, and the mean sum_k
+// W_k x_k of row threadIdx.x, in node order (0 past the last row).
+template <int DIM, int N>
+__device__ __forceinline__ double row_mean(const double* __restrict__ in, int rows,
+                                           const Tab<double>& td, double* sx) {
+  constexpr int n = N + 1;
+  constexpr int NP = DIM == 2 ? n * n : n, RS = RowStride<NP>::value;
+  __shared__ double sw[NP];
+  const int first = blockIdx.x * kRowsPerBlock, cnt = min(kRowsPerBlock, rows - first);
+  const double* x = in + (size_t)first * NP;
+  if (threadIdx.x < NP) sw[threadIdx.x] = DIM == 2 ? td.w[threadIdx.x % n] * td.w[threadIdx.x / n] : td.w[threadIdx.x];
+  for (int t = threadIdx.x; t < cnt * NP; t += kRowsPerBlock) sx[(t / NP) * RS + t % NP] = x[t];
+  __syncthreads();
+  double mu = 0.0;
+  if (int(threadIdx.x) < cnt) {
+    const double* r = sx + threadIdx.x * RS;
+#pragma unroll
+    for (int kk = 0; kk < NP; ++kk) mu += sw[kk] * r[kk];
+  }
+  return mu;
+}
+
 // FP32_BULK state conversion: FP64 nodal values <-> FP64 mean + FP32 fluctuation.
+// Bound by the FP64 pipe (a conversion costs as much there as an FMA), so per value
+// one FMA and one addition: the weights' products once per block, the rounding to
+// FP32 on the bit pattern, the block's rows through shared memory.  512 x 512 elements
+// of N = 4, four variables: 0.159 ms, with a thread per row that formed each product
+// and converted 0.182.
 template <int DIM, int N, int M>
 __global__ void k_split_state(const double* __restrict__ in, float* __restrict__ fl,
                               double* __restrict__ mean, float* __restrict__ mean_f, int ne,
-                              Tab<double> td) {
+                              const __grid_constant__ Tab<double> td) {
   constexpr int n = N + 1;
-  constexpr int NP = DIM == 2 ? n * n : n;
-  const int idx = blockIdx.x * blockDim.x + threadIdx.x;  // one thread per (v, e)
-  if (idx >= M * ne) return;
-  const double* x = in + (size_t)idx * NP;
-  double mu = 0.0;
-  for (int kk = 0; kk < NP; ++kk) {
-    const int pp = DIM == 2 ? kk % n : kk, qq = DIM == 2 ? kk / n : 0;
-    mu += (DIM == 2 ? td.w[pp] * td.w[qq] : td.w[pp]) * x[kk];
+  constexpr int NP = DIM == 2 ? n * n : n, RS = RowStride<NP>::value;
+  __shared__ double sx[kRowsPerBlock * RS], sm[kRowsPerBlock];
+  const int rows = M * ne, first = blockIdx.x * kRowsPerBlock, cnt = min(kRowsPerBlock, rows - first);
+  const double mu = row_mean<DIM, N>(in, rows, td, sx);
+  sm[threadIdx.x] = mu;
+  if (int(threadIdx.x) < cnt) {
+    mean[first + threadIdx.x] = mu;
+    mean_f[first + threadIdx.x] = float(mu);
   }
-  mean[idx] = mu;
-  mean_f[idx] = float(mu);
-  for (int kk = 0; kk < NP; ++kk) fl[(size_t)idx * NP + kk] = float(x[kk] - mu);
+  __syncthreads();
+  float* out = fl + (size_t)first * NP;
+  for (int t = threadIdx.x; t < cnt * NP; t += kRowsPerBlock) {
+    const int r = t / NP;
+    out[t] = to_float(sx[r * RS + t - r * NP] - sm[r]);
+  }
 }
 
 // Element means sum_k W_k u_k of an FP64 state [M][Ne][Np] -> [M][Ne].
 template <int DIM, int N, int M>
 __global__ void k_element_means(const double* __restrict__ u, double* __restrict__ mean, int ne,
-                                Tab<double> td) {
-  constexpr int n = N + 1;
-  constexpr int NP = DIM == 2 ? n * n : n;
-  const int idx = blockIdx.x * blockDim.x + threadIdx.x;  // one thread per (v, e)
-  if (idx >= M * ne) return;
-  const double* x = u + (size_t)idx * NP;
-  double mu = 0.0;
-  for (int kk = 0; kk < NP; ++kk) {
-    const int pp = DIM == 2 ? kk % n : kk, qq = DIM == 2 ? kk / n : 0;
-    mu += (DIM == 2 ? td.w[pp] * td.w[qq] : td.w[pp]) * x[kk];
-  }
-  mean[idx] = mu;
+                                const __grid_constant__ Tab<double> td) {
+  constexpr int NP = DIM == 2 ? (N + 1) * (N + 1) : N + 1;
+  __shared__ double sx[kRowsPerBlock * RowStride<NP>::value];
+  const int row = blockIdx.x * kRowsPerBlock + threadIdx.x;
+  const double mu = row_mean<DIM, N>(u, M * ne, td, sx);
+  if (row < M * ne) mean[row] = mu;
 }
 
 template <int NP>

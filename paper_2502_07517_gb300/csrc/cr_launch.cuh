@@ -136,8 +136,8 @@ struct Impl {
     const size_t nvals = (size_t)M * P.m.ne * NP;
     if constexpr (MIXED) {
       const int nthr = M * P.m.ne;
-      k_split_state<DIM, N, M><<<(nthr + 255) / 256, 256, 0, s>>>(in, P.b.u, P.b.umean, P.b.umean_f,
-                                                                 P.m.ne, P.td);
+      k_split_state<DIM, N, M><<<(nthr + kRowsPerBlock - 1) / kRowsPerBlock, kRowsPerBlock, 0, s>>>(
+          in, P.b.u, P.b.umean, P.b.umean_f, P.m.ne, P.td);
       return cudaGetLastError();
     } else {
       return cudaMemcpyAsync(P.b.u, in, nvals * sizeof(double), cudaMemcpyDefault, s);
@@ -161,7 +161,8 @@ struct Impl {
       return cudaMemcpyAsync(out, P.b.umean, (size_t)M * P.m.ne * sizeof(double), cudaMemcpyDefault, s);
     } else {
       const int nthr = M * P.m.ne;
-      k_element_means<DIM, N, M><<<(nthr + 255) / 256, 256, 0, s>>>(P.b.u, out, P.m.ne, P.td);
+      k_element_means<DIM, N, M><<<(nthr + kRowsPerBlock - 1) / kRowsPerBlock, kRowsPerBlock, 0, s>>>(
+          P.b.u, out, P.m.ne, P.td);
       return cudaGetLastError();
     }
   }

@@ -35,6 +35,20 @@ __device__ __forceinline__ double widen_f32(float x) {
   return m < 0x00800000u ? __hiloint2double(int(b & 0x80000000u), 0)
                          : __hiloint2double(int(hi | (b & 0x80000000u)), int(b << 29));
 }
+// double(x), from the bit pattern in FP32's normal range and for 0.
+__device__ __forceinline__ double to_double(float x) {
+  const unsigned m = __float_as_uint(x) & 0x7fffffffu;
+  return m - 0x00800000u >= 0x7f000000u && m != 0u ? double(x) : widen_f32(x);
+}
+// float(x) (round to nearest, ties to even), on the bit pattern in FP32's normal
+// range and for 0.  A carry out of the largest exponent leaves infinity's pattern.
+__device__ __forceinline__ float to_float(double x) {
+  const unsigned long long b = (unsigned long long)__double_as_longlong(x), m = b & 0x7fffffffffffffffull;
+  const unsigned s = unsigned(b >> 32) & 0x80000000u;
+  if (unsigned(m >> 32) - 0x38100000u < 0x0fe00000u)
+    return __uint_as_float(s | (unsigned((m + 0x0fffffffull + ((m >> 29) & 1ull)) >> 29) - (896u << 23)));
+  return m == 0ull ? __uint_as_float(s) : float(x);
+}
 __device__ __forceinline__ float rcp_f32(float x) {
   float r;
   asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(x));
