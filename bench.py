@@ -38,9 +38,13 @@ MEASURED_PEAKS = os.path.join(ROOT, "MEASURED_PEAKS.json")
 SM_COUNT, SM_MAX_MHZ = 152, 2070.0
 # DRAM bytes (read + write) per element of the dominant kernel, from one ncu
 # capture of the current kernel at 384x384 (147,456 elements; the traffic
-# scales with the element count): FP64 k_local 589.5 MB, FP32 bulk k_local
-# 283.4 MB (the k_local summaries under profiles/).
-NCU_TRAFFIC_PER_ELEMENT = {("fp64", "k_local"): 589.46e6 / 147456, ("fp32", "k_local"): 283.41e6 / 147456}
+# scales with the element count): FP64 k_local 790.9 MB, FP32 bulk k_local
+# 276.1 MB (the k_local summaries under profiles/).
+NCU_TRAFFIC_PER_ELEMENT = {("fp64", "k_local"): 790.87e6 / 147456, ("fp32", "k_local"): 276.13e6 / 147456}
+# FP64 flops the FP64 kernel executes per solution point on the FP64 pipe (FMA 2),
+# from the same capture: the contractions run in fixed point on the integer pipe
+# and decisions in FP32, so the algorithmic count is not what the pipe does.
+NCU_FP64_FLOPS_PER_POINT = {"k_local": 345.5}
 PEAK_FP64_TFLOPS = SM_COUNT * 2 * 2 * SM_MAX_MHZ * 1e6 / 1e12
 PEAK_FP32_TFLOPS = SM_COUNT * 128 * 2 * SM_MAX_MHZ * 1e6 / 1e12
 
@@ -269,10 +273,10 @@ def train_alpha_network(degree, stream, seeds=range(1000, 1008), nx=96, snaps=(0
 
 
 def alu_roofline(prob, nodes, kms, mixed, ms_per_step):
-    """ALU roofline of the dominant kernel of a 2D Euler step: algorithmic
-    flops (flop_model) per launch over the kernel's CUDA-event time, against
-    the FP64 or FP32 peak; kms = per-kernel ms (k_local, k_face, k_update,
-    k_finish_step)."""
+    """ALU roofline of the dominant kernel of a 2D Euler step: flops per launch
+    over the kernel's CUDA-event time, against the FP64 or FP32 peak (FP32 bulk:
+    the algorithmic flops of flop_model; FP64: those executed on the FP64
+    pipe); kms = per-kernel ms (k_local, k_face, k_update, k_finish_step)."""
     names = ["k_local", "k_face", "k_update", "k_finish_step"]
     dom = int(np.argmax(kms[:3]))
     flops = flop_model(2, prob["degree"], "euler2d")
@@ -280,8 +284,14 @@ def alu_roofline(prob, nodes, kms, mixed, ms_per_step):
     peak = PEAK_FP32_TFLOPS if mixed else PEAK_FP64_TFLOPS
     mode = "fp32" if mixed else "fp64"
     ne = nodes // (prob["degree"] + 1) ** 2
+    executed = flops[dom] if mixed else NCU_FP64_FLOPS_PER_POINT.get(names[dom], flops[dom])
+    algorithmic, achieved = achieved, executed * nodes / (kms[dom] * 1e-3) / 1e12
     return {"bound": "alu", "achieved": achieved, "peak": peak, "unit": "TFLOP/s",
             "frac": achieved / peak, "kernel": names[dom],
+            "executed_flops_per_point": executed, "algorithmic_tflops": algorithmic,
+            "note": None if mixed else "achieved counts the flops executed on the FP64 pipe; the D contractions and "
+                    "traces run in fixed point on the integer pipe and screened decisions in FP32, so the "
+                    "algorithmic rate is not bounded by that pipe",
             "traffic": (NCU_TRAFFIC_PER_ELEMENT[(mode, names[dom])] * ne
                         if (mode, names[dom]) in NCU_TRAFFIC_PER_ELEMENT else None),
             "peak_source": "derived: 152 SMs x %s FMA lanes x 2 x 2070 MHz"
