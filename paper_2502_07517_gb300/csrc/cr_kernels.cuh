@@ -898,13 +898,20 @@ using UpdateShape = BlockShape<NP, (MIXED && THREADS > 128 ? 128 : THREADS)>;
 // spills 0.7 kB per thread there (2D Euler N = 4, 512 x 512; 4.14 ms with the
 // integer stage sums, which came after these); blocks of 128
 // threads 4.84 ms (per-block tables and neighbours), of 352 4.44.  The ten-moment
-// equations (six variables) keep two.
-template <int DIM, class EQ, bool MIXED> struct LocalBlocks {
+// equations (six variables) two.  The systems with N <= 3 hold fewer sums per thread:
+// where a mesh has more blocks than those fill the chip with, one block more per SM
+// (`many`): 2D Euler 256 x 256, N = 1, 2, 3: 105, 257, 472 -> 93, 242, 450 us, ten-moment N
+// = 2, 3: 765, 1,416 -> 753, 1,378; a mesh that fits at once gains nothing and pays
+// for the spills (40 x 40, N = 3: 50.0 -> 52.5), and so does N = 4 (4.17 -> 4.25 ms,
+// ten-moment 2.99 -> 3.12).
+template <int DIM, int N, class EQ, bool MIXED> struct LocalBlocks {
   static constexpr int value = DIM == 2 && !MIXED && EQ::M <= 4 ? 3 : MinBlocks<MIXED>::local;
+  static constexpr int many = DIM == 2 && !MIXED && EQ::M >= 4 && N <= 3 ? value + 1 : value;
 };
 
-template <int DIM, int N, class EQ, typename real, bool MIXED, int THREADS = 256>
-__global__ void __launch_bounds__(THREADS, LocalBlocks<DIM, EQ, MIXED>::value * (256 / THREADS))
+template <int DIM, int N, class EQ, typename real, bool MIXED, int THREADS = 256,
+          int BLOCKS = LocalBlocks<DIM, N, EQ, MIXED>::value>
+__global__ void __launch_bounds__(THREADS, BLOCKS * (256 / THREADS))
     k_local(const __grid_constant__ KParams<real> P) {
   wait_for_previous_kernel();
   local_phase<DIM, N, EQ, real, MIXED, BlockShape<DIM == 2 ? (N + 1) * (N + 1) : N + 1, THREADS>::T>(

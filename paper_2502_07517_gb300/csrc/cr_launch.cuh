@@ -25,6 +25,7 @@ struct Impl {
   static constexpr int NP = DIM == 2 ? n * n : n;
   static constexpr int M = EQ::M;
   static constexpr int NFN = DIM == 2 ? n : 1;
+  using LB = LocalBlocks<DIM, N, EQ, MIXED>;
   // variables per node in the element kernel's shared arrays (VarPack pads FP32 to pairs)
   static constexpr int MV = (M + VarPack<real>::VL - 1) / VarPack<real>::VL * VarPack<real>::VL;
 
@@ -50,6 +51,11 @@ struct Impl {
     err = cudaFuncSetAttribute(k_local<DIM, N, EQ, real, MIXED>,
                                cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem_local(EPB));
     if (err != cudaSuccess) return err;
+    if constexpr (LB::many > LB::value) {
+      err = cudaFuncSetAttribute(k_local<DIM, N, EQ, real, MIXED, 256, LB::many>,
+                                 cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem_local(EPB));
+      if (err != cudaSuccess) return err;
+    }
     err = cudaFuncSetAttribute(k_update<DIM, N, EQ, real, MIXED>,
                                cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem_update(EPB));
     if (err != cudaSuccess) return err;
@@ -86,7 +92,11 @@ struct Impl {
   template <int THREADS>
   static cudaError_t local_in(const KParams<real>& P, cudaStream_t s) {
     constexpr int E = BlockShape<NP, THREADS>::EPB;
-    return chain(&k_local<DIM, N, EQ, real, MIXED, THREADS>, (P.m.ne + E - 1) / E, E * NP, smem_local(E), s, P);
+    const int blocks = (P.m.ne + E - 1) / E;
+    if constexpr (LB::many > LB::value)  // more blocks than are resident at once: one more per SM
+      if (blocks > 152 * LB::value)
+        return chain(&k_local<DIM, N, EQ, real, MIXED, THREADS, LB::many>, blocks, E * NP, smem_local(E), s, P);
+    return chain(&k_local<DIM, N, EQ, real, MIXED, THREADS>, blocks, E * NP, smem_local(E), s, P);
   }
   template <int THREADS>
   static cudaError_t update_in(const KParams<real>& P, cudaStream_t s) {

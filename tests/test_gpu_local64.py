@@ -107,6 +107,22 @@ def test_low_pressure_beside_the_screens(N, pressure):
     assert_parity(g, ref, rtol=bar, extra_scale=flux_increment(prob, dg, dt))
 
 
+@pytest.mark.parametrize("eq,N,nx,ny", [("euler", 1, 171, 170), ("euler", 1, 171, 171), ("euler", 2, 113, 112),
+                                        ("euler", 2, 113, 114), ("euler", 3, 86, 84), ("euler", 3, 86, 85),
+                                        ("tenmoment", 3, 70, 69), ("tenmoment", 3, 70, 70)])
+def test_meshes_about_the_resident_blocks(eq, N, nx, ny):
+    """Meshes that just fit on the chip at once and that just do not (the element
+    kernel then asks for one block more per SM)."""
+    make = wl.euler2d_vortex if eq == "euler" else wl.tenmoment2d_voronoi
+    prob, u = make(nx=nx, ny=ny, degree=N, seed=N)
+    d = oracle_desc(prob)
+    dt = 0.5 * oracle.dt(d, u)
+    ref, st, dg = oracle.step(d, u, dt, want_diag=True)
+    assert st == 0
+    g = gpu_run(prob, u, dt_fixed=dt)[0]
+    assert_parity(g, ref, extra_scale=flux_increment(prob, dg, dt))
+
+
 @pytest.mark.parametrize("N", [2, 3, 4])
 def test_alpha_beside_its_threshold(N):
     """Elements whose modal energy fraction lies within a few percent of the one
