@@ -34,7 +34,7 @@
 // ms, the stage residuals in shared memory and a third resident block -> 4.51 ms,
 // neighbour data and tables loaded by all threads at once -> 4.35 ms, the N = 4
 // stage sums in integers -> 4.15 ms; ten-moment
-// N = 3 at 256 x 256 2.61 -> 1.42 ms; 1D Euler N = 4, whole step, 4,000 elements 53
+// N = 3 at 256 x 256 2.61 -> 1.42 ms (1.38 with a third resident block); 1D Euler N = 4, whole step, 4,000 elements 53
 // -> 49 us, 60,000 elements 314 -> 163 us.
 #pragma once
 #include "cr_common.cuh"
