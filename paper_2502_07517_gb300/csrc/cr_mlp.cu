@@ -607,19 +607,35 @@ cr_status cr_mlp_train(int nin, float* params, const float* X, const float* t, i
     ok(cudaMemsetAsync(mom, 0, sizeof(float) * P, s));
     ok(cudaMemsetAsync(var, 0, sizeof(float) * P, s));
   }
-  std::vector<int> perm;
-  std::vector<float2> corr;
+  // The host arrays of an epoch (sample order, bias corrections) are read by copies
+  // that may still be queued behind earlier epochs' kernels when the call returns to
+  // the host, so an epoch writes the pair that the last one did not use, once the
+  // event behind that pair's own copies has passed.  The next order is drawn while
+  // the device runs, and no epoch waits for the one before it.
+  struct HostEpoch {
+    std::vector<int> perm;
+    std::vector<float2> corr;
+    cudaEvent_t copied = nullptr;
+    ~HostEpoch() {
+      if (copied) cudaEventDestroy(copied);
+    }
+  } host[2];
   try {
-    perm.resize(n);
-    if (by_epoch) corr.resize(nb);
+    for (HostEpoch& h : host) {
+      h.perm.resize(n);
+      if (by_epoch) h.corr.resize(nb);
+    }
   } catch (const std::bad_alloc&) {
     st = CR_E_NOMEM;
   }
+  for (HostEpoch& h : host)
+    if (st == CR_OK) ok(cudaEventCreateWithFlags(&h.copied, cudaEventDisableTiming));
   uint64_t rs = seed;
   int step = 0;
   for (int ep = 0; ep < epochs && st == CR_OK; ++ep) {
-    // (the order of the next epoch is drawn while the device runs this one: no
-    // epoch waits for another on the host)
+    HostEpoch& h = host[ep & 1];
+    if (ep >= 2 && !ok(cudaEventSynchronize(h.copied))) break;
+    int* perm = h.perm.data();
     for (int i = 0; i < n; ++i) perm[i] = i;
     for (int i = n - 1; i > 0; --i) {  // Fisher-Yates with a seeded splitmix64
       const int j = int(splitmix64(&rs) % uint64_t(i + 1));
@@ -627,18 +643,21 @@ cr_status cr_mlp_train(int nin, float* params, const float* X, const float* t, i
       perm[i] = perm[j];
       perm[j] = tmp;
     }
-    ok(cudaMemcpyAsync(idx, perm.data(), sizeof(int) * n, cudaMemcpyHostToDevice, s));
+    ok(cudaMemcpyAsync(idx, perm, sizeof(int) * n, cudaMemcpyHostToDevice, s));
     if (by_epoch) {
+      float2* corr = h.corr.data();
       for (int k = 0; k < nb; ++k) {
         ++step;
         corr[k].x = 1.0f - powf(0.9f, float(step));
         corr[k].y = 1.0f - powf(0.999f, float(step));
       }
       float2* dcorr = reinterpret_cast<float2*>(mem + o_corr);
-      ok(cudaMemcpyAsync(dcorr, corr.data(), sizeof(float2) * nb, cudaMemcpyHostToDevice, s));
+      ok(cudaMemcpyAsync(dcorr, corr, sizeof(float2) * nb, cudaMemcpyHostToDevice, s));
+      if (st == CR_OK) ok(cudaEventRecord(h.copied, s));
       if (st == CR_OK) ok(dispatch_epoch(nin, params, mom, var, X, t, idx, n, most, dcorr, lr, el, s));
       continue;
     }
+    if (st == CR_OK) ok(cudaEventRecord(h.copied, s));
     ok(cudaMemsetAsync(el, 0, sizeof(float), s));
     float* grad = at(o_grad);
     for (int b0 = 0; b0 < n && st == CR_OK; b0 += batch) {
