@@ -515,7 +515,11 @@ cudaError_t launch_epoch(float* prm, float* mom, float* var, const float* X, con
   int C = 1;
   while (C < kMaxCluster && C < chunks) C *= 2;
   const size_t smem = EpochShape<NIN>::smem((chunks + C - 1) / C);
-  cudaError_t e = cudaFuncSetAttribute(k_mlp_epoch<NIN>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+  // the limit belongs to the kernel, not to the call: every call sets the one of the
+  // largest minibatch, so that calls of several threads do not lower each other's
+  constexpr int kMost = (kEpochBlocks + kMaxCluster - 1) / kMaxCluster;
+  cudaError_t e = cudaFuncSetAttribute(k_mlp_epoch<NIN>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                       (int)EpochShape<NIN>::smem(kMost));
   if (e != cudaSuccess) return e;
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = dim3(C);

@@ -1,11 +1,13 @@
 """cr_mlp_train under the conditions of a training program: long sample orders over
-several epochs, also behind other work on the stream.
+several epochs, also behind other work on the stream, and two threads at once.
 
-Tolerance: as in tests/test_gpu_mlp_train.py an Adam step differs by
+Tolerance of the first: as in tests/test_gpu_mlp_train.py an Adam step differs by
 at most 3e-3 * 1e-4 from the FP64 one; over K steps on parameters of standard
 deviation 0.2 that is K * 1.5e-6 of their 2-norm, and a mixed-up order moves them by
 far more.
 """
+import threading
+
 import numpy as np
 import pytest
 
@@ -57,3 +59,38 @@ def test_orders_of_several_epochs(behind):
     off = np.linalg.norm(got.cpu().numpy().astype(np.float64) - q) / np.linalg.norm(q)
     assert off <= 1.5e-6 * k, off
     assert abs(loss - np.mean(losses)) <= 1e-5 * np.mean(losses)
+
+
+def test_two_threads():
+    """Calls with small and large minibatches at once (they need different amounts of
+    shared memory) give what each gives alone."""
+    import torch
+    nin, n = 25, 3000
+    rng = np.random.default_rng(1)
+    p = rng.normal(0.0, 0.2, mlp.param_count(nin)).astype(np.float32)
+    X = torch.from_numpy(rng.uniform(0.0, 1.0, (n, nin)).astype(np.float32)).cuda()
+    t = torch.from_numpy(rng.uniform(0.0, 1.0, n).astype(np.float32)).cuda()
+    one = {b: torch.from_numpy(p).cuda() for b in (64, 3000)}
+    for b, q in one.items():
+        crkfr.cr_mlp_train(nin, q, X[:n if b > 64 else 64], t[:n if b > 64 else 64], batch=b, epochs=1, lr=3e-3, seed=3)
+    errors = []
+
+    def work(b):
+        try:
+            stream = torch.cuda.Stream()
+            m = n if b > 64 else 64
+            for _ in range(150):
+                q = torch.from_numpy(p).cuda()
+                torch.cuda.synchronize()
+                crkfr.cr_mlp_train(nin, q, X[:m], t[:m], batch=b, epochs=1, lr=3e-3, seed=3, stream=stream.cuda_stream)
+                if not torch.equal(q, one[b]):
+                    raise AssertionError("different parameters at batch %d" % b)
+        except Exception as e:          # noqa: BLE001
+            errors.append(repr(e))
+
+    threads = [threading.Thread(target=work, args=(b,)) for b in (64, 3000, 64, 3000)]
+    for th in threads:
+        th.start()
+    for th in threads:
+        th.join()
+    assert not errors, errors[:3]

@@ -1,7 +1,8 @@
 """Host side of cr_mlp_train against a stand-in for the CUDA runtime whose stream
 runs nothing before it has to: every copy reads its host memory as late as the
 runtime may (at the next wait for it).  The sample orders and bias corrections that
-the epochs then see must be those of the seed.
+the epochs then see must be those of the seed.  It also sees the kernel's shared
+memory limit and each launch's need.
 """
 import json
 import os
@@ -114,3 +115,14 @@ def test_every_epoch_sees_its_own_order(call, n, batch, epochs):
         want = [1.0 - 0.9 ** (step + 1 + k) for k in range(len(e["corr"]))]
         np.testing.assert_allclose(e["corr"], want, rtol=1e-5)
         step += len(want)
+
+
+def test_shared_memory_limit_is_the_same_for_every_call(call):
+    """The limit is a property of the kernel: a call that set a lower one between
+    another thread's limit and launch would make that launch fail."""
+    limits, needs = set(), []
+    for n, batch in ((10, 1), (700, 64), (700, 700), (3072, 3072)):
+        out = call(n, batch, 1, 3)
+        limits |= {e["limit"] for e in out if "limit" in e}
+        needs += [e["smem"] for e in out if "smem" in e]
+    assert len(limits) == 1 and max(needs) <= min(limits)
