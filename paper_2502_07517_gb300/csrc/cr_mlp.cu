@@ -230,6 +230,16 @@ constexpr int kHS = kH + 4;                              // row stride of the hi
                                                          // of 8 rows hit all banks: 4 x odd)
 constexpr int x_stride(int nin) { return 4 * (((nin + 3) / 4) | 1); }
 
+// Samples of chunk c of minibatch k (k batch < n; batch and c kChunk stay in the int
+// range, (k + 1) batch need not).
+__host__ __device__ constexpr int chunk_samples(int n, int batch, int k, int c) {
+  const int total = batch < n - k * batch ? batch : n - k * batch;
+  return total - c * kChunk < kChunk ? total - c * kChunk : kChunk;
+}
+static_assert(chunk_samples(2147483647, 3072, 699050, 0) == kChunk && chunk_samples(2147483647, 3072, 699050, 31) == 63 &&
+                  chunk_samples(700, 512, 1, 2) == 60,
+              "the last minibatch of the largest sample count");
+
 template <int NIN> struct EpochShape {
   static constexpr int P = param_count(NIN), XS = x_stride(NIN);
   static constexpr int PER = (kChunk * NIN + kEpochThreads - 1) / kEpochThreads;
@@ -284,7 +294,7 @@ __global__ void __launch_bounds__(kEpochThreads, 1)
   float rx[PER], rt = 0.0f;
   auto fetch = [&](int k, int c) {
     const int base = k * batch + c * kChunk;
-    const int cnt = min(kChunk, min(n, (k + 1) * batch) - base);
+    const int cnt = chunk_samples(n, batch, k, c);
 #pragma unroll
     for (int r = 0; r < PER; ++r) {
       const int t = tid + r * kEpochThreads, s = t / NIN;
