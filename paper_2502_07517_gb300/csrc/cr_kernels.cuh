@@ -1485,7 +1485,10 @@ __device__ T indicator_alpha(const Mesh& m, const Tab<T>& tb, T* E, T* Tm, T* re
 // the logistic reaches 1e-3 (Mesh::ind_zero is 0.97 of its square root).  A mode's
 // FP32 error is below (2i+1)(2j+1) 3.2e-6 of the weighted mean of the magnitudes
 // the indicator variable is formed from (S), its norm over the top modes below
-// 5e-4 of that mean.  Smooth elements so need none of the FP64 transform, sums
+// 5e-4 of that mean.  Energies below 2^-126 count as 0 here and those above 2^128 as
+// infinite, so nothing is clear unless the norm the top modes are compared with is
+// above 1e-15 (which a flushed energy, 2^-63 in the norm, does not touch) and the
+// total below 1e18.  Smooth elements so need none of the FP64 transform, sums
 // and logistic (k_update 1.50 -> 0.60 ms at 512 x 512 N = 4 with the limiter's
 // points screened likewise).  Called by every thread; buf: shared memory for 7
 // epb NP floats.
@@ -1533,7 +1536,8 @@ __device__ bool indicator_clear(const Mesh& m, const Tab<double>& td, const Phys
     const float d = 5e-4f * red[(4 * epb + el) * NP];
     const float tot = sqrt_f32(red[(0 * epb + el) * NP]), top = sqrt_f32(red[(1 * epb + el) * NP]);
     const float low = sqrt_f32(red[(2 * epb + el) * NP]), top1 = sqrt_f32(red[(3 * epb + el) * NP]);
-    unclear = !(top + d < m.ind_zero * (tot - d)) || !(N < 2 || top1 + d < m.ind_zero * (low - d));
+    const float most = m.ind_zero * (tot - d), most1 = m.ind_zero * (low - d);
+    unclear = !(tot < 1e18f && most > 1e-15f && top + d < most) || !(N < 2 || (most1 > 1e-15f && top1 + d < most1));
   }
   return !__syncthreads_or(unclear);
 }

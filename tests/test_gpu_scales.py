@@ -1,0 +1,72 @@
+"""Data far from 1: states scaled by powers of ten, where the comparisons that the
+FP64 kernels first make in FP32 leave FP32's range, against the oracle.
+
+The smoothness indicator's alpha is compared to 1e-9: at its threshold
+it changes by s / T = 1e4 times the change of an energy fraction, whose rounding is
+a few 1e-16 times the number of modes, and the tiny steps taken move the state by
+1e-13.
+"""
+import numpy as np
+import pytest
+
+import oracle
+from paper_2502_07517_gb300 import crkfr
+from paper_2502_07517_gb300 import workloads as wl
+from tests._oracle_util import oracle_desc
+from tests.test_gpu_parity import gpu_run
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture(scope="module", autouse=True)
+def _built():
+    import torch
+    if not torch.cuda.is_available():
+        pytest.skip("no CUDA device")
+    from paper_2502_07517_gb300 import build
+    build.build()
+
+
+def _modes(prob, cells, lo, hi, seed):
+    """1 + c L_N(x), the energy fraction of the top mode between lo and hi."""
+    N, rng = prob["degree"], np.random.default_rng(seed)
+    top = np.polynomial.legendre.Legendre.basis(N)(2.0 * wl.gl_nodes01(N)[0] - 1.0)
+    frac = np.exp(rng.uniform(np.log(lo), np.log(hi), cells))
+    c = np.sqrt(frac / (1.0 - frac))[:, None]
+    return 1.0 + c * np.tile(top, (N + 1) ** (prob["dim"] - 1))[None, :]
+
+
+def _check_alpha(prob, u, precisions=(crkfr.CR_FP64,)):
+    d = oracle_desc(prob)
+    dt = 1e-13 * oracle.dt(d, u)
+    dg = oracle.step(d, u, dt, want_diag=True)[2]
+    assert 0 < np.count_nonzero(dg["alpha_raw"])
+    for precision in precisions:
+        for steps in (1, 2):          # alpha from the input, then from the update
+            alpha = gpu_run(prob, u, dt_fixed=dt, nsteps=steps, precision=precision)[1]
+            if precision == crkfr.CR_FP64:
+                np.testing.assert_allclose(alpha, dg["alpha"], rtol=0, atol=1e-9)
+            elif steps == 1:
+                np.testing.assert_allclose(alpha, dg["alpha"], rtol=0, atol=1e-5)
+
+
+@pytest.mark.parametrize("N", [3, 4])
+@pytest.mark.parametrize("rho_p", [1e-22, 1e-20, 1e-18, 1e-17, 1e-16, 1e-10, 1.0, 1e10, 1e17, 3e19, 1e20, 1e21, 1e23])
+def test_indicator_of_scaled_states(N, rho_p):
+    prob, u = wl.euler2d_vortex(nx=16, ny=8, degree=N, seed=N, perturb=0.0)
+    prob = dict(prob, limiter=frozenset({"blend"}))
+    edge = 0.5 * 10.0 ** (-1.8 * (N + 1.0) ** 0.25) * 0.25
+    s = np.sqrt(rho_p)
+    p = s * _modes(prob, u.shape[1], 0.3 * edge, 8.0 * edge, N)
+    rho = s * np.ones_like(p)
+    _check_alpha(prob, wl.euler_conservative(rho, 0.1 * np.ones_like(p), 0.0 * p, p, 1.4, 2),
+                 (crkfr.CR_FP64, crkfr.CR_FP32_BULK) if 1e-10 <= rho_p <= 1e10 else (crkfr.CR_FP64,))
+
+
+@pytest.mark.parametrize("dim", [1, 2])
+@pytest.mark.parametrize("size", [1e-25, 1e-19, 1e-18, 1e-17, 1e-3, 1e18, 3e19, 1e20, 1e22])
+def test_indicator_of_scaled_scalars(dim, size):
+    prob, u = wl.linadv_random(nx=24, ny=9, dim=dim, degree=4, seed=1, adv=(0.7, -0.4))
+    prob = dict(prob, limiter=frozenset({"blend"}))
+    edge = 0.5 * 10.0 ** (-1.8 * 5.0 ** 0.25) * 0.25
+    _check_alpha(prob, size * _modes(prob, u.shape[1], 0.3 * edge, 8.0 * edge, dim)[None])
