@@ -30,28 +30,6 @@ __device__ __forceinline__ int neighbour(const Mesh& m, int e, int f) {
   return iy < m.ny - 1 ? e + m.nx : (m.bcy == 0 ? e - m.nx * (m.ny - 1) : -1);
 }
 
-// minmod of three slopes: the one of smallest magnitude when all three share a
-// nonzero sign, else 0.
-__device__ __forceinline__ float minmod3(float a, float b, float c) {
-  if (a > 0.0f && b > 0.0f && c > 0.0f) return fminf(a, fminf(b, c));
-  if (a < 0.0f && b < 0.0f && c < 0.0f) return fmaxf(a, fmaxf(b, c));
-  return 0.0f;
-}
-// FP64 version on the bit patterns (integer pipe; the FP64 pipe is the scarce
-// unit): sign bits must agree and no magnitude may be zero; for finite numbers
-// of one sign the order of the magnitude bits is the order of the magnitudes.
-__device__ __forceinline__ double minmod3(double a, double b, double c) {
-  const unsigned long long ia = (unsigned long long)__double_as_longlong(a);
-  const unsigned long long ib = (unsigned long long)__double_as_longlong(b);
-  const unsigned long long ic = (unsigned long long)__double_as_longlong(c);
-  const unsigned long long mag = 0x7fffffffffffffffull;
-  const unsigned long long ma = ia & mag, mb = ib & mag, mc = ic & mag;
-  if (((ia ^ ib) | (ia ^ ic)) >> 63 || ma == 0ull || mb == 0ull || mc == 0ull) return 0.0;
-  unsigned long long mm = ma < mb ? ma : mb;
-  mm = mm < mc ? mm : mc;
-  return __longlong_as_double((long long)(mm | (ia & ~mag)));
-}
-
 // All admissibility constraints P_k > 0, evaluated exactly (Sec. 2 eq. (uad.form)).
 template <class EQ, typename real>
 __device__ __forceinline__ bool admissible(const real* u, const Phys<real>& ph) {

@@ -43,18 +43,6 @@
 
 namespace crk {
 
-// minmod of the slopes d1 b1, d2 b2, d3 b3 (b > 0) with f1, f2, f3 = b in FP32.
-__device__ __forceinline__ double minmod_scaled(double d1, double d2, double d3, double b1, double b2,
-                                                double b3, float f1, float f2, float f3) {
-  const long long i1 = __double_as_longlong(d1), i2 = __double_as_longlong(d2), i3 = __double_as_longlong(d3);
-  if (((i1 ^ i2) | (i1 ^ i3)) < 0 || (i1 << 1) == 0 || (i2 << 1) == 0 || (i3 << 1) == 0) return 0.0;
-  const float m1 = fabsf(trunc_f32(d1)) * f1, m2 = fabsf(trunc_f32(d2)) * f2, m3 = fabsf(trunc_f32(d3)) * f3;
-  const float lim = fminf(m1, fminf(m2, m3)) * (1.0f + kTieF);
-  const bool c1 = m1 <= lim, c2 = m2 <= lim, c3 = m3 <= lim;
-  if (int(c1) + int(c2) + int(c3) != 1) return minmod3(d1 * b1, d2 * b2, d3 * b3);
-  return (c1 ? d1 : (c2 ? d2 : d3)) * (c1 ? b1 : (c2 ? b2 : b3));
-}
-
 // Flux in direction dir with the normal velocity and the squared sound speed
 // (the wave speed is |vn| + sqrt(c2)); equations without one: vn = the speed.
 template <class EQ>

@@ -16,6 +16,11 @@ constexpr float kTieF = 1.9073486e-6f;  // 2^-19
 // from: ten times the FP32 rounding of those sums and products.
 constexpr float kMarginF = 2e-5f;
 
+// Magnitudes between which FP32 comparisons of truncated FP64 numbers hold: below
+// 2^-126 a truncated number keeps stray bits, and products of two numbers, or of one
+// and a mesh factor, stay far from both ends of FP32's range.
+constexpr float kTinyF = 1e-30f, kHugeF = 1e30f;
+
 // x as FP32, truncated, from the bit pattern (a conversion instruction runs on
 // the FP64 pipe): magnitudes below FP32's normal range give a value below
 // 2^-126, larger ones its largest finite value; NaN gives a large value.
@@ -62,6 +67,43 @@ __device__ __forceinline__ float sqrt_f32(float x) {
   float r;
   asm("sqrt.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(fmaxf(x, 0.0f)));
   return r;
+}
+
+// minmod of three slopes: the one of smallest magnitude when all three share a
+// nonzero sign, else 0.
+__device__ __forceinline__ float minmod3(float a, float b, float c) {
+  if (a > 0.0f && b > 0.0f && c > 0.0f) return fminf(a, fminf(b, c));
+  if (a < 0.0f && b < 0.0f && c < 0.0f) return fmaxf(a, fmaxf(b, c));
+  return 0.0f;
+}
+// FP64 version on the bit patterns (integer pipe; the FP64 pipe is the scarce
+// unit): sign bits must agree and no magnitude may be zero; for finite numbers
+// of one sign the order of the magnitude bits is the order of the magnitudes.
+__device__ __forceinline__ double minmod3(double a, double b, double c) {
+  const unsigned long long ia = (unsigned long long)__double_as_longlong(a);
+  const unsigned long long ib = (unsigned long long)__double_as_longlong(b);
+  const unsigned long long ic = (unsigned long long)__double_as_longlong(c);
+  const unsigned long long mag = 0x7fffffffffffffffull;
+  const unsigned long long ma = ia & mag, mb = ib & mag, mc = ic & mag;
+  if (((ia ^ ib) | (ia ^ ic)) >> 63 || ma == 0ull || mb == 0ull || mc == 0ull) return 0.0;
+  unsigned long long mm = ma < mb ? ma : mb;
+  mm = mm < mc ? mm : mc;
+  return __longlong_as_double((long long)(mm | (ia & ~mag)));
+}
+
+// minmod of the slopes d1 b1, d2 b2, d3 b3 (b > 0) with f1, f2, f3 = b in FP32: the
+// smallest is picked in FP32 where it is the smallest by kTieF and all three lie in
+// the range of kTinyF, kHugeF, else in FP64.
+__device__ __forceinline__ double minmod_scaled(double d1, double d2, double d3, double b1, double b2,
+                                                double b3, float f1, float f2, float f3) {
+  const long long i1 = __double_as_longlong(d1), i2 = __double_as_longlong(d2), i3 = __double_as_longlong(d3);
+  if (((i1 ^ i2) | (i1 ^ i3)) < 0 || (i1 << 1) == 0 || (i2 << 1) == 0 || (i3 << 1) == 0) return 0.0;
+  const float m1 = fabsf(trunc_f32(d1)) * f1, m2 = fabsf(trunc_f32(d2)) * f2, m3 = fabsf(trunc_f32(d3)) * f3;
+  const float lim = fminf(m1, fminf(m2, m3)) * (1.0f + kTieF);
+  const bool c1 = m1 <= lim, c2 = m2 <= lim, c3 = m3 <= lim;
+  if (!(lim > kTinyF && m1 + m2 + m3 < kHugeF) || int(c1) + int(c2) + int(c3) != 1)
+    return minmod3(d1 * b1, d2 * b2, d3 * b3);
+  return (c1 ? d1 : (c2 ? d2 : d3)) * (c1 ? b1 : (c2 ? b2 : b3));
 }
 
 // Flux in direction dir, normal velocity and squared sound speed in FP32 (see

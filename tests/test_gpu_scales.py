@@ -1,7 +1,9 @@
 """Data far from 1: states scaled by powers of ten, where the comparisons that the
 FP64 kernels first make in FP32 leave FP32's range, against the oracle.
 
-The smoothness indicator's alpha is compared to 1e-9: at its threshold
+The scheme is scale free apart from the limiters' 1e-12, so the bar is the one of
+tests/test_gpu_parity.py, relative to the largest value and flux increment of each
+variable.  The smoothness indicator's alpha is compared to 1e-9: at its threshold
 it changes by s / T = 1e4 times the change of an energy fraction, whose rounding is
 a few 1e-16 times the number of modes, and the tiny steps taken move the state by
 1e-13.
@@ -13,7 +15,7 @@ import oracle
 from paper_2502_07517_gb300 import crkfr
 from paper_2502_07517_gb300 import workloads as wl
 from tests._oracle_util import oracle_desc
-from tests.test_gpu_parity import gpu_run
+from tests.test_gpu_parity import assert_parity, flux_increment, gpu_run
 
 pytestmark = pytest.mark.gpu
 
@@ -70,3 +72,16 @@ def test_indicator_of_scaled_scalars(dim, size):
     prob = dict(prob, limiter=frozenset({"blend"}))
     edge = 0.5 * 10.0 ** (-1.8 * 5.0 ** 0.25) * 0.25
     _check_alpha(prob, size * _modes(prob, u.shape[1], 0.3 * edge, 8.0 * edge, dim)[None])
+
+
+@pytest.mark.parametrize("N", [2, 4])
+@pytest.mark.parametrize("size", [1e-60, 1e-42, 1e-38, 1e-30, 1e30, 1e39, 1e60])
+def test_slopes_of_scaled_scalars(N, size):
+    prob, u = wl.linadv_random(nx=11, ny=7, dim=2, degree=N, seed=3, adv=(0.7, -1.2))
+    prob, u = dict(prob, limiter=frozenset({"blend", "mh"})), size * u
+    d = oracle_desc(prob, alpha_fixed=1.0)
+    dt = 0.5 * oracle.dt(d, u)
+    ref, st, dg = oracle.step(d, u, dt, want_diag=True)
+    assert st == 0
+    g = gpu_run(prob, u, dt_fixed=dt, alpha_fixed=1.0)[0]
+    assert_parity(g, ref, extra_scale=flux_increment(prob, dg, dt))
