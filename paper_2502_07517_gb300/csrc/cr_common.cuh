@@ -307,12 +307,16 @@ __device__ __forceinline__ float sqrt_pos(float x) { return sqrt(x > 0.0f ? x : 
 __device__ __forceinline__ double sqrt_pos(double x) {
   const int h = __double2hiint(x);
   if (unsigned(h - 0x00100000) >= 0x7fe00000u) return gt0(x) ? sqrt(x) : 0.0;
+#ifdef __CUDA_ARCH__
   double y;
   asm("rsqrt.approx.ftz.f64 %0, %1;" : "=d"(y) : "d"(x));
   double g = x * y;
   const double hf = __hiloint2double(__double2hiint(y) - (1 << 20), __double2loint(y));
   g = fma(fma(-g, g, x), hf, g);
   return fma(fma(-g, g, x), hf, g);
+#else
+  return sqrt(x);
+#endif
 }
 // 1 / x.  FP64: one step r (1 + e + e^2), e = 1 - x r, of the third-order
 // (Halley-type) iteration on the hardware's 20-bit approximation: e^3 is below

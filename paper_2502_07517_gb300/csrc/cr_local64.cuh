@@ -66,18 +66,6 @@ __device__ __forceinline__ void flux_c2(const double* u, int dir, double* f, dou
   }
 }
 
-// max(|vL| + sqrt(cL), |vR| + sqrt(cR)), c <= 0 counted as 0: the larger side
-// is picked in FP32 unless the two are within kTieF.
-__device__ __forceinline__ double wave_max(double vL, double cL, double vR, double cR) {
-  const float sL = fabsf(trunc_f32(vL)) + sqrt_f32(trunc_f32(cL));
-  const float sR = fabsf(trunc_f32(vR)) + sqrt_f32(trunc_f32(cR));
-  if (fabsf(sL - sR) > kTieF * (sL + sR)) {
-    const bool left = sL > sR;
-    return fabs(left ? vL : vR) + sqrt_pos(left ? cL : cR);
-  }
-  return fmax(fabs(vL) + sqrt_pos(cL), fabs(vR) + sqrt_pos(cR));
-}
-
 // Twice the Rusanov flux (the factor 1/2 goes into the caller's constants,
 // exactly).
 template <class EQ>

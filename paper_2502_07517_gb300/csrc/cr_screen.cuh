@@ -2,7 +2,8 @@
 // instruction per 16 cycles and SM; a decision whose answer is clear by a margin
 // above the FP32 rounding needs none of it.  Every screen answers "clear" or
 // "not clear", and what is not clear is decided in FP64 as before, so the
-// results do not depend on the screens.
+// results do not depend on the screens.  (Some of it also compiles for the host:
+// tests/test_screens.py holds the screens against FP64.)
 #pragma once
 #include "cr_common.cuh"
 
@@ -23,13 +24,13 @@ constexpr float kTinyF = 1e-30f, kHugeF = 1e30f;
 
 // x as FP32, truncated, from the bit pattern (a conversion instruction runs on
 // the FP64 pipe): magnitudes below FP32's normal range give a value below
-// 2^-126, larger ones its largest finite value; NaN gives a large value.
+// 2^-126, those from 2^128 on and NaN an infinity, with which no comparison
+// against a margin of its own size holds.
 __device__ __forceinline__ float trunc_f32(double x) {
   const int h = __double2hiint(x);
-  int m = (h & 0x7fffffff) - (896 << 20);
-  m = min(max(m, 0), 0x0fefffff);
+  const int m = max((h & 0x7fffffff) - (896 << 20), 0);
   const unsigned b = __funnelshift_l((unsigned)__double2loint(x), (unsigned)m, 3);
-  return __uint_as_float(b | (unsigned(h) & 0x80000000u));
+  return __uint_as_float((m < 0x0ff00000 ? b : 0x7f800000u) | (unsigned(h) & 0x80000000u));
 }
 __device__ __forceinline__ float trunc_f32(float x) { return x; }
 
@@ -55,18 +56,26 @@ __device__ __forceinline__ float to_float(double x) {
   return m == 0ull ? __uint_as_float(s) : float(x);
 }
 __device__ __forceinline__ float rcp_f32(float x) {
+#ifdef __CUDA_ARCH__
   float r;
   asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(x));
   return r;
+#else
+  return 1.0f / x;
+#endif
 }
 
 __device__ __forceinline__ bool finite_bits(double x) { return (__double2hiint(x) & 0x7ff00000) != 0x7ff00000; }
 __device__ __forceinline__ bool finite_bits(float x) { return isfinite(x); }
 
 __device__ __forceinline__ float sqrt_f32(float x) {
+#ifdef __CUDA_ARCH__
   float r;
   asm("sqrt.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(fmaxf(x, 0.0f)));
   return r;
+#else  // (the tests: as the device's, subnormal numbers count as 0)
+  return x >= 1.17549435e-38f ? sqrtf(x) : 0.0f;
+#endif
 }
 
 // minmod of three slopes: the one of smallest magnitude when all three share a
@@ -104,6 +113,19 @@ __device__ __forceinline__ double minmod_scaled(double d1, double d2, double d3,
   if (!(lim > kTinyF && m1 + m2 + m3 < kHugeF) || int(c1) + int(c2) + int(c3) != 1)
     return minmod3(d1 * b1, d2 * b2, d3 * b3);
   return (c1 ? d1 : (c2 ? d2 : d3)) * (c1 ? b1 : (c2 ? b2 : b3));
+}
+
+// max(|vL| + sqrt(cL), |vR| + sqrt(cR)), c <= 0 counted as 0: the larger side
+// is picked in FP32 unless the two are within kTieF, one is infinite there, or
+// both are so small that a c below 2^-126 (0 in FP32: 2^-63 in the speed) counts.
+__device__ __forceinline__ double wave_max(double vL, double cL, double vR, double cR) {
+  const float sL = fabsf(trunc_f32(vL)) + sqrt_f32(trunc_f32(cL));
+  const float sR = fabsf(trunc_f32(vR)) + sqrt_f32(trunc_f32(cR));
+  if (sL + sR > 1e-12f && fabsf(sL - sR) > kTieF * (sL + sR)) {
+    const bool left = sL > sR;
+    return fabs(left ? vL : vR) + sqrt_pos(left ? cL : cR);
+  }
+  return fmax(fabs(vL) + sqrt_pos(cL), fabs(vR) + sqrt_pos(cR));
 }
 
 // Flux in direction dir, normal velocity and squared sound speed in FP32 (see

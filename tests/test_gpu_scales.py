@@ -85,3 +85,35 @@ def test_slopes_of_scaled_scalars(N, size):
     assert st == 0
     g = gpu_run(prob, u, dt_fixed=dt, alpha_fixed=1.0)[0]
     assert_parity(g, ref, extra_scale=flux_increment(prob, dg, dt))
+
+
+@pytest.mark.parametrize("speed", [1e-21, 1e21])
+def test_squared_sound_speeds_beyond_the_fp32_range(speed):
+    prob, u = wl.euler2d_vortex(nx=11, ny=9, degree=3, seed=1)
+    prob = dict(prob, limiter=frozenset({"blend", "mh"}))
+    rng, shape = np.random.default_rng(2), u.shape[1:]
+    rho, p = rng.uniform(0.5, 2.0, shape), speed ** 2 * np.exp(rng.uniform(-3, 3, shape))
+    u = wl.euler_conservative(rho, speed * rng.uniform(-1, 1, shape), speed * rng.uniform(-1, 1, shape), p, 1.4, 2)
+    d = oracle_desc(prob, alpha_fixed=1.0)
+    dt = 0.5 * oracle.dt(d, u)
+    ref, st, dg = oracle.step(d, u, dt, want_diag=True)
+    assert st == 0
+    g = gpu_run(prob, u, dt_fixed=dt, alpha_fixed=1.0)[0]
+    assert_parity(g, ref, extra_scale=flux_increment(prob, dg, dt))
+
+
+@pytest.mark.parametrize("state", [(1e39, 1e60, 1e60), (1e300, 1e300, 1e40), (1e-45, 1e-30, 1e-45)])
+@pytest.mark.parametrize("precision", [crkfr.CR_FP64, crkfr.CR_FP32_BULK], ids=["fp64", "fp32"])
+def test_inadmissible_input_is_refused_at_every_scale(state, precision):
+    """Negative pressures that FP32 cannot show."""
+    rho, mom, E = state
+    if precision == crkfr.CR_FP32_BULK and max(state) > 1e38:
+        pytest.skip("beyond the bulk type")
+    prob, u = wl.euler2d_vortex(nx=4, ny=4, degree=3, seed=1)
+    u = np.ones_like(u) * np.array([rho, 0.0, 0.0, E])[:, None, None]
+    u[1, 5, 3] = mom
+    assert E - 0.5 * mom * mom / rho < 0
+    ctx = crkfr.cr_init_mesh(crkfr.desc_from_problem(prob, precision=precision))
+    with pytest.raises(crkfr.CrError):
+        crkfr.cr_set_state(ctx, u)
+        crkfr.cr_step(ctx, 1, 1e300, 1e-300)

@@ -32,7 +32,18 @@ static inline float __frcp_rn(float x) { return 1.0f / x; }
 using std::isfinite; using std::max; using std::min;
 #include "cr_screen.cuh"
 using namespace crk;
+using Euler = EqEuler<2>;
 extern "C" {
+float truncated(double x) { return trunc_f32(x); }
+int above_eps(const double* u) {
+  float s[4], A[4];
+  for (int v = 0; v < 4; ++v) {
+    s[v] = trunc_f32(u[v]);
+    A[v] = fabsf(s[v]);
+  }
+  return clearly_above_eps<Euler>(s, A, 0.4f);
+}
+double speed(const double* s) { return wave_max(s[0], s[1], s[2], s[3]); }
 double minmod(const double* d, const double* b) {
   return minmod_scaled(d[0], d[1], d[2], b[0], b[1], b[2], trunc_f32(b[0]), trunc_f32(b[1]), trunc_f32(b[2]));
 }
@@ -49,7 +60,8 @@ def lib(tmp_path_factory):
     subprocess.run(["g++", "-O2", "-std=c++17", "-ffp-contract=off", "-shared", "-fPIC", "-I", os.path.join(cuda, "include"),
                     "-I", os.path.join(ROOT, "paper_2502_07517_gb300", "csrc"), str(src), "-o", str(out)], check=True)
     lib = ctypes.CDLL(str(out))
-    lib.minmod.restype = ctypes.c_double
+    lib.minmod.restype = lib.speed.restype = ctypes.c_double
+    lib.truncated.restype, lib.truncated.argtypes = ctypes.c_float, [ctypes.c_double]
     return lib
 
 
@@ -72,3 +84,41 @@ def test_minmod_takes_the_smallest_slope(lib, size, other):
         s = d * b
         want = 0.0 if not ((s > 0).all() or (s < 0).all()) else s[np.argmin(np.abs(s))]
         assert lib.minmod(_p(*d), _p(*b)) == want, (d, b)
+
+
+@pytest.mark.parametrize("size", [1e-150, 1e-60, 1e-42, 1e-25, 1e-20, 1e-19, 1e-12, 1.0, 1e12, 1e18, 1e20, 1e30, 1e38, 1e60, 1e150])
+@pytest.mark.parametrize("ratio", [1e-4, 1.0, 1e4])
+def test_wave_speed_is_the_larger_one(lib, size, ratio):
+    rng = np.random.default_rng(5)
+    for it in range(400):
+        v = size * ratio * rng.uniform(-1.0, 1.0, 2)
+        c = (size * rng.uniform(0.1, 3.0, 2)) ** 2 * rng.choice([1.0, 1.0, 0.0, -1.0], 2)
+        want = max(abs(v) + np.sqrt(np.maximum(c, 0.0)))
+        assert lib.speed(_p(v[0], c[0], v[1], c[1])) == want, (v, c)
+
+
+@pytest.mark.parametrize("x", [1.0, -3.1415926535, 1e-30, 2.0 ** -126, 3.4e38, -2.0 ** 128, 1e39, -1e300, float("inf"),
+                               float("nan"), 0.0, -0.0, 1e-40, -1e-300])
+def test_truncation(lib, x):
+    y = lib.truncated(x)
+    if not abs(x) < 2.0 ** 128:
+        assert abs(y) == np.inf and (np.isnan(x) or np.sign(y) == np.sign(x))
+    elif abs(x) >= 2.0 ** -126:
+        assert 0 <= (x - y) / x < 2.0 ** -23
+    else:
+        assert abs(y) < 2.0 ** -126
+
+
+@pytest.mark.parametrize("size", SIZES)
+def test_no_inadmissible_state_is_clear(lib, size):
+    """Euler states whose pressure is negative, for the reason of one momentum or energy
+    of another size than the rest."""
+    rng = np.random.default_rng(4)
+    for it in range(400):
+        with np.errstate(over="ignore"):
+            rho, mom, e = np.minimum(size * 10.0 ** (rng.uniform(-40, 40, 3) if it % 2 else rng.uniform([0, 0, 0], [4, 40, 4])), 1e150)
+        s = np.array([rho, mom, rng.choice([-1.0, 0.0, 1.0]) * mom, e])
+        with np.errstate(over="ignore", divide="ignore", invalid="ignore", under="ignore"):
+            p = 0.4 * (s[3] - 0.5 * (s[1] / s[0] * s[1] + s[2] / s[0] * s[2]))
+        if not (s[0] >= 1e-12 and p >= 1e-12):
+            assert not lib.above_eps(_p(*s)), s
