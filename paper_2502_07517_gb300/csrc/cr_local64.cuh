@@ -80,26 +80,6 @@ __device__ __forceinline__ void rusanov_twice(const double* uL, const double* uR
   for (int v = 0; v < EQ::M; ++v) out[v] = fma(-lam, uR[v] - uL[v], fL[v] + fR[v]);
 }
 
-// FP32 screen of the MUSCL-Hancock states: s is a state and A bounds the
-// magnitudes its parts are summed from.  True only when the state is admissible
-// by a margin above the FP32 rounding of the sums and products.
-template <class EQ>
-__device__ __forceinline__ bool clearly_admissible(const float* s, const float* A) {
-  if constexpr (EQ::K == 0) return true;
-  if (!(s[0] > kMarginF * A[0])) return false;
-  if constexpr (IsEuler<EQ>::value) {
-    constexpr int E = EQ::M - 1;
-    const float k2 = E == 3 ? s[1] * s[1] + s[2] * s[2] : s[1] * s[1], a2 = E == 3 ? A[1] * A[1] + A[2] * A[2] : A[1] * A[1];
-    return s[E] * s[0] - 0.5f * k2 > kMarginF * (A[E] * A[0] + a2);
-  } else if constexpr (EQ::M == 6) {
-    const float a11 = 2.0f * s[0] * s[3] - s[1] * s[1], a22 = 2.0f * s[0] * s[5] - s[2] * s[2];
-    const float a12 = 2.0f * s[0] * s[4] - s[1] * s[2];
-    const float B = 2.0f * A[0] * (A[3] + A[4] + A[5]) + A[1] * A[1] + A[2] * A[2];
-    return a11 > kMarginF * B && a11 * a22 - a12 * a12 > 5.0f * kMarginF * B * B;
-  }
-  return true;
-}
-
 // MUSCL-Hancock states of one node (Sec. 4.2): the evolved states at its
 // subcell faces (in one dimension the y states are not formed), or the node value where one of them is not admissible.  nb(v,
 // dir, up) is the neighbour node's value along the line; hx, hy = dt / (2 w h).

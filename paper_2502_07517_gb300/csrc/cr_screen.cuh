@@ -151,6 +151,29 @@ __device__ __forceinline__ void flux_c2_f32(const float* u, int dir, float* f, f
   }
 }
 
+// FP32 screen of the MUSCL-Hancock states: s is a state and A bounds the
+// magnitudes its parts are summed from.  True only when the state is admissible
+// by a margin above the FP32 rounding of the sums and products.  The products are
+// of second order in the state (ten-moment: fourth), so their margin, too, has to be
+// in FP32's range: near vacuum (rho p below 1e-25, ten-moment 1e-13) nothing is clear.
+template <class EQ>
+__device__ __forceinline__ bool clearly_admissible(const float* s, const float* A) {
+  if constexpr (EQ::K == 0) return true;
+  if (!(s[0] > kMarginF * A[0] && A[0] > kTinyF)) return false;
+  if constexpr (IsEuler<EQ>::value) {
+    constexpr int E = EQ::M - 1;
+    const float k2 = E == 3 ? s[1] * s[1] + s[2] * s[2] : s[1] * s[1], a2 = E == 3 ? A[1] * A[1] + A[2] * A[2] : A[1] * A[1];
+    const float margin = kMarginF * (A[E] * A[0] + a2);
+    return fminf(A[E], margin) > kTinyF && s[E] * s[0] - 0.5f * k2 > margin;
+  } else if constexpr (EQ::M == 6) {
+    const float a11 = 2.0f * s[0] * s[3] - s[1] * s[1], a22 = 2.0f * s[0] * s[5] - s[2] * s[2];
+    const float a12 = 2.0f * s[0] * s[4] - s[1] * s[2], a345 = A[3] + A[4] + A[5];
+    const float B = 2.0f * A[0] * a345 + A[1] * A[1] + A[2] * A[2], margin = 5.0f * kMarginF * B * B;
+    return fminf(a345, margin) > kTinyF && a11 > kMarginF * B && a11 * a22 - a12 * a12 > margin;
+  }
+  return true;
+}
+
 // Constraint k of the state s in FP32 and the bound of its error, A[v] bounding
 // the magnitudes s[v] is summed from.
 template <class EQ>

@@ -43,6 +43,14 @@ int above_eps(const double* u) {
   }
   return clearly_above_eps<Euler>(s, A, 0.4f);
 }
+int admissible(const double* u, int m) {
+  float s[6], A[6];
+  for (int v = 0; v < m; ++v) {
+    s[v] = trunc_f32(u[v]);
+    A[v] = fabsf(s[v]);
+  }
+  return m == 4 ? clearly_admissible<Euler>(s, A) : clearly_admissible<EqTenMoment>(s, A);
+}
 double speed(const double* s) { return wave_max(s[0], s[1], s[2], s[3]); }
 double minmod(const double* d, const double* b) {
   return minmod_scaled(d[0], d[1], d[2], b[0], b[1], b[2], trunc_f32(b[0]), trunc_f32(b[1]), trunc_f32(b[2]));
@@ -122,3 +130,28 @@ def test_no_inadmissible_state_is_clear(lib, size):
             p = 0.4 * (s[3] - 0.5 * (s[1] / s[0] * s[1] + s[2] / s[0] * s[2]))
         if not (s[0] >= 1e-12 and p >= 1e-12):
             assert not lib.above_eps(_p(*s)), s
+
+
+@pytest.mark.parametrize("size", SIZES + [1e-9, 1e-10, 3e-11, 1e-11, 3e-12, 1e-12, 1e-13, 1e-19, 1e-21])
+@pytest.mark.parametrize("m", [4, 6])
+def test_states_at_and_past_the_edge_are_not_clear(lib, size, m):
+    """Pressures (ten-moment: their determinants) of 0 and below, at every size; and
+    ordinary states are clear."""
+    rng = np.random.default_rng(6)
+    for it in range(400):
+        rho, v1, v2, a, b = np.exp(rng.uniform(-3.0, 3.0, 5)) * np.array([1.0, *rng.choice([-1.0, 1.0], 2), 1.0, 1.0])
+        if it % 2 and m == 6:
+            v1 = v2 = 0.0
+        over = rng.choice([1.0, 1.0 + 1e-6, 1.0 + 1e-3, 2.0])
+        if m == 4:
+            u = np.array([rho, rho * v1, rho * v2, 0.5 * rho * (v1 * v1 + v2 * v2) / over])
+            good = u + np.array([0.0, 0.0, 0.0, a + u[3]])
+        else:
+            u = np.array([rho, rho * v1, rho * v2, 0.5 * (a + rho * v1 * v1), 0.5 * (over * np.sqrt(a * b) + rho * v1 * v2),
+                          0.5 * (b + rho * v2 * v2)])
+            good = np.array([rho, 0.0, 0.0, 0.5 * a, 0.1 * min(a, b), 0.5 * b])
+        scale = 2.0 ** np.round(np.log2(size))            # (exactly the same state at another size)
+        with np.errstate(under="ignore"):
+            assert not lib.admissible(_p(*(u * scale)), m), u
+        if 1e-3 < size < 1e3:
+            assert lib.admissible(_p(*(good * scale)), m), good
