@@ -175,7 +175,9 @@ __device__ __forceinline__ bool clearly_admissible(const float* s, const float* 
 }
 
 // Constraint k of the state s in FP32 and the bound of its error, A[v] bounding
-// the magnitudes s[v] is summed from.
+// the magnitudes s[v] is summed from.  kTinyF covers what is below FP32's normal
+// range, and in the ten-moment constraint 1e-18 what a flushed h^2 + p12^2 (2^-126)
+// takes from its root.
 template <class EQ>
 __device__ __forceinline__ void screened_constraint(const float* s, const float* A, int k, float gm1, float* P,
                                                     float* err) {
@@ -184,7 +186,7 @@ __device__ __forceinline__ void screened_constraint(const float* s, const float*
   if constexpr (EQ::K > 0) {
     if (k == 0) {
       *P = s[0];
-      *err = kMarginF * A[0];
+      *err = kMarginF * A[0] + kTinyF;
     } else if constexpr (IsEuler<EQ>::value) {
       constexpr int E = EQ::M - 1;
       const float r = __frcp_rn(s[0]), v1 = s[1] * r, v2 = E == 3 ? s[2] * r : 0.0f;
@@ -194,14 +196,14 @@ __device__ __forceinline__ void screened_constraint(const float* s, const float*
         e += fabsf(v2) * A[2];
       }
       *P = gm1 * (s[E] - 0.5f * kin);
-      *err = kMarginF * gm1 * e;
+      *err = kMarginF * gm1 * e + kTinyF;
     } else {
       const float r = __frcp_rn(s[0]), v1 = s[1] * r, v2 = s[2] * r;
       const float p11 = 2.0f * s[3] - s[1] * v1, p12 = 2.0f * s[4] - s[1] * v2, p22 = 2.0f * s[5] - s[2] * v2;
       const float h = 0.5f * (p11 - p22);
       const float w = fabsf(v1) + fabsf(v2);
       *P = 0.5f * (p11 + p22) - sqrt_f32(h * h + p12 * p12);
-      *err = kMarginF * (2.0f * (A[3] + A[4] + A[5]) + 2.0f * w * (A[1] + A[2]) + w * w * A[0]);
+      *err = kMarginF * (2.0f * (A[3] + A[4] + A[5]) + 2.0f * w * (A[1] + A[2]) + w * w * A[0]) + 1e-18f;
     }
   }
 }
@@ -241,7 +243,7 @@ __device__ __forceinline__ bool flux_limiter_idle(const float* uL, const float* 
     aL[v] = fabsf(bL[v]) + cL * a;
     aR[v] = fabsf(bR[v]) + cR * a;
   }
-  bool idle = true;
+  bool idle = fminf(cL, cR) > kTinyF;
 #pragma unroll
   for (int k = 0; k < EQ::K; ++k) {
     float c[M], pl, el, pr, er, hl, fl, hr, fr;

@@ -87,6 +87,39 @@ def test_slopes_of_scaled_scalars(N, size):
     assert_parity(g, ref, extra_scale=flux_increment(prob, dg, dt))
 
 
+def _random_fluid(prob, ne, npts, seed, spread=4.0):
+    rng = np.random.default_rng(seed)
+    draw = lambda lo, hi: np.exp(rng.uniform(np.log(lo), np.log(hi), (ne, npts)))  # noqa: E731
+    rho, v1, v2 = draw(1.0 / spread, spread), rng.uniform(-1, 1, (ne, npts)), rng.uniform(-1, 1, (ne, npts))
+    if prob["equation"] == "euler":
+        return wl.euler_conservative(rho, v1, v2, draw(0.1, 3.0), 1.4, 2)
+    a, b = draw(0.1, 3.0), draw(0.1, 3.0)
+    return wl.tenmoment_conservative(rho, v1, v2, a, rng.uniform(-0.9, 0.9, a.shape) * np.sqrt(a * b), b)
+
+
+@pytest.mark.parametrize("make", [wl.euler2d_vortex, wl.tenmoment2d_voronoi], ids=["euler", "tenmoment"])
+@pytest.mark.parametrize("alpha", [None, 1.0])
+@pytest.mark.parametrize("power", [-200, -150, -126, -120, -70, -66, -63, -50, -43, -36, 60, 83, 120, 150])
+def test_scaled_fluids(make, alpha, power):
+    """A state times a power of two gives the result times that power: no rounding
+    changes, only what is decided in FP32 and what in FP64.  The values that enter a
+    decision are formed by the same formulas at two places, which a compiler may
+    contract differently; the flux limiter's theta multiplies such roundings by up to
+    1e4 here (random nodes), so 1e-9 of the largest value is allowed.  A wrong decision
+    moves it by percents."""
+    prob, u = make(nx=11, ny=9, degree=3, seed=1)
+    lim = {"mh", "flux"} | ({"blend"} if alpha else set())
+    prob = dict(prob, limiter=frozenset(lim), source=None)
+    u = _random_fluid(prob, u.shape[1], u.shape[2], 5)
+    d = oracle_desc(prob, alpha_fixed=alpha)
+    dt = 0.5 * oracle.dt(d, u)
+    if oracle.step(d, u, dt)[1]:     # (a mean went negative: nothing to compare)
+        dt *= 0.1
+    ref = gpu_run(prob, u, dt_fixed=dt, alpha_fixed=alpha)[0]
+    g = gpu_run(prob, u * 2.0 ** power, dt_fixed=dt, alpha_fixed=alpha)[0]
+    assert_parity(g * 2.0 ** -power, ref, rtol=1e-9)
+
+
 @pytest.mark.parametrize("speed", [1e-21, 1e21])
 def test_squared_sound_speeds_beyond_the_fp32_range(speed):
     prob, u = wl.euler2d_vortex(nx=11, ny=9, degree=3, seed=1)

@@ -51,6 +51,17 @@ int admissible(const double* u, int m) {
   }
   return m == 4 ? clearly_admissible<Euler>(s, A) : clearly_admissible<EqTenMoment>(s, A);
 }
+int idle(const double* d, int m, double cL, double cR) {  // uL, uR, bL, bR, F
+  float x[5][6];
+  for (int i = 0; i < 5; ++i)
+    for (int v = 0; v < m; ++v) x[i][v] = trunc_f32(d[i * m + v]);
+  Phys<double> ph{};
+  ph.gamma = 1.4;
+  ph.gm1 = 0.4;
+  const float l = trunc_f32(cL), r = trunc_f32(cR);
+  return m == 4 ? flux_limiter_idle<Euler>(x[0], x[1], x[2], x[3], x[4], l, r, 0, ph)
+                : flux_limiter_idle<EqTenMoment>(x[0], x[1], x[2], x[3], x[4], l, r, 0, ph);
+}
 double speed(const double* s) { return wave_max(s[0], s[1], s[2], s[3]); }
 double minmod(const double* d, const double* b) {
   return minmod_scaled(d[0], d[1], d[2], b[0], b[1], b[2], trunc_f32(b[0]), trunc_f32(b[1]), trunc_f32(b[2]));
@@ -155,3 +166,55 @@ def test_states_at_and_past_the_edge_are_not_clear(lib, size, m):
             assert not lib.admissible(_p(*(u * scale)), m), u
         if 1e-3 < size < 1e3:
             assert lib.admissible(_p(*(good * scale)), m), good
+
+
+def _flux(u):
+    v = u[1] / u[0]
+    if len(u) == 4:
+        p = 0.4 * (u[3] - 0.5 * (u[1] ** 2 + u[2] ** 2) / u[0])
+        return np.array([u[1], u[1] * v + p, u[2] * v, (u[3] + p) * v]), abs(v) + np.sqrt(1.4 * p / u[0])
+    v2 = u[2] / u[0]
+    p11, p12 = 2 * u[3] - u[1] * v, 2 * u[4] - u[1] * v2
+    f = np.array([u[1], p11 + u[1] * v, p12 + u[1] * v2, (u[3] + p11) * v, u[4] * v + 0.5 * (p11 * v2 + p12 * v), u[5] * v + p12 * v2])
+    return f, abs(v) + np.sqrt(3 * p11 / u[0])
+
+
+def _constraints(u):
+    if len(u) == 4:
+        return np.array([u[0], 0.4 * (u[3] - 0.5 * (u[1] ** 2 + u[2] ** 2) / u[0])])
+    p11, p12, p22 = 2 * u[3] - u[1] ** 2 / u[0], 2 * u[4] - u[1] * u[2] / u[0], 2 * u[5] - u[2] ** 2 / u[0]
+    return np.array([u[0], 0.5 * (p11 + p22) - np.sqrt((0.5 * (p11 - p22)) ** 2 + p12 ** 2)])
+
+
+@pytest.mark.parametrize("size", [2.0 ** k for k in (-500, -200, -150, -140, -126, -120, -100, -80, -70, -66, -63, -60, -50, -40,
+                                                     -30, 0, 40, 80, 120, 126, 200, 500)])
+@pytest.mark.parametrize("m", [4, 6])
+def test_idle_flux_limiter(lib, m, size):
+    """Where the screen calls the flux limiter idle, both candidates with the flux F
+    keep a tenth of the smaller low-order candidate in every constraint (1e-9 of the
+    constraint's own rounding aside)."""
+    rng = np.random.default_rng(7)
+
+    def state():
+        rho, a, b = np.exp(rng.uniform(-2.0, 2.0, 3))
+        v1, v2 = rng.uniform(-1.0, 1.0, 2)
+        if m == 4:
+            return np.array([rho, rho * v1, rho * v2, a / 0.4 + 0.5 * rho * (v1 * v1 + v2 * v2)])
+        r = rng.choice([0.0, 0.9, 1.0 - 1e-3, 1.0 - 1e-6]) * rng.choice([-1.0, 1.0]) * np.sqrt(a * b)
+        return 0.5 * np.array([2 * rho, 2 * rho * v1, 2 * rho * v2, a + rho * v1 * v1, r + rho * v1 * v2, b + rho * v2 * v2])
+
+    clear = 0
+    for it in range(500):
+        uL, uR, bL, bR = (state() for _ in range(4))
+        (fL, sL), (fR, sR) = _flux(uL), _flux(uR)
+        lam = max(sL, sR)
+        low = 0.5 * (fL + fR) - 0.5 * lam * (uR - uL)
+        F = low + lam * rng.choice([0.01, 0.3, 3.0]) * rng.standard_normal(m)
+        c = 10.0 ** rng.uniform(-3.0, -0.3, 2) / lam
+        if not lib.idle(_p(*(size * np.concatenate([uL, uR, bL, bR, F]))), m, ctypes.c_double(c[0]), ctypes.c_double(c[1])):
+            continue
+        clear += 1
+        lo = np.minimum(_constraints(bL - c[0] * low), _constraints(bR + c[1] * low))
+        hi = np.minimum(_constraints(bL - c[0] * F), _constraints(bR + c[1] * F))
+        assert (hi >= 0.1 * lo - 1e-9 * abs(hi)).all(), (it, lo, hi)
+    assert clear > 20 or not 2.0 ** -30 <= size <= 2.0 ** 40
