@@ -331,9 +331,6 @@ __device__ __forceinline__ double recip(double x) {
   e = fma(e, e, e);
   return fma(r, e, r);
 }
-// a / x (FP64: a times the reciprocal, one rounding more than the division)
-__device__ __forceinline__ float quot(float a, float x) { return a / x; }
-__device__ __forceinline__ double quot(double a, double x) { return a * recip(x); }
 
 struct EqLinAdv {  // u_t + a . grad u = 0, Sec. 5.1.1
   static constexpr int M = 1, K = 0;
@@ -483,7 +480,7 @@ struct EqEuler {
   }
   template <typename real>
   __device__ static real pressure(const real* u, const Phys<real>& ph) {
-    return ph.gm1 * (u[E] - quot(kinetic_rho(u), u[0]));
+    return ph.gm1 * (u[E] - kinetic_rho(u) / u[0]);  // (a division: decisions and the limiters' roots rest on it)
   }
   template <typename real>
   __device__ static void flux_r(const real* u, int dir, real rinv, real* f, real* p_out,
@@ -614,12 +611,12 @@ struct EqTenMoment {
   template <typename real>
   __device__ static real constraint(const real* u, int k, const Phys<real>&) {
     if (k == 0) return u[0];
-    const real rinv = recip(u[0]);
+    const real rinv = real(1) / u[0];
     const real p11 = real(2) * u[3] - u[1] * u[1] * rinv;
     const real p12 = real(2) * u[4] - u[1] * u[2] * rinv;
     const real p22 = real(2) * u[5] - u[2] * u[2] * rinv;
     const real h = real(0.5) * (p11 - p22);
-    return real(0.5) * (p11 + p22) - sqrt_pos(h * h + p12 * p12);
+    return real(0.5) * (p11 + p22) - sqrt(h * h + p12 * p12);
   }
   template <typename real>
   __device__ static bool admissible_fast(const real* u, const Phys<real>&) {

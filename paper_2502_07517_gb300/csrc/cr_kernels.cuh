@@ -1646,7 +1646,7 @@ __device__ __forceinline__ double scaling_root(const double* ubar, const double*
   double lo = 0.0, hi = 1.0, glo = EQ::constraint(ubar, 1, ph) - eps, ghi = g1;
   int last = 0;
   for (int it = 0; it < 60 && hi - lo > kTol; ++it) {
-    double c = lo + (hi - lo) * quot(glo, glo - ghi);
+    double c = lo + (hi - lo) * (glo / (glo - ghi));
     c = fmin(fmax(c, lo + kStep), hi - kStep);
     double tmp[EQ::M];
 #pragma unroll

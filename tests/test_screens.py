@@ -1,6 +1,7 @@
 """The FP32 screens in front of FP64 decisions (csrc/cr_screen.cuh), compiled for
 the host: over all magnitudes of the data, also those outside FP32's range, a
-screen that answers must answer as FP64 does.
+screen that answers must answer as FP64 does.  And the FP64 constraints that decide
+where a screen does not.
 """
 import ctypes
 import os
@@ -62,6 +63,11 @@ int idle(const double* d, int m, double cL, double cR) {  // uL, uR, bL, bR, F
   return m == 4 ? flux_limiter_idle<Euler>(x[0], x[1], x[2], x[3], x[4], l, r, 0, ph)
                 : flux_limiter_idle<EqTenMoment>(x[0], x[1], x[2], x[3], x[4], l, r, 0, ph);
 }
+double constraint(const double* u, int m) {
+  Phys<double> ph{};
+  ph.gm1 = 0.4;
+  return m == 4 ? Euler::constraint(u, 1, ph) : EqTenMoment::constraint(u, 1, ph);
+}
 double speed(const double* s) { return wave_max(s[0], s[1], s[2], s[3]); }
 double minmod(const double* d, const double* b) {
   return minmod_scaled(d[0], d[1], d[2], b[0], b[1], b[2], trunc_f32(b[0]), trunc_f32(b[1]), trunc_f32(b[2]));
@@ -79,7 +85,7 @@ def lib(tmp_path_factory):
     subprocess.run(["g++", "-O2", "-std=c++17", "-ffp-contract=off", "-shared", "-fPIC", "-I", os.path.join(cuda, "include"),
                     "-I", os.path.join(ROOT, "paper_2502_07517_gb300", "csrc"), str(src), "-o", str(out)], check=True)
     lib = ctypes.CDLL(str(out))
-    lib.minmod.restype = lib.speed.restype = ctypes.c_double
+    lib.minmod.restype = lib.speed.restype = lib.constraint.restype = ctypes.c_double
     lib.truncated.restype, lib.truncated.argtypes = ctypes.c_float, [ctypes.c_double]
     return lib
 
@@ -218,3 +224,23 @@ def test_idle_flux_limiter(lib, m, size):
         hi = np.minimum(_constraints(bL - c[0] * F), _constraints(bR + c[1] * F))
         assert (hi >= 0.1 * lo - 1e-9 * abs(hi)).all(), (it, lo, hi)
     assert clear > 20 or not 2.0 ** -30 <= size <= 2.0 ** 40
+
+
+@pytest.mark.parametrize("m", [4, 6])
+def test_constraints_are_the_formula(lib, m):
+    """One rounding per operation (no reciprocal in the place of a division), and no
+    number where an entry is none."""
+    rng = np.random.default_rng(8)
+    for it in range(2000):
+        u = rng.standard_normal(m) * 10.0 ** rng.uniform(-3, 3, m)
+        u[0] = abs(u[0])
+        if m == 4:
+            want = 0.4 * (u[3] - 0.5 * (u[1] * u[1] + u[2] * u[2]) / u[0])
+        else:
+            r = 1.0 / u[0]
+            p11, p12, p22 = 2.0 * u[3] - u[1] * u[1] * r, 2.0 * u[4] - u[1] * u[2] * r, 2.0 * u[5] - u[2] * u[2] * r
+            h = 0.5 * (p11 - p22)
+            want = 0.5 * (p11 + p22) - np.sqrt(h * h + p12 * p12)
+        assert lib.constraint(_p(*u), m) == want
+        u[rng.integers(0, m)] = np.nan
+        assert np.isnan(lib.constraint(_p(*u), m))
