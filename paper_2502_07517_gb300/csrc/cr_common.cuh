@@ -325,11 +325,15 @@ __device__ __forceinline__ double sqrt_pos(double x) {
 // per warp).
 __device__ __forceinline__ float recip(float x) { return 1.0f / x; }
 __device__ __forceinline__ double recip(double x) {
+#ifdef __CUDA_ARCH__
   double r;
   asm("rcp.approx.ftz.f64 %0, %1;" : "=d"(r) : "d"(x));
   double e = fma(-x, r, 1.0);
   e = fma(e, e, e);
   return fma(r, e, r);
+#else
+  return 1.0 / x;
+#endif
 }
 
 struct EqLinAdv {  // u_t + a . grad u = 0, Sec. 5.1.1

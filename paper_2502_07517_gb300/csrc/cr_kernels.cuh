@@ -18,6 +18,7 @@
 // [M][EPB][Np] so that consecutive threads touch consecutive words.
 #pragma once
 #include "cr_common.cuh"
+#include "cr_root.cuh"
 #include "cr_screen.cuh"
 
 namespace crk {
@@ -1628,52 +1629,14 @@ __device__ __forceinline__ void rate_and_finish(const Mesh& m, const Phys<T>& ph
   finish_block(ctl, brate, advance, dtd, last, nblk);
 }
 
-// Largest theta (to 2^-50) with P_2(ubar + theta (pt - ubar)) >= eps, for a
-// point with P_2(pt) - eps = g1 < 0 and an admissible mean: a bracket [lo, hi]
-// with the constraint met at lo and missed at hi, narrowed by chords with the
-// Illinois rule (a side kept twice halves its value; every step moves at least
-// 2^-51 into the bracket).  P_2 is concave along the segment and close to a
-// line, so 7 to 10 evaluations do what a bisection does in 50; the evaluations
-// were most of the update kernel on steep ten-moment data (FP32 bulk, 211 x 173
-// elements, N = 3: 293 -> 125 us with the shorter reciprocals and square roots
-// of the constraint).  Both end where the rounding of P_2 decides its sign: against
-// 80-bit arithmetic, on 6,893 random 1D Euler segments, the mean error of theta is
-// 6.8e-16, a bisection's 8.4e-16.
-template <class EQ>
-__device__ __forceinline__ double scaling_root(const double* ubar, const double* pt, double g1, double eps,
-                                               const Phys<double>& ph) {
-  constexpr double kTol = 8.881784197001252e-16, kStep = 4.440892098500626e-16;  // 2^-50, 2^-51
-  double lo = 0.0, hi = 1.0, glo = EQ::constraint(ubar, 1, ph) - eps, ghi = g1;
-  int last = 0;
-  for (int it = 0; it < 60 && hi - lo > kTol; ++it) {
-    double c = lo + (hi - lo) * (glo / (glo - ghi));
-    c = fmin(fmax(c, lo + kStep), hi - kStep);
-    double tmp[EQ::M];
-#pragma unroll
-    for (int v = 0; v < EQ::M; ++v) tmp[v] = ubar[v] + c * (pt[v] - ubar[v]);
-    const double gc = EQ::constraint(tmp, 1, ph) - eps;
-    if (gc >= 0.0) {
-      lo = c;
-      glo = gc;
-      if (last == 1) ghi *= 0.5;
-      last = 1;
-    } else {
-      hi = c;
-      ghi = gc;
-      if (last == 2) glo *= 0.5;
-      last = 2;
-    }
-  }
-  return lo;
-}
-
 // The scaling limiter (Sec. 3.2) of a block in which some point needs it, in FP64:
 // theta_1 for the density, theta_2 for the second constraint (scaling_root), per
 // element.  Called by every thread of the block; node values come and go in the
 // rows of the reduction buffer behind the first ([M] ur, FP32 bulk then [M] fl; only
 // elements with a failing point change and do FP64 work), means and limiter scalars
-// in sEl.  Out of line: most blocks never come here, and the update kernel keeps its
-// registers.
+// in sEl.  Out of line, as most blocks never come here (k_update with it inline and out
+// of line: ten-moment FP32 bulk, 211 x 173 elements, 0.116 and 0.118 ms; FP32-bulk Euler
+// at 512 x 512, which never comes here, 0.334 and 0.338).
 template <int DIM, int N, class EQ, typename real, bool MIXED, int T>
 __device__ __noinline__ void limit_block(const KParams<real>& P, const Tab<double>& td, double* sU, double* sRed,
                                          const double* sEl, int need, bool mean_ok, bool traces) {
@@ -1745,9 +1708,8 @@ __device__ __noinline__ void limit_block(const KParams<real>& P, const Tab<doubl
       for (int t = 0; t < np2; ++t) pts[t][0] = ubar[0] + th1 * (pts[t][0] - ubar[0]);
     }
     for (int t = 0; t < np2; ++t) {
-      const double g1 = EQ::constraint(pts[t], 1, P.phd) - eps2;
-      if (g1 >= 0.0) continue;
-      const double lo = scaling_root<EQ>(ubar, pts[t], g1, eps2, P.phd);
+      if (EQ::constraint(pts[t], 1, P.phd) >= eps2) continue;
+      const double lo = scaling_root<EQ>(ubar, pts[t], eps2, P.phd);
       tmin = OpMinBits()(tmin, lo);
     }
   }
@@ -2100,97 +2062,19 @@ __device__ __forceinline__ void update_body(const KParams<real>& P, const Tab<re
     // with a failing point takes the FP64 result below: the others keep their
     // values bit for bit, whichever elements share their block.
     if (__syncthreads_or(valid && need)) {
-      // (the limiter out of line: ten-moment FP32 bulk, 211 x 173 elements, k_update
-      // 0.123 -> 0.106 ms, FP64 256 x 256 0.254 -> 0.221; FP32-bulk Euler, where few
-      // blocks limit, keeps it inline: 0.305 against 0.315 ms at 512 x 512)
-      if constexpr (!MIXED || M == 6) {
-        // node values through the free rows of the reduction buffer, so that they
-        // can stay in registers here
-        real* X = reinterpret_cast<real*>(sRed + stride);
+      // node values through the free rows of the reduction buffer, so that they can
+      // stay in registers here
+      real* X = reinterpret_cast<real*>(sRed + stride);
 #pragma unroll
-        for (int v = 0; v < M; ++v) {
-          X[v * stride + tid] = ur[v];
-          if constexpr (MIXED) X[(M + v) * stride + tid] = fl[v];
-        }
-        limit_block<DIM, N, EQ, real, MIXED, T>(P, td, sU, sRed, sEl, need, mean_ok, traces);
+      for (int v = 0; v < M; ++v) {
+        X[v * stride + tid] = ur[v];
+        if constexpr (MIXED) X[(M + v) * stride + tid] = fl[v];
+      }
+      limit_block<DIM, N, EQ, real, MIXED, T>(P, td, sU, sRed, sEl, need, mean_ok, traces);
 #pragma unroll
-        for (int v = 0; v < M; ++v) {
-          ur[v] = X[v * stride + tid];
-          if constexpr (MIXED) fl[v] = X[(M + v) * stride + tid];
-        }
-      } else {
-        // FP64 path (oracle's limiter): points in FP64
-        double pts[1 + SPT][M];
-        int np2 = 1;
-        __syncthreads();
-        RED(0) = need ? 0.0 : 1.0;
-        elem_reduce<NP, 1>(sRed, epb, el, k, OpMin());
-        const bool elem_need = RED0(0) == 0.0;
-        __syncthreads();
-#pragma unroll
-        for (int v = 0; v < M; ++v) {
-          if constexpr (MIXED) pts[0][v] = ubar[v] + double(fl[v]);
-          else pts[0][v] = double(ur[v]);
-        }
-#pragma unroll
-        for (int v = 0; v < M; ++v) ATU(v, k) = pts[0][v];
-        __syncthreads();
-        if (traces) {
-#pragma unroll
-          for (int mm = 0; mm < SPT; ++mm) {
-            const int sl = k + mm * NP;
-            if (sl < NSLOT) {
-              const int side = sl / NFN, j = sl - side * NFN;
-#pragma unroll
-              for (int v = 0; v < M; ++v) {
-                double acc = 0.0;
-#pragma unroll
-                for (int r = 0; r < n; ++r) {
-                  const double l = (side & 1) ? td.l1[r] : td.l0[r];
-                  acc += l * ATU(v, side < 2 ? r + n * j : j + n * r);
-                }
-                pts[np2][v] = acc;
-              }
-              ++np2;
-            }
-          }
-        }
-        double rmin = pts[0][0];
-        for (int t = 1; t < np2; ++t) rmin = fmin(rmin, pts[t][0]);
-        RED(0) = rmin;
-        elem_reduce<NP, 1>(sRed, epb, el, k, OpMin());
-        rmin = RED0(0);
-        __syncthreads();
-        if (mean_ok && rmin < eps1) {
-          const double th1 = (ubar[0] - eps1) / (ubar[0] - rmin);
-          for (int t = 0; t < np2; ++t) pts[t][0] = ubar[0] + th1 * (pts[t][0] - ubar[0]);
-        }
-        double tmin = 1.0;
-        if (mean_ok)
-          for (int t = 0; t < np2; ++t) {
-            const double g1 = EQ::constraint(pts[t], 1, P.phd) - eps2;
-            if (g1 >= 0.0) continue;
-            const double lo = scaling_root<EQ>(ubar, pts[t], g1, eps2, P.phd);
-            tmin = fmin(tmin, lo);
-          }
-        RED(0) = tmin;
-        elem_reduce<NP, 1>(sRed, epb, el, k, OpMin());
-        const double th2 = RED0(0);
-        __syncthreads();
-        if (th2 < 1.0)
-          for (int t = 0; t < np2; ++t)
-#pragma unroll
-            for (int v = 0; v < M; ++v) pts[t][v] = ubar[v] + th2 * (pts[t][v] - ubar[v]);
-        // status tests only the mean (above): the limited points are admissible
-        // in exact arithmetic, and a tiny constraint value at a face trace is
-        // below the rounding of its interpolation
-        if (elem_need) {
-#pragma unroll
-          for (int v = 0; v < M; ++v) {
-            if constexpr (MIXED) fl[v] = real(pts[0][v] - ubar[v]);
-            ur[v] = real(pts[0][v]);
-          }
-        }
+      for (int v = 0; v < M; ++v) {
+        ur[v] = X[v * stride + tid];
+        if constexpr (MIXED) fl[v] = X[(M + v) * stride + tid];
       }
     }
   }
