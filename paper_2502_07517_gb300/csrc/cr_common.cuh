@@ -303,10 +303,10 @@ __device__ __forceinline__ float sqrt_pos(float x) { return sqrt(x > 0.0f ? x : 
 // = y / 2 from the hardware's approximation y of 1 / sqrt(x) (20 bits; 2^-40 and
 // then below the rounding of the last FMA, so the error is that rounding's).
 // Five FP64 instructions, where sqrt() takes nine (measured 143 SM cycles per
-// warp).  Outside the normal range: sqrt().
+// warp).  Below 2^-900, where the residuals would lose bits, and for infinity: sqrt().
 __device__ __forceinline__ double sqrt_pos(double x) {
   const int h = __double2hiint(x);
-  if (unsigned(h - 0x00100000) >= 0x7fe00000u) return gt0(x) ? sqrt(x) : 0.0;
+  if (unsigned(h - 0x07b00000) >= 0x78400000u) return gt0(x) ? sqrt(x) : 0.0;
 #ifdef __CUDA_ARCH__
   double y;
   asm("rsqrt.approx.ftz.f64 %0, %1;" : "=d"(y) : "d"(x));
@@ -320,17 +320,29 @@ __device__ __forceinline__ double sqrt_pos(double x) {
 }
 // 1 / x.  FP64: one step r (1 + e + e^2), e = 1 - x r, of the third-order
 // (Halley-type) iteration on the hardware's 20-bit approximation: e^3 is below
-// 2^-60, so the error is the rounding of the last FMA (and x = 0 or inf gives
-// NaN).  Three FP64 instructions, where the division takes five (86 SM cycles
-// per warp).
+// 2^-60, so the error is the rounding of the last FMA.  Three FP64 instructions,
+// where the division takes five (86 SM cycles per warp).  Outside 2^-1000 .. 2^1000
+// the same on x 2^+-200; 0, infinity and NaN have the approximation's own result.
+// (tests/test_gpu_recip.py: within 0.53 units in the last place.)
 __device__ __forceinline__ float recip(float x) { return 1.0f / x; }
 __device__ __forceinline__ double recip(double x) {
 #ifdef __CUDA_ARCH__
-  double r;
-  asm("rcp.approx.ftz.f64 %0, %1;" : "=d"(r) : "d"(x));
-  double e = fma(-x, r, 1.0);
-  e = fma(e, e, e);
-  return fma(r, e, r);
+  auto approx = [](double z) {
+    double r;
+    asm("rcp.approx.ftz.f64 %0, %1;" : "=d"(r) : "d"(z));
+    return r;
+  };
+  auto step = [](double z, double r) {
+    double e = fma(-z, r, 1.0);
+    e = fma(e, e, e);
+    return fma(r, e, r);
+  };
+  const int h = __double2hiint(x) & 0x7fffffff;
+  if (unsigned(h - 0x01700000) >= 0x7d000000u) {
+    const double k = h < 0x3ff00000 ? 1.6069380442589903e60 : 6.223015277861142e-61, z = x * k, r = approx(z);
+    return h >= 0x7ff00000 || z == 0.0 ? r : step(z, r) * k;
+  }
+  return step(x, approx(x));
 #else
   return 1.0 / x;
 #endif
