@@ -9,10 +9,12 @@
 // product of the low limbs is dropped) and one rounding at the end.  A sum over
 // two lines with matrices A and B takes the exponents so that |A| |x| and |B| |y|
 // have one scale, and needs no alignment.  Per term, truncating the value costs
-// at most 2^-56 of the largest max|a| max|x|, rounding the coefficient 2^-57 and
-// the dropped product 2^-56; an FMA chain rounds every partial sum to 2^-53.
-// Against exact rational arithmetic the mean error is half of the FMA chain's
-// (tests/test_fixed_point.py).
+// at most 2^-56 of max|a| times the largest value of that exponent, rounding the
+// coefficient 2^-57 and the dropped product 2^-56; an FMA chain rounds every partial sum
+// to 2^-53.  Against exact rational arithmetic, lines that reach that exponent have
+// half of the FMA chain's mean error (tests/test_fixed_point.py); the element kernel's
+// exponent is that of the element and variable, and it sees to lines further down
+// (kSpareBits in cr_local64.cuh; tests/test_fixed_point_range.py).
 //
 // Conversions between FP64 and integers or FP32 run on the same FP64 pipe (18
 // cycles), so those are done on the bit patterns as well.
@@ -95,6 +97,8 @@ CRK_HD void fix_mad(FixAcc& acc, int2 x, int2 a) {
   acc.m += (long long)x.x * a.y;
   acc.m += (long long)x.y * a.x;
 }
+// (the mixed products start at half a unit, so that their shift rounds)
+CRK_HD FixAcc fix_zero() { return FixAcc{0, 1ll << (kLimb - 1)}; }
 CRK_HD long long fix_sum(const FixAcc& acc) { return acc.h + (acc.m >> kLimb); }
 
 // r 2^(e - 1023) rounded to FP64 (nearest, ties away from zero), |r| < 2^63;

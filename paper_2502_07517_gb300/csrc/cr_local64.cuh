@@ -10,7 +10,8 @@
 //   - the D contractions and the face traces (40% of the FP64 work) run in
 //     fixed point on the integer pipe (cr_fixed.cuh); the FR volume term takes
 //     each stage's fluxes with b_i in its matrices and accumulates in fixed
-//     point, so the time-averaged fluxes are never formed;
+//     point, so the time-averaged fluxes are never formed; elements whose values
+//     spread too far for a common exponent take their stages in FP64 (stages_fp64);
 //   - the trace of the time-averaged solution is the average of the stage
 //     traces, and the wave speed of the u^n trace shares the first stage's flux;
 //   - which of the three slopes minmod takes, which of two wave speeds is the
@@ -27,15 +28,10 @@
 //     and the face kernel forms the FP64 data itself where the inequality is not
 //     clear (exact_face_data).  The update is the same: alpha = 0 leaves the
 //     high-order part alone, and theta is decided as in FP64.
-// Measured (k_local, the same workload): the contractions and the first decisions
-// 12.57 -> 8.42 ms (612 FP64 instructions per point), the low-order scheme in FP32
-// -> 5.60 ms, traces and volume term on the integer pipe as well (251 FP64
-// instructions, 56% of the pipe, 28% of the issue slots: latency bound) -> 5.03
-// ms, the stage residuals in shared memory and a third resident block -> 4.51 ms,
-// neighbour data and tables loaded by all threads at once -> 4.35 ms, the N = 4
-// stage sums in integers -> 4.15 ms; ten-moment
-// N = 3 at 256 x 256 2.61 -> 1.42 ms (1.38 with a third resident block); 1D Euler N = 4, whole step, 4,000 elements 53
-// -> 49 us, 60,000 elements 314 -> 163 us.
+// k_local, before (the general body in FP64) and now: 2D Euler N = 4, 512 x 512, 12.57
+// and 4.1 ms (58% of the FP64 pipe, 37% of the issue slots: latency bound);
+// ten-moment N = 3, 256 x 256, 2.61 and 1.52 ms; 1D Euler N = 4, whole step, 4,000 elements
+// 53 and 51 us, 60,000 elements 314 and 163 us.
 #pragma once
 #include "cr_common.cuh"
 #include "cr_fixed.cuh"
@@ -355,7 +351,181 @@ __host__ __device__ constexpr size_t local64_extra(int epb) {
   constexpr size_t src = (EQ::M == 6 || HasGravity<EQ>::value ? EQ::M * (DIM == 2 ? n * n : n) : 0)  // the averaged source,
                          + (N == 4 ? 3 * EQ::M * (DIM == 2 ? n * n : n) : 0);                      // stage residuals
   return (size_t)epb * (1 + src) * sizeof(double) + (size_t)(2 * (1 + S) * n * n + 2 * n) * sizeof(int2) +
-         (size_t)(S * S + 4 * n) * sizeof(double) + (size_t)epb * (5 + 2 * EQ::M) * sizeof(int);
+         (size_t)(S * S + 4 * n) * sizeof(double) + (size_t)epb * (6 + 2 * EQ::M) * sizeof(int);
+}
+
+// A sum in fixed point is as good as FP64's as long as its largest term lies within
+// 2^kSpareBits (a trace: 2^kSpareTrace) of the element's largest value of that variable.
+// Error against the FMA chain's, root mean square, for sums so far down, N = 1 .. 4:
+// smooth lines 0.22, 0.44, 1.09, 0.30, random ones 0.47 to 0.67, lines through 0 0.55 to
+// 0.85; traces 0.73 to 1.02.  An element with a node whose two lines of fluxes, which
+// enter one sum, both lie below that, but not all at 0, takes its stages in FP64
+// (stages_fp64), unless four units of the sum times dt are below half a unit of the
+// node's value, which they are added to.  So does one with such a line of a trace, unless
+// the trace's unit, as it enters the update (at most by 1 / dt), is below that of the flux
+// sums.  Ten-moment data of steep cells (64 x 64, N = 3): 2 to 6% of the elements; shear
+// through 0 beside gravity: none.
+constexpr int kSpareBits = 2, kSpareTrace = 3;
+
+// Whether a sum of this node's has lost bits: small has, per variable v, bit 2v where
+// the node's own fluxes are below the line, 2v + 1 where its stage state is.  Out of line:
+// few nodes are so small.
+template <int DIM, int N, int M, int STRIDE>
+__device__ __noinline__ bool sums_lose_bits(const int2* xA, int line_x, int line_y, unsigned small) {
+  constexpr int n = N + 1;
+  const int2* xB = xA + M * STRIDE;
+  const int2* xC = xB + M * STRIDE;
+  int top, any;
+  auto look = [&](const int2* X, int base, int step) {
+#pragma unroll 1
+    for (int r = 0; r < n; ++r) {
+      const int2 x = X[base + step * r];
+      top = max(top, abs(x.x));
+      any |= x.x | x.y;
+    }
+  };
+  bool lost = false;
+#pragma unroll 1
+  for (int v = 0; v < M; ++v) {
+#pragma unroll 1
+    for (int c = 0; c < (DIM == 2 ? 3 : 2); ++c) {  // the fluxes' sum, the traces along x and y
+      if (!((small >> (2 * v + (c > 0))) & 1u)) continue;
+      top = any = 0;
+      look((c == 0 ? xB : xA) + v * STRIDE, c == 2 ? line_y : line_x, c == 2 ? n : 1);
+      if (DIM == 2 && c == 0) look(xC + v * STRIDE, line_y, n);
+      lost = lost || (top < (1 << (28 - (c == 0 ? kSpareBits : kSpareTrace))) && any != 0);
+    }
+  }
+  return lost;
+}
+
+// The stages, traces and the high-order part of the update in FP64 throughout, for the
+// elements of the block with redo set: the same quantities as the fixed-point stages
+// of local_body_f64, which they overwrite in memory (where the element is blended,
+// P.b.P comes with the low-order residual).  Every thread of the block calls it; s0
+// holds u^n, the three arrays behind it are free; alpha: the elements' coefficients.
+template <int DIM, int N, class EQ, int T>
+__device__ __noinline__ void stages_fp64(const KParams<double>& P, const Tab<double>& tb, int blk, double* s0,
+                                         const double* alpha, const int* redo) {
+  constexpr int n = N + 1, NP = DIM == 2 ? n * n : n, M = EQ::M, S = Tableau<N>::S;
+  constexpr int NSIDE = 2 * DIM, NFN = DIM == 2 ? n : 1, NSLOT = NSIDE * NFN, SPT = (NSLOT + NP - 1) / NP;
+  constexpr int epb = (T + NP - 1) / NP, epr = T / NP, stride = epb * NP, arr = M * stride;
+  using TB = Tableau<N>;
+  const Mesh& m = P.m;
+  const int tid = threadIdx.x, el = tid / NP, k = tid - el * NP, p = DIM == 2 ? k % n : k, q = DIM == 2 ? k / n : 0;
+  const int e = blk * epr + el, line_x = el * NP + n * q, line_y = el * NP + p;
+  const bool on = el < epr && e < m.ne && redo[el];
+  const double dt = P.b.ctl->dt_step, a = on && ((m.limiter & kLimBlend) || m.alpha_mode == 1) ? alpha[el] : 0.0;
+  double* sA = s0 + arr;
+  double* sB = sA + arr;
+  double* sC = sB + arr;
+  const bool has_src = (M == 6 && m.source == 1) || (HasGravity<EQ>::value && m.source == 2);
+  double dWx = m.grav[0], dWy = m.grav[1];
+  if (M == 6 && has_src) {
+    const double x = m.x0 + (e % m.nx + tb.xi[p]) * m.dx, y = DIM == 2 ? m.y0 + (e / m.nx + tb.xi[q]) * m.dy : 0.0;
+    source_grad<DIM, double>(m, x - m.src_cx, DIM == 2 ? y - m.src_cy : 0.0, &dWx, &dWy);
+  }
+  double L[S][M], Fa[M], Ga[M], Sa[M], ea[SPT][M], Ut[SPT][M];
+  for (int v = 0; v < M; ++v) {
+    Fa[v] = Ga[v] = Sa[v] = 0.0;
+    for (int mm = 0; mm < SPT; ++mm) ea[mm][v] = Ut[mm][v] = 0.0;
+  }
+#pragma unroll 1
+  for (int i = 0; i < S; ++i) {
+    const double b = TB::b(i);
+    double src[M];
+    if (on) {
+      double u[M], f[M], g[M];
+      vld_sh<M, stride>(u, s0 + tid);
+      for (int j = 0; j < i; ++j) vfma(u, -dt * TB::a(i, j), L[j]);
+      if (DIM == 2) EQ::flux_xy(u, f, g, P.ph);
+      else EQ::flux(u, 0, f, P.ph);
+      vst_sh<M, stride>(sA + tid, u);
+      vst_sh<M, stride>(sB + tid, f);
+      vfma(Fa, b, f);
+      if (DIM == 2) {
+        vst_sh<M, stride>(sC + tid, g);
+        vfma(Ga, b, g);
+      }
+      if (has_src) {
+        source_eval<EQ>(u, dWx, dWy, src);
+        vfma(Sa, b, src);
+      }
+    }
+    __syncthreads();
+    if (on && i < S - 1) {
+#pragma unroll
+      for (int v = 0; v < M; ++v) {
+        double h = 0.0;
+#pragma unroll
+        for (int r = 0; r < n; ++r) h = fma(P.ds.Dx[p * n + r], sB[v * stride + line_x + r], h);
+        if (DIM == 2)
+#pragma unroll
+          for (int r = 0; r < n; ++r) h = fma(P.ds.Dy[q * n + r], sC[v * stride + line_y + n * r], h);
+        L[i][v] = has_src ? h - src[v] : h;
+      }
+    }
+    if (i == 0 || b != 0.0) {
+#pragma unroll
+      for (int mm = 0; mm < SPT; ++mm) {
+        const FaceSlot fs = face_slot<NSLOT, NFN>(tid + mm * T);
+        const int eg = blk * epr + fs.el;
+        if (fs.el >= epr || eg >= m.ne || !redo[fs.el]) continue;
+        const int side = fs.side, j = fs.j, base = fs.el * NP + (side < 2 ? n * j : j), step = side < 2 ? 1 : n;
+        auto trace = [&](const double* X, double (&t)[M]) {
+#pragma unroll
+          for (int v = 0; v < M; ++v) {
+            t[v] = 0.0;
+#pragma unroll
+            for (int r = 0; r < n; ++r) t[v] = fma((side & 1) ? tb.l1[r] : tb.l0[r], X[v * stride + base + step * r], t[v]);
+          }
+        };
+        double ut[M], fn[M];
+        trace(sA, ut);
+        if (i == 0) {
+          P.b.slot[slot_index(0, side, eg, j, NSIDE, m.ne, NFN)] = EQ::speed(ut, side >> 1, P.ph);
+          if (m.dissipation == 1)
+            for (int v = 0; v < M; ++v) P.b.slot[slot_index(1 + v, side, eg, j, NSIDE, m.ne, NFN)] = ut[v];
+        }
+        if (b == 0.0) continue;
+        vfma(Ut[mm], b, ut);
+        if (m.dissipation == 2)
+          for (int v = 0; v < M; ++v) P.b.slot[slot_index(1 + 4 * M + i * M + v, side, eg, j, NSIDE, m.ne, NFN)] = ut[v];
+        if (m.central == 0) EQ::flux(ut, side >> 1, fn, P.ph);
+        else trace(side < 2 ? sB : sC, fn);
+        vfma(ea[mm], b, fn);
+      }
+    }
+    __syncthreads();
+  }
+  vst_sh<M, stride>(sB + tid, Fa);
+  if (DIM == 2) vst_sh<M, stride>(sC + tid, Ga);
+  __syncthreads();
+  if (on) {
+#pragma unroll
+    for (int v = 0; v < M; ++v) {
+      double h = 0.0;
+#pragma unroll
+      for (int r = 0; r < n; ++r) h = fma(P.ds.Dtx[p * n + r], sB[v * stride + line_x + r], h);
+      if (DIM == 2)
+#pragma unroll
+        for (int r = 0; r < n; ++r) h = fma(P.ds.Dty[q * n + r], sC[v * stride + line_y + n * r], h);
+      h = fma(-(dt * (1.0 - a)), h, s0[v * stride + tid]);
+      if (has_src) h = fma(dt, Sa[v], h);
+      double* val = P.b.P + ((size_t)v * m.ne + e) * NP + k;
+      *val = gt0(a) ? fma(-(dt * a), *val, h) : h;
+    }
+  }
+#pragma unroll
+  for (int mm = 0; mm < SPT; ++mm) {
+    const FaceSlot fs = face_slot<NSLOT, NFN>(tid + mm * T);
+    const int eg = blk * epr + fs.el;
+    if (fs.el >= epr || eg >= m.ne || !redo[fs.el]) continue;
+    for (int v = 0; v < M; ++v) {
+      if (m.dissipation != 1) P.b.slot[slot_index(1 + v, fs.side, eg, fs.j, NSIDE, m.ne, NFN)] = Ut[mm][v];
+      P.b.slot[slot_index(1 + M + v, fs.side, eg, fs.j, NSIDE, m.ne, NFN)] = ea[mm][v];
+    }
+  }
 }
 
 template <int DIM, int N, class EQ, int T>
@@ -406,13 +576,14 @@ __device__ __forceinline__ void local_body_f64(const KParams<double>& P, const T
   int* sNbr = reinterpret_cast<int*>(sWy + n);                // [epb][4]
   int* sKey = sNbr + epb * 4;                                 // exponents [fluxes, state][epb][M]
   int* sFull = sKey + 2 * epb * M;                            // [epb] low-order scheme in FP64
+  int* sRedo = sFull + epb;                                   // [epb] stages to be done in FP64
 
   double un[M];
 #pragma unroll
   for (int v = 0; v < M; ++v) un[v] = P.b.u[((size_t)v * m.ne + ee) * NP + k];
   for (int t = tid; t < 2 * epb * M; t += T) sKey[t] = 0;
   for (int t = tid; t < epb; t += T) {
-    sFull[t] = 0;
+    sFull[t] = sRedo[t] = 0;
     sAlpha[t] = m.alpha_mode == 1 ? m.alpha_fixed : 0.0;
   }
   __syncthreads();
@@ -515,14 +686,20 @@ __device__ __forceinline__ void local_body_f64(const KParams<double>& P, const T
   int* const kf = sKey + el * M;
   int* const ku = kf + epb * M;
   const int o0 = P.ds.oD[0], o1 = DIM == 2 ? P.ds.oD[1] : o0;
-  const int kmin = kMinLineExp + max(o0, o1), kmax = kMaxLineExp + min(o0, o1);
+  const int kmin = kMinLineExp + max(o0, o1), kmax = kMaxLineExp + min(o0, o1), exp_dt = exp_of(dt) - 1023;
 
   // The fluxes of this node, and where its traces are wanted the stage state,
   // into the node arrays in fixed point, and a barrier.  An element keeps its
   // exponents from the first stage until a value needs two more bits; then
-  // (rarely: the vote) it takes the larger ones.
+  // (rarely: the vote) it takes the larger ones.  An element in which a sum of this
+  // stage loses bits, or whose exponents are out of range, is marked for stages_fp64.
   auto put_nodes = [&](const double (&f)[M], const double (&g)[M], const double (&u)[M], int i, bool traces) {
     const bool first = i == 0;
+    auto check_range = [&]() {
+#pragma unroll
+      for (int v = 0; v < M; ++v)
+        if (kf[v] > kmax || ku[v] > kMaxLineExp) sRedo[el] = 1;
+    };
     if (first) {
 #pragma unroll
       for (int v = 0; v < M; ++v) {
@@ -530,23 +707,46 @@ __device__ __forceinline__ void local_body_f64(const KParams<double>& P, const T
         atomicMax(ku + v, max(exp_of(u[v]), kMinLineExp));
       }
       __syncthreads();
+      check_range();
     }
-    unsigned over = 0u;  // bit 2v: f[v] or g[v] outgrew the exponent, 2v + 1: u[v]
+    // bits 2v: f[v] and g[v] (the larger one), 2v + 1: u[v]: outside the spare bits below
+    // the exponent and the one above; over: above; small: below (sums_lose_bits)
+    unsigned odd = 0u, over = 0u, small = 0u;
     auto put_all = [&]() {
 #pragma unroll
       for (int v = 0; v < M; ++v) {
-        const int E = kf[v];
-        over |= unsigned((DIM == 2 ? max(exp_of(f[v]) + o0, exp_of(g[v]) + o1) : exp_of(f[v]) + o0) > E + 1) << (2 * v);
+        const int E = kf[v], own = DIM == 2 ? max(exp_of(f[v]) + o0, exp_of(g[v]) + o1) : exp_of(f[v]) + o0;
+        odd |= unsigned(unsigned(own - (E - kSpareBits)) > unsigned(kSpareBits + 1)) << (2 * v);
         xB[v * stride + tid] = to_fixed(f[v], E - o0);
         if (DIM == 2) xC[v * stride + tid] = to_fixed(g[v], E - o1);
         if (traces) {
           const int Eu = ku[v];
-          over |= unsigned(exp_of(u[v]) > Eu + 1) << (2 * v + 1);
+          odd |= unsigned(unsigned(exp_of(u[v]) - (Eu - kSpareTrace)) > unsigned(kSpareTrace + 1)) << (2 * v + 1);
           xA[v * stride + tid] = to_fixed(u[v], Eu);
         }
       }
     };
+    auto sort_out = [&]() {  // (and a number below the unit becomes one unit: it is not 0)
+      over = small = 0u;
+      auto unit = [](double x) { return make_int2(0, (__double_as_longlong(x) << 1) == 0 ? 0 : (__double2hiint(x) >> 31) | 1); };
+#pragma unroll
+      for (int v = 0; v < M; ++v) {
+        const int E = kf[v], xf = exp_of(f[v]) + o0, xg = DIM == 2 ? exp_of(g[v]) + o1 : xf, own = max(xf, xg);
+        over |= unsigned(own > E + 1) << (2 * v);
+        // (the unit of a sum is 2^E, that of a product in it 2^(E + 57))
+        small |= unsigned(own < E - kSpareBits && E + exp_dt + 56 > exp_of(u[v])) << (2 * v);
+        if (xf < E - 57) xB[v * stride + tid] = unit(f[v]);
+        if (DIM == 2 && xg < E - 57) xC[v * stride + tid] = unit(g[v]);
+        if (traces) {
+          const int Eu = ku[v], xu = exp_of(u[v]);
+          over |= unsigned(xu > Eu + 1) << (2 * v + 1);
+          small |= unsigned(xu < Eu - kSpareTrace && Eu - exp_dt > E + 57) << (2 * v + 1);
+          if (xu < Eu - 57) xA[v * stride + tid] = unit(u[v]);
+        }
+      }
+    };
     put_all();
+    if (odd) sort_out();
     if (first) {
       __syncthreads();
     } else if (__syncthreads_or(valid && over)) {
@@ -561,6 +761,8 @@ __device__ __forceinline__ void local_body_f64(const KParams<double>& P, const T
       }
       __syncthreads();
       put_all();
+      sort_out();
+      check_range();
 #pragma unroll
       for (int v = 0; v < M; ++v) {
         const int d = min(63, kf[v] - before[v]);
@@ -572,14 +774,14 @@ __device__ __forceinline__ void local_body_f64(const KParams<double>& P, const T
       }
       __syncthreads();
     }
+    if (small && valid && sums_lose_bits<DIM, N, M, stride>(xA, line_x, line_y, small)) sRedo[el] = 1;
   };
-  const double kNaN = __longlong_as_double(0x7ff8000000000000ll);
   // Trace along the line (base, step) of node values X with exponent E.
   auto trace_dot = [&](const int2* X, int E, int base, int step, const int2* l) -> double {
-    FixAcc acc{0, 0};
+    FixAcc acc = fix_zero();
 #pragma unroll
     for (int r = 0; r < n; ++r) fix_mad(acc, X[base + step * r], l[r]);
-    return E > kMaxLineExp ? kNaN : from_fixed(fix_sum(acc), E + P.ds.oL);
+    return from_fixed(fix_sum(acc), E + P.ds.oL);
   };
 
 #pragma unroll
@@ -613,8 +815,7 @@ __device__ __forceinline__ void local_body_f64(const KParams<double>& P, const T
           }
           sum += rest >> low;
         }
-        const int E = kf[v];
-        ui[v] = E > kmax ? kNaN : fma(-sAdt[i], from_fixed(sum, E + (i >= 4 ? low : 0)), ui[v]);
+        ui[v] = fma(-sAdt[i], from_fixed(sum, kf[v] + (i >= 4 ? low : 0)), ui[v]);
       }
     } else {
 #pragma unroll
@@ -647,7 +848,7 @@ __device__ __forceinline__ void local_body_f64(const KParams<double>& P, const T
       const int W = M - v0 < 2 ? M - v0 : 2;
       FixAcc lo[2], hi[2];
 #pragma unroll
-      for (int w = 0; w < 2; ++w) lo[w] = hi[w] = FixAcc{0, 0};
+      for (int w = 0; w < 2; ++w) lo[w] = hi[w] = fix_zero();
 #pragma unroll
       for (int d = 0; d < DIM; ++d) {
 #pragma unroll
@@ -677,8 +878,7 @@ __device__ __forceinline__ void local_body_f64(const KParams<double>& P, const T
             else reinterpret_cast<long long*>(i == 3 ? sD : sL + i * arr)[v * stride + tid] = r;
             continue;
           }
-          const int E = kf[v];
-          double L = E > kmax ? kNaN : from_fixed(fix_sum(lo[w]), E);
+          double L = from_fixed(fix_sum(lo[w]), kf[v]);
           if (kSrcEq && has_src) L -= src[v];
           if (kShL && i < 4) (i == 3 ? sD : sL + i * arr)[v * stride + tid] = L;
           else Lst[i < S - 1 ? i : 0][v] = L;
@@ -737,8 +937,7 @@ __device__ __forceinline__ void local_body_f64(const KParams<double>& P, const T
     const double dho = dt * (1.0 - a);
 #pragma unroll
     for (int v = 0; v < M; ++v) {
-      const int E = kf[v];
-      double h = E > kmax ? kNaN : fma(-dho, from_fixed(ho[v], E + P.ds.oDt), s0[v * stride + tid]);
+      double h = fma(-dho, from_fixed(ho[v], kf[v] + P.ds.oDt), s0[v * stride + tid]);
       if (SRC && has_src) h = fma(dt, sS[v * stride + tid], h);
       if (valid) P.b.P[((size_t)v * m.ne + e) * NP + k] = h;
     }
@@ -852,7 +1051,7 @@ __device__ __forceinline__ void local_body_f64(const KParams<double>& P, const T
 #pragma unroll
       for (int v = 0; v < M; ++v) {
         double* val = P.b.P + ((size_t)v * m.ne + e) * NP + k;
-        *val = fma(-(dt * a), LO[v], *val);
+        *val = sRedo[el] ? LO[v] : fma(-(dt * a), LO[v], *val);  // (stages_fp64 adds it to its high-order part)
       }
     }
     // face-node data for the face kernel: evolved boundary state u* and the
@@ -893,6 +1092,9 @@ __device__ __forceinline__ void local_body_f64(const KParams<double>& P, const T
       }
     }
   }
+  // (at the end, where least is alive: called behind the stages it cost 5% of the
+  // kernel where no element needs it)
+  if (__syncthreads_or(valid && sRedo[el])) stages_fp64<DIM, N, EQ, T>(P, tb, blk, s0, sAlpha, sRedo);
 }
 
 }  // namespace crk
