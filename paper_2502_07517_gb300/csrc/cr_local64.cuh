@@ -216,7 +216,9 @@ __device__ __noinline__ void put_hancock_states(const KParams<double>& P, const 
 
 // The same in FP32, for elements whose low-order scheme only feeds the screen of
 // the flux limiter (see the body).  Returns false where admissibility is not
-// clear in FP32 (the FP64 form then decides).
+// clear in FP32, by the margin that the limiter's bases need, or a boundary node and
+// its neighbour inside the element are too unlike for those (like_neighbour); the FP64
+// form then decides.
 template <int DIM, int N, class EQ, class Nb>
 __device__ __forceinline__ bool hancock_states_f32(const Mesh& m, const Phys<float>& ph, const Tab<double>& tb,
                                                    const float (&un)[EQ::M], float alpha, int p, int q, float hx,
@@ -225,7 +227,25 @@ __device__ __forceinline__ bool hancock_states_f32(const Mesh& m, const Phys<flo
   constexpr int M = EQ::M;
 #pragma unroll
   for (int v = 0; v < M; ++v) xm[v] = xp[v] = ym[v] = yp[v] = un[v];
-  if (!(m.limiter & kLimMH)) return EQ::K == 0 || un[0] > 1e-30f;
+  bool ok = true;
+  if constexpr (EQ::K > 0) {
+#pragma unroll
+    for (int dir = 0; dir < DIM; ++dir) {
+      const int c = dir == 0 ? p : q;
+#pragma unroll
+      for (int v = 0; v < M; ++v)
+        if (v == 0 || v == M - 1 || (M == 6 && v == 3)) {
+          if (c == 0) ok = ok && like_neighbour<EQ>(v, un[v], nb(v, dir, 1));
+          if (c == N) ok = ok && like_neighbour<EQ>(v, un[v], nb(v, dir, 0));
+        }
+    }
+  }
+  if (!(m.limiter & kLimMH)) {
+    float A[M];
+#pragma unroll
+    for (int v = 0; v < M; ++v) A[v] = fabsf(un[v]);
+    return ok && clearly_admissible<EQ>(un, A, kLikeF);
+  }
   const float beta = 2.0f - alpha;
   float sx[M], sy[M], A[M];
   auto slopes = [&](float (&sl)[M], int c, int dir) {
@@ -257,15 +277,16 @@ __device__ __forceinline__ bool hancock_states_f32(const Mesh& m, const Phys<flo
   }
 #pragma unroll
   for (int v = 0; v < M; ++v) A[v] = fabsf(un[v]) + fabsf(sx[v]) + (DIM == 2 ? fabsf(sy[v]) : 0.0f) + fabsf(ex[v]);
-  bool ok = clearly_admissible<EQ>(xm, A) && clearly_admissible<EQ>(xp, A);
+  auto clear = [&](const float (&s)[M]) { return clearly_admissible<EQ>(s, A, kLikeF); };
+  ok = ok && clear(xm) && clear(xp);
   vsub(xm, xm, ex);
   vsub(xp, xp, ex);
-  ok = ok && clearly_admissible<EQ>(xm, A) && clearly_admissible<EQ>(xp, A);
+  ok = ok && clear(xm) && clear(xp);
   if (DIM == 2) {
-    ok = ok && clearly_admissible<EQ>(ym, A) && clearly_admissible<EQ>(yp, A);
+    ok = ok && clear(ym) && clear(yp);
     vsub(ym, ym, ex);
     vsub(yp, yp, ex);
-    ok = ok && clearly_admissible<EQ>(ym, A) && clearly_admissible<EQ>(yp, A);
+    ok = ok && clear(ym) && clear(yp);
   }
   return ok;
 }

@@ -153,23 +153,24 @@ __device__ __forceinline__ void flux_c2_f32(const float* u, int dir, float* f, f
 
 // FP32 screen of the MUSCL-Hancock states: s is a state and A bounds the
 // magnitudes its parts are summed from.  True only when the state is admissible
-// by a margin above the FP32 rounding of the sums and products.  The products are
+// by a margin above the FP32 rounding of the sums and products (by: more of one).  The products are
 // of second order in the state (ten-moment: fourth), so their margin, too, has to be
 // in FP32's range: near vacuum (rho p below 1e-25, ten-moment 1e-13) nothing is clear.
 template <class EQ>
-__device__ __forceinline__ bool clearly_admissible(const float* s, const float* A) {
+__device__ __forceinline__ bool clearly_admissible(const float* s, const float* A, float by = kMarginF) {
   if constexpr (EQ::K == 0) return true;
-  if (!(s[0] > kMarginF * A[0] && A[0] > kTinyF)) return false;
+  if (!(s[0] > by * A[0] && A[0] > kTinyF)) return false;
   if constexpr (IsEuler<EQ>::value) {
     constexpr int E = EQ::M - 1;
     const float k2 = E == 3 ? s[1] * s[1] + s[2] * s[2] : s[1] * s[1], a2 = E == 3 ? A[1] * A[1] + A[2] * A[2] : A[1] * A[1];
-    const float margin = kMarginF * (A[E] * A[0] + a2);
+    const float margin = by * (A[E] * A[0] + a2);
     return fminf(A[E], margin) > kTinyF && s[E] * s[0] - 0.5f * k2 > margin;
   } else if constexpr (EQ::M == 6) {
     const float a11 = 2.0f * s[0] * s[3] - s[1] * s[1], a22 = 2.0f * s[0] * s[5] - s[2] * s[2];
     const float a12 = 2.0f * s[0] * s[4] - s[1] * s[2], a345 = A[3] + A[4] + A[5];
     const float B = 2.0f * A[0] * a345 + A[1] * A[1] + A[2] * A[2], margin = 5.0f * kMarginF * B * B;
-    return fminf(a345, margin) > kTinyF && a11 > kMarginF * B && a11 * a22 - a12 * a12 > margin;
+    const float b11 = 2.0f * A[0] * A[3] + A[1] * A[1], b22 = 2.0f * A[0] * A[5] + A[2] * A[2];  // (by: of each pressure)
+    return fminf(a345, margin) > kTinyF && a11 > fmaxf(kMarginF * B, by * b11) && a22 > by * b22 && a11 * a22 - a12 * a12 > margin;
   }
   return true;
 }
@@ -208,6 +209,48 @@ __device__ __forceinline__ void screened_constraint(const float* s, const float*
   }
 }
 
+// Rusanov flux of two states in FP32, and per variable the magnitudes its rounding
+// (truncated states included) is kMarginF of: besides the fluxes and jumps themselves
+// the energies, of which pressures are differences, and those times the speeds; and
+// what the sound speed loses in that difference, up to 1.1e-6 V^2 / c with V^2 = 2 E /
+// rho (Mach 30: half of the rest).
+template <class EQ>
+__device__ __forceinline__ void rusanov_f32(const float* uL, const float* uR, int dir, const Phys<float>& ph, float* lo,
+                                            float* a) {
+  constexpr int M = EQ::M, E = M == 3 ? 2 : 3;
+  float fL[M], fR[M], vL, vR, c2L, c2R;
+  flux_c2_f32<EQ>(uL, dir, fL, &vL, &c2L, ph);
+  flux_c2_f32<EQ>(uR, dir, fR, &vR, &c2R, ph);
+  const float cL = sqrt_f32(c2L), cR = sqrt_f32(c2R);
+  const float lam = fmaxf(fabsf(vL) + cL, fabsf(vR) + cR);
+  float SL = 0.0f, SR = 0.0f;
+#pragma unroll
+  for (int v = E; v < M; ++v) {
+    SL += fabsf(uL[v]);
+    SR += fabsf(uR[v]);
+  }
+  const float S = 2.0f * (SL + SR), V2 = 2.0f * fmaxf(SL / uL[0], SR / uR[0]);
+  const float V = fmaxf(lam, sqrt_f32(V2)), jump = lam + 0.03f * V2 * rcp_f32(fminf(cL, cR));
+#pragma unroll
+  for (int v = 0; v < M; ++v) {
+    lo[v] = 0.5f * (fL[v] + fR[v]) - 0.5f * lam * (uR[v] - uL[v]);
+    a[v] = fabsf(fL[v]) + fabsf(fR[v]) + jump * (fabsf(uL[v]) + fabsf(uR[v])) + (v == 0 ? 0.0f : v < E ? S : S * V);
+  }
+}
+
+// Whether a node next to u's inside the element is like it: the limiter's bases in
+// FP32 (hancock_states_f32) hold the subcell flux between the two, whose rounding the
+// margin of the face does not see.  With the density within a factor of 2, energies at
+// most twice as large and both states admissible by kLikeF (Mach 25), it is below that
+// margin.
+constexpr float kLikeF = 2e-3f;
+template <class EQ>
+__device__ __forceinline__ bool like_neighbour(int v, float u, float nb) {
+  constexpr int E = EQ::M - 1;
+  if (v == 0) return nb <= 2.0f * u && u <= 2.0f * nb;
+  return !(v == E || (EQ::M == 6 && v == 3)) || nb <= 2.0f * u;
+}
+
 // Whether the flux limiter of an interior face is clearly idle (theta = 1) for
 // the flux F: both candidates base -+ c F clear a tenth of the smaller
 // low-order candidate (and those are clearly positive) in every constraint.
@@ -221,27 +264,12 @@ __device__ __forceinline__ bool flux_limiter_idle(const float* uL, const float* 
   Phys<float> ph;
   ph.gamma = trunc_f32(phd.gamma);
   ph.gm1 = trunc_f32(phd.gm1);
-  float fL[M], fR[M], sL, sR, lo[M], aL[M], aR[M];
-  EQ::flux_speed(uL, dir, fL, &sL, ph);
-  EQ::flux_speed(uR, dir, fR, &sR, ph);
-  const float lam = fmaxf(sL, sR);
-  // magnitudes the fluxes are summed from: besides their own size, the energies
-  // (pressures are differences of energies) and those times the speeds
-  float SL = 0.0f, SR = 0.0f;
-#pragma unroll
-  for (int v = M == 3 ? 2 : 3; v < M; ++v) {
-    SL += fabsf(uL[v]);
-    SR += fabsf(uR[v]);
-  }
-  const float S = 2.0f * (SL + SR);
-  const float V = fmaxf(lam, sqrt_f32(2.0f * fmaxf(SL / uL[0], SR / uR[0])));
+  float lo[M], a[M], aL[M], aR[M];
+  rusanov_f32<EQ>(uL, uR, dir, ph, lo, a);
 #pragma unroll
   for (int v = 0; v < M; ++v) {
-    lo[v] = 0.5f * (fL[v] + fR[v]) - 0.5f * lam * (uR[v] - uL[v]);
-    const float a = fabsf(fL[v]) + fabsf(fR[v]) + lam * (fabsf(uL[v]) + fabsf(uR[v])) + fabsf(F[v]) +
-                    (v == 0 ? 0.0f : v < (M == 3 ? 2 : 3) ? S : S * V);
-    aL[v] = fabsf(bL[v]) + cL * a;
-    aR[v] = fabsf(bR[v]) + cR * a;
+    aL[v] = fabsf(bL[v]) + cL * (a[v] + fabsf(F[v]));
+    aR[v] = fabsf(bR[v]) + cR * (a[v] + fabsf(F[v]));
   }
   bool idle = fminf(cL, cR) > kTinyF;
 #pragma unroll

@@ -68,6 +68,28 @@ double constraint(const double* u, int m) {
   ph.gm1 = 0.4;
   return m == 4 ? Euler::constraint(u, 1, ph) : EqTenMoment::constraint(u, 1, ph);
 }
+void low_flux(const double* d, int m, float* lo, float* a) {  // uL, uR
+  float x[2][6];
+  for (int i = 0; i < 2; ++i)
+    for (int v = 0; v < m; ++v) x[i][v] = trunc_f32(d[i * m + v]);
+  Phys<float> ph{};
+  ph.gamma = 1.4f;
+  ph.gm1 = 0.4f;
+  if (m == 4) rusanov_f32<Euler>(x[0], x[1], 0, ph, lo, a);
+  else rusanov_f32<EqTenMoment>(x[0], x[1], 0, ph, lo, a);
+}
+int like(const double* d, int m) {  // u, its neighbour: alike, and both admissible by kLikeF
+  float x[2][6], A[2][6];
+  bool ok = true;
+  for (int i = 0; i < 2; ++i)
+    for (int v = 0; v < m; ++v) {
+      x[i][v] = trunc_f32(d[i * m + v]);
+      A[i][v] = fabsf(x[i][v]);
+    }
+  for (int v = 0; v < m; ++v) ok = ok && (m == 4 ? like_neighbour<Euler>(v, x[0][v], x[1][v]) : like_neighbour<EqTenMoment>(v, x[0][v], x[1][v]));
+  for (int i = 0; i < 2; ++i) ok = ok && (m == 4 ? clearly_admissible<Euler>(x[i], A[i], kLikeF) : clearly_admissible<EqTenMoment>(x[i], A[i], kLikeF));
+  return ok;
+}
 double speed(const double* s) { return wave_max(s[0], s[1], s[2], s[3]); }
 double minmod(const double* d, const double* b) {
   return minmod_scaled(d[0], d[1], d[2], b[0], b[1], b[2], trunc_f32(b[0]), trunc_f32(b[1]), trunc_f32(b[2]));
@@ -244,3 +266,37 @@ def test_constraints_are_the_formula(lib, m):
         assert lib.constraint(_p(*u), m) == want
         u[rng.integers(0, m)] = np.nan
         assert np.isnan(lib.constraint(_p(*u), m))
+
+
+@pytest.mark.parametrize("m", [4, 6])
+@pytest.mark.parametrize("unlike", [1.0, 2.0, 10.0, 1e3, 1e6])
+def test_margins_of_the_low_order_fluxes(lib, m, unlike):
+    """The FP32 Rusanov flux of any two states within its own margin, at Mach numbers up
+    to 200; and that between a node and an inner neighbour, where the two are alike,
+    within the margin of a face whose two sides are like the node."""
+    rng = np.random.default_rng(9)
+    f32 = lambda k: (ctypes.c_float * k)()  # noqa: E731
+    seen = 0
+    for it in range(3000):
+        pair = []
+        for i in range(2):
+            rho, mach = unlike ** rng.uniform(-i, i), 10.0 ** rng.uniform(-1.0, 2.3)
+            a, b = rho * unlike ** rng.uniform(-i, i) * np.exp(rng.uniform(-1.0, 1.0, 2))
+            v1, v2 = mach * np.sqrt(1.4 * a / rho) * rng.uniform(-1.0, 1.0, 2)
+            if m == 4:
+                pair.append(np.array([rho, rho * v1, rho * v2, a / 0.4 + 0.5 * rho * (v1 * v1 + v2 * v2)]))
+            else:
+                r = rng.uniform(-0.9, 0.9) * np.sqrt(a * b)
+                pair.append(0.5 * np.array([2 * rho, 2 * rho * v1, 2 * rho * v2, a + rho * v1 * v1, r + rho * v1 * v2,
+                                            b + rho * v2 * v2]))
+        (fL, sL), (fR, sR) = _flux(pair[0]), _flux(pair[1])
+        want = 0.5 * (fL + fR) - 0.5 * max(sL, sR) * (pair[1] - pair[0])
+        lo, a, lo2, a2 = f32(m), f32(m), f32(m), f32(m)
+        lib.low_flux(_p(*np.concatenate(pair)), m, lo, a)
+        err = np.abs(np.array(lo[:], dtype=np.float64) - want)
+        assert not (err > 2e-5 * np.array(a[:])).any(), (it, pair, err, a[:])
+        if lib.like(_p(*np.concatenate(pair)), m):
+            seen += 1
+            lib.low_flux(_p(*np.concatenate([pair[0], pair[0]])), m, lo2, a2)
+            assert not (err > 2e-5 * np.array(a2[:])).any(), (it, pair, err, a2[:])
+    assert seen > 100 or unlike > 2.0
