@@ -63,15 +63,26 @@ struct Impl {
                                 cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem_update(EPB));
   }
 
-  // One-dimensional FP64 meshes with fewer than kSmallNodes solution points:
-  // blocks of kSmallThreads threads.  The kernels are bound by the FP64 pipe of the
-  // SMs that have work, and 256-thread blocks leave SMs idle (1D Euler N = 4, us
-  // per step: 4,000 elements 62 -> 53, 10,000 92 -> 76, but 20,000 133 -> 137 and
-  // 30,000 166 -> 188).  FP32 bulk is latency bound: the same within 1%.
+  static int sm_count() {
+    int dev = 0, n = 0;
+    if (cudaGetDevice(&dev) != cudaSuccess || cudaDeviceGetAttribute(&n, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess)
+      return 152;
+    return n;
+  }
+
+  // One-dimensional FP64 meshes whose blocks of kSmallThreads threads are all resident
+  // at once take those (the kernels are bound by the FP64 pipe of the SMs that have
+  // work, and 256-thread blocks leave SMs idle); past that a second wave begins, where
+  // 256-thread blocks may still fit.  us per step with 64 and 256 threads, 152 SMs: 1D
+  // Euler N = 4 (72,960 nodes at once), 10,000 nodes 63 and 68, 60,000 72 and 75, 77,000 93
+  // and 71, 120,000 100 and 102; N = 2 (76,608) 60,000 62 and 64, 77,000 72 and 60; linear
+  // advection N = 3, 40,000 27 and 29.  FP32 bulk is latency bound: the same within 1%.
   static constexpr bool kHasSmall = DIM == 1 && !MIXED;
   static constexpr int kSmallThreads = 64;
-  static constexpr long long kSmallNodes = 152ll * 512;
-  static bool small(const KParams<real>& P) { return kHasSmall && (long long)P.m.ne * NP < kSmallNodes; }
+  static bool small(const KParams<real>& P) {
+    constexpr int E = BlockShape<NP, kSmallThreads>::EPB;
+    return kHasSmall && (P.m.ne + E - 1) / E <= sm_count() * LB::value * (256 / kSmallThreads);
+  }
 
   // Launch behind the previous kernel of the step (wait_for_previous_kernel).
   template <class... A>
@@ -94,7 +105,7 @@ struct Impl {
     constexpr int E = BlockShape<NP, THREADS>::EPB;
     const int blocks = (P.m.ne + E - 1) / E;
     if constexpr (LB::many > LB::value)  // more blocks than are resident at once: one more per SM
-      if (blocks > 152 * LB::value)
+      if (blocks > sm_count() * LB::value)
         return chain(&k_local<DIM, N, EQ, real, MIXED, THREADS, LB::many>, blocks, E * NP, smem_local(E), s, P);
     return chain(&k_local<DIM, N, EQ, real, MIXED, THREADS>, blocks, E * NP, smem_local(E), s, P);
   }
@@ -113,7 +124,7 @@ struct Impl {
     const KParams<real>& P = *static_cast<const KParams<real>*>(pv);
     const int nfaces = P.m.ny * P.m.nfx * NFN + (DIM == 2 ? P.m.nfy * P.m.nx * n : 0);
     // few face nodes: one warp per block, so that every SM has some
-    const int threads = nfaces < 152 * 4 * 32 ? 32 : 256;
+    const int threads = nfaces < sm_count() * 4 * 32 ? 32 : 256;
     return chain(&k_face<DIM, N, EQ, real>, (nfaces + threads - 1) / threads, threads, 0, s, P);
   }
   static cudaError_t launch_update(const void* pv, cudaStream_t s) {
