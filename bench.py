@@ -44,7 +44,7 @@ NCU_TRAFFIC_PER_ELEMENT = {("fp64", "k_local"): 790.87e6 / 147456, ("fp32", "k_l
 # FP64 flops the FP64 kernel executes per solution point on the FP64 pipe (FMA 2),
 # from the same capture: the contractions run in fixed point on the integer pipe
 # and decisions in FP32, so the algorithmic count is not what the pipe does.
-NCU_FP64_FLOPS_PER_POINT = {"k_local": 345.5}
+NCU_FP64_FLOPS_PER_POINT = {("k_local", 4): 345.5}
 PEAK_FP64_TFLOPS = SM_COUNT * 2 * 2 * SM_MAX_MHZ * 1e6 / 1e12
 PEAK_FP32_TFLOPS = SM_COUNT * 128 * 2 * SM_MAX_MHZ * 1e6 / 1e12
 
@@ -284,12 +284,13 @@ def alu_roofline(prob, nodes, kms, mixed, ms_per_step):
     peak = PEAK_FP32_TFLOPS if mixed else PEAK_FP64_TFLOPS
     mode = "fp32" if mixed else "fp64"
     ne = nodes // (prob["degree"] + 1) ** 2
-    executed = flops[dom] if mixed else NCU_FP64_FLOPS_PER_POINT.get(names[dom], flops[dom])
+    counted = None if mixed else NCU_FP64_FLOPS_PER_POINT.get((names[dom], prob["degree"]))
+    executed = flops[dom] if counted is None else counted
     algorithmic, achieved = achieved, executed * nodes / (kms[dom] * 1e-3) / 1e12
     return {"bound": "alu", "achieved": achieved, "peak": peak, "unit": "TFLOP/s",
             "frac": achieved / peak, "kernel": names[dom],
             "executed_flops_per_point": executed, "algorithmic_tflops": algorithmic,
-            "note": None if mixed else "achieved counts the flops executed on the FP64 pipe; the D contractions and "
+            "note": None if counted is None else "achieved counts the flops executed on the FP64 pipe; the D contractions and "
                     "traces run in fixed point on the integer pipe and screened decisions in FP32, so the "
                     "algorithmic rate is not bounded by that pipe",
             "traffic": (NCU_TRAFFIC_PER_ELEMENT[(mode, names[dom])] * ne

@@ -1709,7 +1709,7 @@ __device__ __noinline__ void limit_block(const KParams<real>& P, const Tab<doubl
     }
     for (int t = 0; t < np2; ++t) {
       if (EQ::constraint(pts[t], 1, P.phd) >= eps2) continue;
-      const double lo = scaling_root<EQ>(ubar, pts[t], eps2, P.phd);
+      const double lo = scaling_root<EQ, MIXED>(ubar, pts[t], eps2, P.phd);
       tmin = OpMinBits()(tmin, lo);
     }
   }

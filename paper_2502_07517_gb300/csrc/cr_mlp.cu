@@ -223,7 +223,9 @@ bool nin_supported(int nin) {
 // Every sum runs in the order of k_mlp_grad and k_mlp_reduce (units and samples
 // ascending, chunk by chunk).
 // Measured (50,000 samples of 16 inputs, batch 512, two epochs, whole call):
-// 7.93 -> 1.82 ms.
+// 7.93 -> 1.82 ms.  Up to 48 chunks (3,072 samples): past that one cluster falls behind
+// the grid of one launch per step (16 inputs, ms per epoch, this kernel and that: 3,073
+// samples 0.63 and 0.75, 6,000 0.59 and 0.50).
 constexpr int kEpochThreads = 352;                       // 11 warps: one gradient item per thread
 constexpr int kMaxCluster = 8, kEpochBlocks = 48;        // chunks per minibatch the kernel takes
 constexpr int kHS = kH + 4;                              // row stride of the hidden arrays (128-bit reads

@@ -37,7 +37,7 @@ template <class EQ> static void both(const double* ubar, const double* pt, doubl
   Phys<double> ph{};
   ph.gm1 = 0.4;
   evaluations = 0;
-  out[0] = scaling_root<Counted<EQ>>(ubar, pt, eps, ph);
+  out[0] = scaling_root<Counted<EQ>, true>(ubar, pt, eps, ph);
   out[1] = evaluations;
   double lo = 0.0, hi = 1.0, u[6];
   for (int i = 0; i < 50; ++i) {
