@@ -38,12 +38,13 @@ MEASURED_PEAKS = os.path.join(ROOT, "MEASURED_PEAKS.json")
 SM_COUNT, SM_MAX_MHZ = 152, 2070.0
 # DRAM bytes (read + write) per element of the dominant kernel, from one ncu
 # capture of the current kernel at 384x384 (147,456 elements; the traffic
-# scales with the element count): FP64 k_local 790.9 MB, FP32 bulk k_local
+# scales with the element count): FP64 k_local 868.0 MB, FP32 bulk k_local
 # 276.1 MB (the k_local summaries under profiles/).
-NCU_TRAFFIC_PER_ELEMENT = {("fp64", "k_local"): 790.87e6 / 147456, ("fp32", "k_local"): 276.13e6 / 147456}
+NCU_TRAFFIC_PER_ELEMENT = {("fp64", "k_local"): 868.05e6 / 147456, ("fp32", "k_local"): 276.13e6 / 147456}
 # FP64 flops the FP64 kernel executes per solution point on the FP64 pipe (FMA 2),
 # from the same capture: the contractions run in fixed point on the integer pipe
-# and decisions in FP32, so the algorithmic count is not what the pipe does.
+# and decisions in FP32, so the algorithmic count is not what the pipe does (kernel
+# and degree that were counted; without a count the algorithmic flops are reported).
 NCU_FP64_FLOPS_PER_POINT = {("k_local", 4): 345.5}
 PEAK_FP64_TFLOPS = SM_COUNT * 2 * 2 * SM_MAX_MHZ * 1e6 / 1e12
 PEAK_FP32_TFLOPS = SM_COUNT * 128 * 2 * SM_MAX_MHZ * 1e6 / 1e12

@@ -83,8 +83,8 @@ __device__ __forceinline__ void face_tile(const BatchArgs<real>& A, KParams<real
   else face_body<2, 4, Eq2, real>(*sP, tile.blk);
 }
 
-// Resident blocks per SM: as the single-problem kernels (MinBlocks), scaled
-// from 256-thread blocks to T threads.
+// Resident blocks per SM: MinBlocks, scaled from 256-thread blocks to T threads.  (In
+// FP64 the single-problem kernels of one degree take more: LocalBlocks, UpdateBlocks.)
 template <typename real, int T, int PHASE>
 struct BatchMinBlocks {
   static constexpr bool MIXED = sizeof(real) == 4;

@@ -873,14 +873,14 @@ using UpdateShape = BlockShape<NP, (MIXED && THREADS > 128 ? 128 : THREADS)>;
 
 // Blocks of the element kernel.  FP64 in two dimensions (cr_local64.cuh): three
 // resident blocks (80 registers) so that one block's integer phases overlap
-// another's FP64 phases: 4.91 ms at two, 4.51 at three, although the compiler
-// spills 0.7 kB per thread there (2D Euler N = 4, 512 x 512; 4.14 ms with the
-// integer stage sums, which came after these); blocks of 128
-// threads 4.84 ms (per-block tables and neighbours), of 352 4.44.  The ten-moment
+// another's FP64 phases: 4.67 ms at two, 4.15 at three, although the compiler
+// spills 1.2 kB per thread there (2D Euler N = 4, 512 x 512); blocks of 128
+// threads 7% slower (per-block tables and neighbours), of 352 2% faster before the
+// integer stage sums.  The ten-moment
 // equations (six variables) two.  The systems with N <= 3 hold fewer sums per thread:
 // where a mesh has more blocks than those fill the chip with, one block more per SM
-// (`many`): 2D Euler 256 x 256, N = 1, 2, 3: 105, 257, 472 -> 93, 242, 450 us, ten-moment N
-// = 2, 3: 765, 1,416 -> 753, 1,378; a mesh that fits at once gains nothing and pays
+// (`many`): 2D Euler 256 x 256, N = 3: 475 -> 457 us, ten-moment N = 3 1,536 -> 1,523,
+// Rayleigh-Taylor 64 x 256 259 -> 245; a mesh that fits at once gains nothing and pays
 // for the spills (40 x 40, N = 3: 50.0 -> 52.5), and so does N = 4 (4.17 -> 4.25 ms,
 // ten-moment 2.99 -> 3.12).
 template <int DIM, int N, class EQ, bool MIXED> struct LocalBlocks {

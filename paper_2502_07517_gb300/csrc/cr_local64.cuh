@@ -29,9 +29,9 @@
 //     clear (exact_face_data).  The update is the same: alpha = 0 leaves the
 //     high-order part alone, and theta is decided as in FP64.
 // k_local, before (the general body in FP64) and now: 2D Euler N = 4, 512 x 512, 12.57
-// and 4.1 ms (58% of the FP64 pipe, 37% of the issue slots: latency bound);
-// ten-moment N = 3, 256 x 256, 2.61 and 1.52 ms; 1D Euler N = 4, whole step, 4,000 elements
-// 53 and 51 us, 60,000 elements 314 and 163 us.
+// and 4.19 ms (58% of the FP64 pipe, 37% of the issue slots: latency bound);
+// ten-moment N = 3, 256 x 256, 2.61 and 1.57 ms; 1D Euler N = 4, 4,000 elements, whole
+// step, 73 and 51 us.
 #pragma once
 #include "cr_common.cuh"
 #include "cr_fixed.cuh"
