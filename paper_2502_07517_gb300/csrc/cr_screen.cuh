@@ -2,7 +2,9 @@
 // instruction per 16 cycles and SM; a decision whose answer is clear by a margin
 // above the FP32 rounding needs none of it.  Every screen answers "clear" or
 // "not clear", and what is not clear is decided in FP64 as before, so the
-// results do not depend on the screens.  (Some of it also compiles for the host:
+// results do not depend on the screens.  Magnitudes outside FP32's range are never
+// clear: truncation makes those from 2^128 on infinite, and every comparison asks for
+// values, margins or norms well above 2^-126 (kTinyF and the bounds stated there).  (Some of it also compiles for the host:
 // tests/test_screens.py holds the screens against FP64.)
 #pragma once
 #include "cr_common.cuh"
